@@ -209,8 +209,8 @@ static void fill_bytes_per_iter(SystemImpl& S) {
   const int nu = S.op.nu_pre + S.op.nu_post;
   for (size_t l = 1; l < S.levels.size(); ++l) {
     const Level& L = S.levels[l];
-    b += nu * ((double)(L.P.sum_sq - L.P.real_sq) + 0.5 * (double)L.P.real_sq) * esz;  // smoother (n_j^2 per
-                                                                                      // patch, real ones half)
+    b += nu * ((double)(L.P.uniq_sq - L.P.uniq_real_sq) + 0.5 * (double)L.P.uniq_real_sq) * esz;  // smoother (n_j^2 per
+                                                                                      // stored block, real ones half)
     b += std::max(1, nu) * ((double)(L.A.nnz_alg - L.A.nnz_real) + 0.5 * (double)L.A.nnz_real) * esz;  // SpMVs
     if (L.kind == 2) b += (double)L.nK * (2.0 * L.nI * L.nS + L.nI * L.nI) * esz; // condense + backsub
   }
@@ -294,13 +294,18 @@ void setup_system(SystemImpl& S, const dpgmg_problem* pb, const dpgmg_opts* op, 
   if (ECSRDev* cg = cg_operator_of(S)) cg->nnz_real = packed_entries(*cg);
   for (size_t l = 1; l < S.levels.size() && S.plan; ++l) {
     PatchDev& P = S.levels[l].P;
-    P.real_sq = 0;
+    P.real_sq = P.uniq_real_sq = 0;
     if (!P.rflag || P.np == 0) continue;
     std::vector<uint8_t> fl((size_t)P.np);
     DPG_CUDA(cudaMemcpy(fl.data(), P.rflag, (size_t)P.np, cudaMemcpyDeviceToHost));
     const std::vector<int64_t>& pp = S.plan->lv[l].P.ptr;
+    const std::vector<int32_t>& own = S.plan->lv[l].prep;
     for (int64_t j = 0; j < P.np; ++j)
-      if (fl[j]) P.real_sq += (pp[j + 1] - pp[j]) * (pp[j + 1] - pp[j]);
+      if (fl[j]) {
+        const int64_t sq = (pp[j + 1] - pp[j]) * (pp[j + 1] - pp[j]);
+        P.real_sq += sq;
+        if (own[j] == j) P.uniq_real_sq += sq;
+      }
   }
   fill_bytes_per_iter(S);
 }
@@ -697,7 +702,6 @@ int dpgmg_spmv_group(dpgmg_handle h, dpgmg_system sys, int level, int set, int* 
     if (level < 1 || level >= (int)S.levels.size()) return DPGMG_ERR_ARG;
     g = &S.levels[level].A.gsel[slot];
   }
-  if (set) *g = set;
   if (group) *group = *g;
   return DPGMG_OK;
 }

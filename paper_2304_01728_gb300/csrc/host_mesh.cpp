@@ -8,6 +8,9 @@
 #include <stdexcept>
 #include <thread>
 #include <tuple>
+#include <array>
+#include <cstring>
+#include <unordered_map>
 
 namespace dpgmg {
 
@@ -624,6 +627,85 @@ std::vector<int64_t> patch_sizes(const MeshL& m, bool macro, int H, const int nc
           cnt[W[0][a] + (int64_t)(nco[0] + 1) * (W[1][b] + (int64_t)(nco[1] + 1) * W[2][q])] += nd;
   }
   return cnt;
+}
+
+// ------------------------------------------------------------ cell classes
+namespace {
+struct Key8 {
+  std::array<int32_t, 8> v;
+  bool operator==(const Key8& o) const { return v == o.v; }
+};
+struct Key8Hash {
+  size_t operator()(const Key8& k) const {
+    uint64_t h = 0x9E3779B97F4A7C15ull;
+    for (int32_t x : k.v) {
+      h ^= (uint64_t)(uint32_t)x + 0x9E3779B97F4A7C15ull + (h << 6) + (h >> 2);
+      h *= 0xBF58476D1CE4E5B9ull;
+    }
+    return (size_t)(h ^ (h >> 31));
+  }
+};
+}  // namespace
+
+std::vector<int32_t> element_classes(const MeshL& m, const std::vector<double>& wavespeed) {
+  std::vector<int32_t> id((size_t)m.nelem);
+  std::unordered_map<uint64_t, std::array<int32_t, 64>> cls;   // wavespeed bits -> id per impedance-face mask
+  int32_t next = 0;
+  for (int64_t e = 0; e < m.nelem; ++e) {
+    int ec[3], bm = 0;
+    m.elem_coord(e, ec);
+    for (int d = 0; d < 3; ++d) {
+      if (ec[d] == 0) bm |= 1 << (2 * d);
+      if (ec[d] == m.n[d] - 1) bm |= 1 << (2 * d + 1);
+    }
+    uint64_t key;
+    std::memcpy(&key, &wavespeed[e], sizeof key);
+    auto it = cls.find(key);
+    if (it == cls.end()) {
+      it = cls.emplace(key, std::array<int32_t, 64>()).first;
+      it->second.fill(-1);
+    }
+    int32_t& c = it->second[bm];
+    if (c < 0) c = next++;
+    id[e] = c;
+  }
+  return id;
+}
+
+std::vector<int32_t> macro_classes(const int nf[3], const std::vector<int32_t>& fine) {
+  const int nc[3] = {nf[0] / 2, nf[1] / 2, nf[2] / 2};
+  std::vector<int32_t> id((size_t)nc[0] * nc[1] * nc[2]);
+  std::unordered_map<Key8, int32_t, Key8Hash> cls;
+  size_t q = 0;
+  for (int k = 0; k < nc[2]; ++k)
+    for (int j = 0; j < nc[1]; ++j)
+      for (int i = 0; i < nc[0]; ++i) {
+        Key8 key;
+        for (int o = 0; o < 8; ++o)
+          key.v[o] = fine[(2 * i + (o & 1)) +
+                          (size_t)nf[0] * ((2 * j + ((o >> 1) & 1)) + (size_t)nf[1] * (2 * k + (o >> 2)))];
+        id[q++] = cls.emplace(key, (int32_t)cls.size()).first->second;
+      }
+  return id;
+}
+
+std::vector<int32_t> patch_classes(const int nco[3], const std::vector<int32_t>& cells) {
+  std::vector<int32_t> id((size_t)(nco[0] + 1) * (nco[1] + 1) * (nco[2] + 1));
+  std::unordered_map<Key8, int32_t, Key8Hash> cls;
+  size_t q = 0;
+  for (int k = 0; k <= nco[2]; ++k)
+    for (int j = 0; j <= nco[1]; ++j)
+      for (int i = 0; i <= nco[0]; ++i) {
+        Key8 key;
+        for (int o = 0; o < 8; ++o) {
+          const int c[3] = {i - 1 + (o & 1), j - 1 + ((o >> 1) & 1), k - 1 + (o >> 2)};
+          bool in = true;
+          for (int d = 0; d < 3; ++d) in = in && c[d] >= 0 && c[d] < nco[d];
+          key.v[o] = in ? cells[c[0] + (size_t)nco[0] * (c[1] + (size_t)nco[1] * c[2])] : -1;
+        }
+        id[q++] = cls.emplace(key, (int32_t)cls.size()).first->second;
+      }
+  return id;
 }
 
 // ----------------------------------------------------------- transitions

@@ -157,6 +157,15 @@ inline int64_t patch_ldr(int64_t n) { return (n + 3) & ~(int64_t)3; }
 // macro = true selects the h-level smoothing space (fine DOFs on the coarse skeleton).
 std::vector<int64_t> patch_sizes(const MeshL& m, bool macro, int H, const int nco[3], bool r2);
 
+// Classes of the cells of a level, by everything their matrices depend on:
+// finest elements by impedance faces and wavespeed (Sec. 2's forms on a uniform
+// mesh), coarse elements of an h-transition by the classes of their children;
+// patches by the classes of the cells around their vertex (-1: none there).
+// Ids count up from 0 in the order of first appearance.
+std::vector<int32_t> element_classes(const MeshL& m, const std::vector<double>& wavespeed);
+std::vector<int32_t> macro_classes(const int nf[3], const std::vector<int32_t>& fine);
+std::vector<int32_t> patch_classes(const int nco[3], const std::vector<int32_t>& cells);
+
 // Macro-grid structure of one h-transition (fine level m, coarse level mc).
 struct MacroHost {
   int nS = 0, nI = 0, nloc_f = 0, nloc_c = 0;

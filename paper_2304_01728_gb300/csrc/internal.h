@@ -87,6 +87,9 @@ struct ECSRDev {
   int gsel[3] = {1, 1, 1};
 };
 
+// outputs x members of a class-product work item
+enum { CLS_64x32 = 0, CLS_64x16, CLS_64x8, CLS_32x32, CLS_32x16 };
+
 struct PatchDev {
   int64_t np = 0, nslots = 0, nvals = 0, max_n = 0, sum_sq = 0;
   int64_t* ptr = nullptr;
@@ -108,6 +111,14 @@ struct PatchDev {
   uint8_t* rflag = nullptr;
   int64_t offU = 0;
   int64_t real_sq = 0;         // sum of n_j^2 over the real patches (host copy, after setup)
+  // Patch classes (classes.cuh): patches whose elements have the same classes
+  // share one stored block (val_ptr).  cls_items: (first member in cls_mem,
+  // members, first output, CLS_* shape); cls_mem: patches class by class.
+  // Null where too few patches share a block for the class product to pay.
+  int4* cls_items = nullptr;
+  int64_t ncls_items = 0;
+  int32_t* cls_mem = nullptr;
+  int64_t uniq_sq = 0, uniq_real_sq = 0;   // sum of n_j^2 over the distinct blocks, and over the real ones
   // Hermitian half storage (lower triangles packed by rows), used for the
   // complex64 operators of the mixed path
   bool half = false;
@@ -192,7 +203,11 @@ struct LevelPlan {
   int H = 2;                       // patch half-width in level-l elements
   Patches P;
   std::vector<int2> ch32, ch64;    // smoother work items of 32 / 64 rows, largest patch first
-  std::vector<int64_t> order;      // inversion order, largest patch first
+  std::vector<int64_t> order;      // inversion order, largest patch first; one patch per class
+  std::vector<int32_t> prep;       // per patch: the patch that owns its stored block (first of its class)
+  std::vector<int4> citems;        // class-product work items (PatchDev::cls_items), or empty
+  std::vector<int32_t> cmem;
+  int64_t uniq_sq = 0;
   int64_t max_n = 0, sum_sq = 0;
 };
 struct HostPlan {

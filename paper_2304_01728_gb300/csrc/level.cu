@@ -22,7 +22,7 @@
 #include "internal.h"
 #include "smoother.cuh"
 #include "block.cuh"
-#include "smoother.cuh"
+#include "classes.cuh"
 
 namespace dpgmg {
 
@@ -515,7 +515,7 @@ constexpr bool kHalfStorageSmoother = false;
 // blocks one CTA each; a cluster of 2 or 4 CTAs per patch spreads those over
 // several SMs.  Chosen so that the level has at least ~4 largest-patch shares
 // per SM; DPGMG_PATCH_TEAM = 1, 2 or 4 overrides the choice.
-static int patch_team(const Patches& P, int64_t max_n) {
+static int patch_team(const LevelPlan& lp, int64_t max_n) {
   if (const char* e = std::getenv("DPGMG_PATCH_TEAM")) {
     const int t = std::atoi(e);
     if (t == 1 || t == 2 || t == 4) return t;
@@ -525,8 +525,8 @@ static int patch_team(const Patches& P, int64_t max_n) {
   DPG_CUDA(cudaGetDevice(&dev));
   DPG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   double sum = 0.0;
-  for (size_t j = 0; j + 1 < P.ptr.size(); ++j) {
-    const double nj = (double)(P.ptr[j + 1] - P.ptr[j]);
+  for (int64_t j : lp.order) {
+    const double nj = (double)(lp.P.ptr[j + 1] - lp.P.ptr[j]);
     sum += nj * nj * nj;
   }
   const double shares = sum / ((double)max_n * max_n * max_n);
@@ -536,13 +536,13 @@ static int patch_team(const Patches& P, int64_t max_n) {
 }
 
 template <class C>
-static void invert_patches(Alloc& A, PatchDev& D, const LevelPlan& lp, C* vals, int64_t offU, int* dinfo,
-                           cudaStream_t st, uint8_t* rpack = nullptr) {
+static void invert_patches(Alloc& A, PatchDev& D, const LevelPlan& lp, const int64_t* dorder, C* vals, int64_t offU,
+                           int* dinfo, cudaStream_t st, uint8_t* rpack = nullptr) {
   const Patches& P = lp.P;
   const size_t sm = (size_t)(NB * NB + 2 * TL * NB) * sizeof(C) + 64;
   DPG_CUDA(cudaFuncSetAttribute(k_patch_invert<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   DPG_CUDA(cudaFuncSetAttribute(k_patch_invert<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  int team = patch_team(P, D.max_n);
+  int team = patch_team(lp, D.max_n);
   cudaLaunchAttribute cattr[1];
   cattr[0].id = cudaLaunchAttributeClusterDimension;
   cattr[0].val.clusterDim.x = (unsigned)team;
@@ -569,8 +569,9 @@ static void invert_patches(Alloc& A, PatchDev& D, const LevelPlan& lp, C* vals, 
   // launches of consecutive patches (largest first) whose scratch copies fit
   // `cap`; offs[q] = scratch offset of the q-th patch within its launch
   const std::vector<int64_t>& order = lp.order;
-  std::vector<int64_t> offs(D.np), starts;
-  for (int64_t q = 0, acc = 0; q < D.np; ++q) {
+  const int64_t nown = (int64_t)order.size();
+  std::vector<int64_t> offs(nown), starts;
+  for (int64_t q = 0, acc = 0; q < nown; ++q) {
     const int64_t j = order[q];
     const int64_t nj = P.ptr[j + 1] - P.ptr[j];
     if (q == 0 || acc + nj * nj > (int64_t)cap) {
@@ -580,9 +581,8 @@ static void invert_patches(Alloc& A, PatchDev& D, const LevelPlan& lp, C* vals, 
     offs[q] = acc;
     acc += nj * nj;
   }
-  starts.push_back(D.np);
+  starts.push_back(nown);
   int64_t* soff = upload(A, offs, st);
-  int64_t* dorder = upload(A, order, st);
   for (size_t c = 0; c + 1 < starts.size(); ++c) {
     const int64_t j0 = starts[c], q = starts[c + 1];
     if (team == 1) {
@@ -593,11 +593,10 @@ static void invert_patches(Alloc& A, PatchDev& D, const LevelPlan& lp, C* vals, 
       cfg.gridDim = dim3((unsigned)((q - j0) * team));
       DPG_CUDA(cudaLaunchKernelEx(&cfg, k_patch_invert<C, true>, (const int64_t*)D.ptr, (const int32_t*)D.dofs,
                                   (const int64_t*)D.val_ptr, vals, scratch, (const int64_t*)soff,
-                                  (const int64_t*)dorder, j0, offU, dinfo, rpack));
+                                  dorder, j0, offU, dinfo, rpack));
       count_launch();
     }
   }
-  A.release(dorder);
   A.release(soff);
   A.release(scratch);
 }
@@ -710,6 +709,12 @@ void patch_recompute_apply_blk(const Level& L, const float2* r, int64_t ldr, flo
   }
 }
 
+// rflag of the patches that share another patch's block
+__global__ void k_copy_flags(uint8_t* __restrict__ rflag, const int32_t* __restrict__ prep, int64_t np) {
+  const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (j < np && prep[j] != j) rflag[j] = rflag[prep[j]];
+}
+
 static void setup_patches(SystemImpl& S, Level& F, const LevelPlan& lp, int* dinfo, cudaStream_t st) {
   Alloc& A = S.mem;
   const Patches& P = lp.P;
@@ -729,7 +734,11 @@ static void setup_patches(SystemImpl& S, Level& F, const LevelPlan& lp, int* din
   D.chunks = upload(A, lp.ch32, st);
   D.nchunks64 = (int64_t)lp.ch64.size();
   D.chunks64 = upload(A, lp.ch64, st);
+  D.uniq_sq = lp.uniq_sq;
+  int64_t* order = upload(A, lp.order, st);   // the patches that own a block
+  const unsigned nown = (unsigned)lp.order.size();
   if (S.op.flags & DPGMG_FLAG_RECOMPUTE_PATCHES) {
+    A.release(order);
     setup_recompute(A, D, lp, F.mesh.offU, F.A, dinfo, st);
     return;
   }
@@ -737,28 +746,117 @@ static void setup_patches(SystemImpl& S, Level& F, const LevelPlan& lp, int* din
     // complex64 blocks, Cholesky, triangular inverse and L^-H L^-1 in FP32; the
     // smoother and its damping estimate use exactly these inverses
     D.inv32 = A.arr<float2>((size_t)std::max<int64_t>(D.nvals, 1));
-    k_patch_gather<float2><<<(unsigned)D.np, 256, 0, st>>>(F.A, D.ptr, D.dofs, D.val_ptr, D.inv32, 0);
+    k_patch_gather<float2><<<nown, 256, 0, st>>>(F.A, D.ptr, D.dofs, D.val_ptr, D.inv32, 0, order);
     DPG_CHECK_LAUNCH();
     // real-path patches keep real inverses (half the smoother's bytes for them)
     if (pack_storage(S)) {
       D.rflag = A.arr<uint8_t>((size_t)std::max<int64_t>(D.np, 1));
       DPG_CUDA(cudaMemsetAsync(D.rflag, 0, (size_t)std::max<int64_t>(D.np, 1), st));
     }
-    invert_patches<float2>(A, D, lp, D.inv32, F.mesh.offU, dinfo, st, D.rflag);
+    invert_patches<float2>(A, D, lp, order, D.inv32, F.mesh.offU, dinfo, st, D.rflag);
+    if (D.rflag && nown < D.np) {
+      int32_t* prep = upload(A, lp.prep, st);
+      k_copy_flags<<<(unsigned)((D.np + 255) / 256), 256, 0, st>>>(D.rflag, prep, D.np);
+      DPG_CHECK_LAUNCH();
+      A.release(prep);
+    }
+    if (!lp.citems.empty()) {
+      D.cls_items = upload(A, lp.citems, st);
+      D.ncls_items = (int64_t)lp.citems.size();
+      D.cls_mem = upload(A, lp.cmem, st);
+      D.variant = SMOOTH_CLASS;   // until setup has timed the variants
+    }
+    A.release(order);
     return;
   }
   D.inv64 = A.arr<double2>((size_t)D.nvals);
-  k_patch_gather<double2><<<(unsigned)D.np, 256, 0, st>>>(F.A, D.ptr, D.dofs, D.val_ptr, D.inv64, 0);
+  k_patch_gather<double2><<<nown, 256, 0, st>>>(F.A, D.ptr, D.dofs, D.val_ptr, D.inv64, 0, order);
   DPG_CHECK_LAUNCH();
   // FP64 inverses (FP64 path, or the mixed path under DPGMG_FLAG_PATCH_FP64,
   // which rounds them to complex64 after theta is estimated)
-  invert_patches<double2>(A, D, lp, D.inv64, F.mesh.offU, dinfo, st);
+  invert_patches<double2>(A, D, lp, order, D.inv64, F.mesh.offU, dinfo, st);
+  A.release(order);
 }
 
 // DPGMG_COARSEST_SMOOTH on a hierarchy with more than one level: level 0 is
 // smoothed (its own operator and vertex patches) instead of solved.
 static bool smooth_coarsest(const SystemImpl& S) {
   return S.op.coarsest == DPGMG_COARSEST_SMOOTH && S.levels.size() > 1;
+}
+
+// Patches of one class share a stored block, except in recompute mode (its
+// windows hold every patch's own block).
+static bool share_patches(const SystemImpl& S) { return !(S.op.flags & DPGMG_FLAG_RECOMPUTE_PATCHES); }
+
+// The class product pays when the blocks are shared by at least
+// CLS_MIN_SHARE patches on average (by entries); below that the streaming
+// product, which keeps more of a block's bytes in flight, reads them.
+constexpr double CLS_MIN_SHARE = 2.0;
+
+// Work items of a class product: mem lists the members class by class, items
+// are (first member, members, first output, CLS_* shape), the longest first
+// (sum length times tile size), so that short ones end the launch.
+template <class F>
+static void class_items(const std::vector<std::vector<int32_t>>& members, F&& size_of, std::vector<int32_t>& mem,
+                        std::vector<int4>& items) {
+  for (const auto& m : members) {
+    const int64_t n = size_of(m[0]), m0 = (int64_t)mem.size();
+    const int cnt = (int)m.size();
+    mem.insert(mem.end(), m.begin(), m.end());
+    for (int64_t a = 0; a < n; a += 64) {
+      const bool half = n - a <= 32;
+      for (int q = 0; q < cnt;) {
+        const int left = cnt - q;
+        const int shape = half ? (left > 16 ? CLS_32x32 : CLS_32x16)
+                               : (left > 16 ? CLS_64x32 : (left > 8 ? CLS_64x16 : CLS_64x8));
+        const int w = shape == CLS_64x8 ? 8 : (shape == CLS_64x16 || shape == CLS_32x16 ? 16 : 32);
+        items.push_back(make_int4((int)m0 + q, std::min(w, left), (int)a, shape));
+        q += w;
+      }
+    }
+  }
+  auto cost = [&](const int4& t) {
+    const int64_t f[5] = {64 * 32, 64 * 16, 64 * 8, 32 * 32, 32 * 16};
+    return size_of(mem[t.x]) * f[t.w];
+  };
+  std::stable_sort(items.begin(), items.end(), [&](const int4& u, const int4& v) { return cost(u) > cost(v); });
+}
+
+// Stored blocks, inversion order and class-product work items of a level's
+// patches.  cells: classes of the level's (macro) elements, or empty (every
+// patch keeps its own block).
+static void plan_patch_classes(LevelPlan& lp, const std::vector<int32_t>& cells, const int nco[3]) {
+  Patches& P = lp.P;
+  const int64_t np = (int64_t)P.ptr.size() - 1;
+  auto size_of = [&](int64_t j) { return P.ptr[j + 1] - P.ptr[j]; };
+  lp.prep.resize(np);
+  std::vector<int32_t> cls;
+  if (cells.empty()) {
+    for (int64_t j = 0; j < np; ++j) lp.prep[j] = (int32_t)j;
+    lp.uniq_sq = lp.sum_sq;
+    return;
+  }
+  cls = patch_classes(nco, cells);
+  std::vector<std::vector<int32_t>> members;
+  for (int64_t j = 0; j < np; ++j) {
+    if (cls[j] == (int32_t)members.size()) members.emplace_back();
+    members[cls[j]].push_back((int32_t)j);
+  }
+  // blocks of the classes' first patches, in patch order; the others point to theirs
+  int64_t off = 0;
+  for (int64_t j = 0; j < np; ++j) {
+    const int32_t f = members[cls[j]][0];
+    if (size_of(f) != size_of(j)) throw Err{DPGMG_ERR_ARG, "patch classes: members of different sizes"};
+    lp.prep[j] = f;
+    P.val_ptr[j] = f == j ? off : P.val_ptr[f];
+    if (f == j) {
+      off += size_of(j) * patch_ld(size_of(j));
+      lp.uniq_sq += size_of(j) * size_of(j);
+    }
+  }
+  P.val_ptr[np] = off;
+  if ((double)lp.sum_sq < CLS_MIN_SHARE * (double)lp.uniq_sq) return;
+  class_items(members, size_of, lp.cmem, lp.citems);
 }
 
 // Host index plan of a hierarchy (every level's integer structures); runs on
@@ -786,7 +884,14 @@ std::shared_ptr<HostPlan> plan_host(const SystemImpl& S) {
     th.emplace_back(guarded(L + 1, [&]() { HP->acg = prep_ecsr(S.levels[L].mesh, element_groups(S.levels[L].mesh)); }));
   }
   const int lmin = smooth_coarsest(S) ? 0 : 1;
-  for (int l = L; l >= lmin; --l) th.emplace_back(guarded(l, [&S, &HP, l]() {
+  // cell classes of every level (the elements of a p-coarsened level keep their classes)
+  std::vector<std::vector<int32_t>> cells(L + 1);
+  if (share_patches(S)) {
+    cells[L] = element_classes(S.levels[L].mesh, S.wavespeed);
+    for (int l = L; l >= 1; --l)
+      cells[l - 1] = S.levels[l].kind == 1 ? cells[l] : macro_classes(S.levels[l].mesh.n, cells[l]);
+  }
+  for (int l = L; l >= lmin; --l) th.emplace_back(guarded(l, [&S, &HP, &cells, l]() {
     const Level& F = S.levels[l];
     const Level& C = S.levels[l > 0 ? l - 1 : 0];   // level 0: the vertex patches of its own mesh
     LevelPlan& lp = HP->lv[l];
@@ -822,8 +927,9 @@ std::shared_ptr<HostPlan> plan_host(const SystemImpl& S) {
         for (int64_t a0 = 0; a0 < size_of(j); a0 += width) ch.push_back(make_int2((int)j, (int)a0));
       std::stable_sort(ch.begin(), ch.end(), [&](const int2& u, const int2& v) { return size_of(u.x) > size_of(v.x); });
     }
-    lp.order.resize(np);
-    for (int64_t j = 0; j < np; ++j) lp.order[j] = j;
+    plan_patch_classes(lp, cells[l > 0 ? l - 1 : 0], C.mesh.n);
+    for (int64_t j = 0; j < np; ++j)
+      if (lp.prep[j] == j) lp.order.push_back(j);
     std::stable_sort(lp.order.begin(), lp.order.end(), [&](int64_t u, int64_t v) { return size_of(u) > size_of(v); });
   }));
   for (auto& t : th) t.join();

@@ -21,6 +21,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "smoother.cuh"
+#include "classes.cuh"
 
 namespace dpgmg {
 
@@ -51,6 +52,9 @@ static void na_smooth(const Level& L, const C* inv_full, const C* inv_half, cons
     DPG_CUDA(cudaFuncSetAttribute(k_patch_apply_h<C, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
     const size_t sm = (size_t)9 * P.max_n * sizeof(C) + 16;
     k_patch_apply_h<C, double2><<<(unsigned)P.np, 256, sm, st>>>(P.ptr, P.dofs, P.hptr, inv_half, r, scratch);
+    DPG_CHECK_LAUNCH();
+  } else if (std::is_same<C, float2>::value && P.variant == SMOOTH_CLASS) {
+    launch_class_apply<double2>(P, r, 0, reinterpret_cast<float2*>(scratch), 0, 1, st);
   } else {
     const size_t sm = (size_t)P.max_n * sizeof(C) + 16;
     int64_t nch = 0;
@@ -58,8 +62,8 @@ static void na_smooth(const Level& L, const C* inv_full, const C* inv_half, cons
     const uint8_t* rflag = std::is_same<C, float2>::value ? P.rflag : nullptr;   // packed complex64 inverses only
     k_patch_apply<C, double2><<<(unsigned)nch, 256, sm, st>>>(P.ptr, P.dofs, P.val_ptr, chunks, inv_full, r, scratch,
                                                               rflag, P.offU);
+    DPG_CHECK_LAUNCH();
   }
-  DPG_CHECK_LAUNCH();
   k_slot_sum<C, double2><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(P.slot_ptr, P.slots, scratch, y, n, L.theta, 0);
   DPG_CHECK_LAUNCH();
 }

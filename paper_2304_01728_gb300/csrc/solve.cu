@@ -24,6 +24,7 @@
 #include "internal.h"
 #include "block.cuh"
 #include "smoother.cuh"
+#include "classes.cuh"
 
 namespace dpgmg {
 
@@ -1317,7 +1318,8 @@ static void configure_smoother_kernels() {
 template <class C> static void patch_product(const PatchDev& P, const C* inv, const C* r, C* pbuf, cudaStream_t st);
 template <>
 void patch_product<float2>(const PatchDev& P, const float2* inv, const float2* r, float2* pbuf, cudaStream_t st) {
-  launch_patch_apply_c64<float2>(P, P.variant, inv, r, pbuf, st);
+  if (P.variant == SMOOTH_CLASS) launch_class_apply<float2>(P, r, 0, pbuf, 0, 1, st);
+  else launch_patch_apply_c64<float2>(P, P.variant, inv, r, pbuf, st);
 }
 template <>
 void patch_product<double2>(const PatchDev& P, const double2* inv, const double2* r, double2* pbuf, cudaStream_t st) {
@@ -1931,6 +1933,13 @@ static void smooth_blk(const Level& L, const C* r, C* y, double theta, int accum
       DPG_CHECK_LAUNCH();
       return;
     }
+    if (P.variant == SMOOTH_CLASS) {   // shared blocks: the K vectors as a second grid dimension, each block read from L2
+      launch_class_apply<float2>(P, r, n, pbuf, ldp, K, st);
+      k_slot_sum_blk<C><<<dim3(nblk(n), (unsigned)K), 256, 0, st>>>(P.slot_ptr, P.slots, pbuf, ldp, y, n, n, theta,
+                                                                     accumulate);
+      DPG_CHECK_LAUNCH();
+      return;
+    }
   }
   if (!inv || cap < 1) {
     for (int k = 0; k < K; ++k) smooth<C>(L, r + k * n, y + k * n, theta, accumulate, pbuf + k * ldp, st);
@@ -2339,13 +2348,20 @@ void prepare_solve(SystemImpl& S, cudaStream_t st) {
       F.A.gsel[0] = pick_group(key, ev, st, [&](int G) { spmv_g<float2>(F.A, F.A.v32, x, nullptr, y, 0, G, st); },
                                F.A.rent != nullptr);
       if (F.P.inv32 && F.P.np) {
-        // smoother product: 1 or 2 columns per lane (32- or 64-column work
+        // smoother product: shared blocks (classes.cuh), or 1 or 2 columns per lane (32- or 64-column work
         // items), the latter at 8 or 6 CTAs per SM; the block smoother takes
         // the same columns per lane
-        const TuneKey skey{F.P.rflag ? 4 : 3, F.mesh.p, F.kind, log2i(F.P.np)};   // packed real blocks or not
-        auto run = [&](int c) { launch_patch_apply_c64<float2>(F.P, c, F.P.inv32, x, W.w32[l].pbuf, st); };
-        F.P.variant = F.P.rflag ? pick_variant(skey, ev, st, {SMOOTH_PER2_WIDE, 2, 1}, run)
-                                : pick_variant(skey, ev, st, {2, SMOOTH_PER2_WIDE, 1}, run);
+        // or not; shared blocks: the number of class work items too (small levels with few members
+        // per class keep the streaming product, which has more CTAs and shorter chains)
+        const TuneKey skey{(F.P.rflag ? 4 : 3) + (F.P.cls_items ? 16 * (1 + log2i(F.P.ncls_items)) : 0), F.mesh.p,
+                           F.kind, log2i(F.P.np)};
+        auto run = [&](int c) {
+          if (c == SMOOTH_CLASS) launch_class_apply<float2>(F.P, x, 0, W.w32[l].pbuf, 0, 1, st);
+          else launch_patch_apply_c64<float2>(F.P, c, F.P.inv32, x, W.w32[l].pbuf, st);
+        };
+        F.P.variant = F.P.cls_items ? pick_variant(skey, ev, st, {SMOOTH_CLASS, SMOOTH_PER2_WIDE, 2, 1}, run)
+                      : F.P.rflag   ? pick_variant(skey, ev, st, {SMOOTH_PER2_WIDE, 2, 1}, run)
+                                    : pick_variant(skey, ev, st, {2, SMOOTH_PER2_WIDE, 1}, run);
         F.P.cols = F.P.variant == 1 ? 1 : 2;
       }
     } else {
@@ -2378,8 +2394,8 @@ int pcg_solve(SystemImpl& S, cudaStream_t st, double2* xout, dpgmg_stats* stats,
   {
     const Level& Ff = S.levels.back();
     const int64_t esz = S.op.precision == DPGMG_PREC_MIXED ? 8 : 16;
-    if (S.prof_which == DPGMG_PROF_SMOOTH_FINE)   // stored entries read once: real packed blocks at half size
-      S.prof_bytes = (Ff.P.sum_sq - Ff.P.real_sq) * esz + Ff.P.real_sq * (esz / 2);
+    if (S.prof_which == DPGMG_PROF_SMOOTH_FINE)   // stored blocks read once: real packed ones at half size
+      S.prof_bytes = (Ff.P.uniq_sq - Ff.P.uniq_real_sq) * esz + Ff.P.uniq_real_sq * (esz / 2);
     else if (S.prof_which == DPGMG_PROF_SPMV_FINE)   // packed real entities at half size
       S.prof_bytes = (Ff.A.nnz_alg - Ff.A.nnz_real) * esz + Ff.A.nnz_real * (esz / 2);
     else if (S.prof_which == DPGMG_PROF_SPMV_CG)     // hi + lo complex64, or hi + lo reals
