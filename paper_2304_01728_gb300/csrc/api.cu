@@ -694,13 +694,20 @@ int dpgmg_spmv_group(dpgmg_handle h, dpgmg_system sys, int level, int set, int* 
   SystemImpl& S = sys->s;
   const int slot = S.op.precision == DPGMG_PREC_MIXED ? 0 : 1;
   int* g = nullptr;
+  bool* cells = nullptr;   // an override also selects the assembled rows
   if (level == -1) {
     ECSRDev* A = cg_operator_of(S);
     if (!A) return DPGMG_ERR_ARG;
     g = &A->gsel[2];
+    cells = &A->cell.df_on;
   } else {
     if (level < 1 || level >= (int)S.levels.size()) return DPGMG_ERR_ARG;
     g = &S.levels[level].A.gsel[slot];
+    cells = &S.levels[level].A.cell.on;
+  }
+  if (set) {
+    *g = set;
+    *cells = false;
   }
   if (group) *group = *g;
   return DPGMG_OK;

@@ -57,6 +57,44 @@ template <class T, class AL> T* upload(Alloc& A, const std::vector<T, AL>& h, cu
 }
 
 // ----------------------------------------------------------- device structs
+// An operator as a sum over its cells, y = sum_K R_K^T A_K R_K x, with one
+// stored matrix per cell class (classes.cuh): the elements of a p level, the
+// macro elements of an h level.  Kept beside the assembled rows when the cells
+// are many per class.
+struct CellOpDev {
+  bool on = false;             // applied in place of the assembled rows (complex64 V-cycle operator)
+  bool df_on = false;          // the same for the double-float CG operator
+  int n = 0;                   // local DOFs of a cell
+  int64_t ncell = 0, ndof = 0, ncls = 0;
+  int32_t* idx = nullptr;      // [ncell][n] DOF, or -1
+  int32_t* cls = nullptr;      // [ncell] class
+  float2* W = nullptr;         // [ncls][n x ld] conj(A_K)^T, complex64, or reals (rflag)
+  float2* Wlo = nullptr;       // low parts (A_K ~ W + Wlo), CG operator only
+  uint8_t* rflag = nullptr;    // [ncls] real once the unit phases are taken out, rows of patch_ldr(n) reals
+  int4* items = nullptr;       // work items as PatchDev::cls_items, over cells
+  int64_t nitems = 0;
+  int4* items16 = nullptr;     // items of at most 16 members (double-float product)
+  int64_t nitems16 = 0;
+  int32_t* mem = nullptr;      // cells class by class
+  // the (cell, local) slots of every DOF: fixed-pitch rows (8 per vertex, 4 per edge and 2 per face DOF, -1 =
+  // none) on a p level, CSR on an h level
+  int32_t* tab = nullptr;
+  int64_t* sptr = nullptr;
+  int32_t* slots = nullptr;
+  int64_t offE = 0, offF = 0, offU = 0;
+  float2* ybuf = nullptr;      // [ncell][n] cell products
+  float4* ydf = nullptr;       // the same in double-float (CG operator only)
+  int64_t stride() const { return n * patch_ld(n); }   // entries per class matrix
+};
+
+// first place of DOF g's row in CellOpDev::tab (also the table's size, for g = ndof)
+#if defined(__CUDACC__)
+__host__ __device__
+#endif
+inline int64_t cell_row(int64_t g, int64_t offE, int64_t offF) {
+  return g < offE ? 8 * g : (g < offF ? 8 * offE + 4 * (g - offE) : 8 * offE + 4 * (offF - offE) + 2 * (g - offF));
+}
+
 struct ECSRDev {
   int64_t nrows = 0, nent = 0, nnz = 0, max_nnz_row = 0;
   int64_t nnz_alg = 0;     // operator entries (algorithmic bytes count these)
@@ -82,6 +120,7 @@ struct ECSRDev {
   // complex64, complex128 and double-float products (1 = one warp per row).
   int2* tasks[4] = {nullptr, nullptr, nullptr, nullptr};
   int64_t ntasks[4] = {0, 0, 0, 0};
+  CellOpDev cell;          // the same operator by cells (mixed path, shared cell matrices), when cell.W is set
   int32_t* null_rows = nullptr;
   int64_t n_null = 0;
   int gsel[3] = {1, 1, 1};
@@ -208,6 +247,10 @@ struct LevelPlan {
   std::vector<int4> citems;        // class-product work items (PatchDev::cls_items), or empty
   std::vector<int32_t> cmem;
   int64_t uniq_sq = 0;
+  std::vector<int32_t> ocls;       // classes of the operator's cells, or empty (no shared cell matrices)
+  std::vector<int64_t> orep;       // first cell of each class
+  std::vector<int4> oitems, oitems16;
+  std::vector<int32_t> omem;
   int64_t max_n = 0, sum_sq = 0;
 };
 struct HostPlan {

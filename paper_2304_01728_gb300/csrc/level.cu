@@ -293,9 +293,133 @@ __global__ void __launch_bounds__(CTA_THREADS) k_macro(MacroArgs<C> a) {
   }
 }
 
+// ------------------------------------------------------- operator by cells
+// Class matrices: one CTA per class c, from the matrix of its first cell
+// (E + (rep[c] - e0) n^2; classes whose first cell is outside e0 .. e0 + ne - 1
+// are skipped): W[k][a] = conj(A[a][k]) (classes.cuh), as reals when every
+// entry is real once the unit phases are taken out (pack; exact test, as
+// k_pack_ops), with low parts when Wlo is given (TE = double2).
+template <class TE>
+__global__ void k_cell_class(const TE* __restrict__ E, int64_t e0, int64_t ne, const int64_t* __restrict__ rep,
+                             const int32_t* __restrict__ idx, int n, int64_t stride, int64_t offU, bool pack,
+                             float2* __restrict__ W, float2* __restrict__ Wlo, uint8_t* __restrict__ rflag) {
+  const int64_t c = blockIdx.x, e = rep[c];
+  if (e < e0 || e >= e0 + ne) return;
+  const TE* A = E + (e - e0) * (size_t)n * n;
+  const int32_t* g = idx + e * n;
+  auto phat = [&](int q) { return g[q] >= 0 && g[q] < offU ? 1 : 0; };
+  bool cplx = !pack;
+  if (pack)
+    for (int q = threadIdx.x; q < n * n; q += blockDim.x)
+      if (mul_i(A[q], phat(q % n) - phat(q / n)).y != 0) cplx = true;
+  cplx = __syncthreads_or(cplx) != 0;
+  float2* Wc = W + c * stride;
+  float2* Lc = Wlo ? Wlo + c * stride : nullptr;
+  const int ld = (int)(cplx ? patch_ld(n) : patch_ldr(n));
+  for (int q = threadIdx.x; q < n * ld; q += blockDim.x) {
+    const int k = q / ld, a = q % ld;
+    double2 v = make_double2(0.0, 0.0);
+    if (a < n) {
+      const TE t = A[(size_t)a * n + k];
+      v = cplx ? make_double2(t.x, -(double)t.y) : make_double2(mul_i(t, phat(k) - phat(a)).x, 0.0);
+    }
+    const float2 h = make_float2((float)v.x, (float)v.y);
+    const float2 l = make_float2((float)(v.x - (double)h.x), (float)(v.y - (double)h.y));
+    if (cplx) {
+      Wc[q] = h;
+      if (Lc) Lc[q] = l;
+    } else {
+      reinterpret_cast<float*>(Wc)[q] = h.x;
+      if (Lc) reinterpret_cast<float*>(Lc)[q] = l.x;
+    }
+  }
+  if (threadIdx.x == 0) rflag[c] = cplx ? 0 : 1;
+}
+
+// 32-bit DOF list of the cells and, on a p level (tab), the slot table: local
+// function i of element e sits at a fixed place (code[i], its position among
+// the elements around the entity) of its DOF's row.
+__global__ void k_cell_index(const int64_t* __restrict__ dofs, const uint8_t* __restrict__ code, int64_t total, int n,
+                             int64_t offE, int64_t offF, int32_t* __restrict__ idx, int32_t* __restrict__ tab) {
+  const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (q >= total) return;
+  const int64_t g = dofs[q];
+  idx[q] = (int32_t)g;
+  if (tab && g >= 0) tab[cell_row(g, offE, offF) + code[q % n]] = (int32_t)q;
+}
+
+// Index data and storage of a level's operator by cells; the matrices follow
+// (k_cell_class).
+static void cell_op_begin(SystemImpl& S, Level& F, const LevelPlan& lp, cudaStream_t st) {
+  if (lp.ocls.empty()) return;   // mixed path only (plan_host)
+  Alloc& A = S.mem;
+  CellOpDev& D = F.A.cell;
+  const bool macro = F.kind == 2;
+  D.n = macro ? F.nS : F.nloc;
+  D.ncell = (int64_t)lp.ocls.size();
+  D.ncls = (int64_t)lp.orep.size();
+  D.ndof = F.mesh.ndof;
+  D.offE = F.mesh.offE;
+  D.offF = F.mesh.offF;
+  D.offU = F.mesh.offU;
+  D.idx = A.arr<int32_t>((size_t)D.ncell * D.n);
+  D.cls = upload(A, lp.ocls, st);
+  D.items = upload(A, lp.oitems, st);
+  D.nitems = (int64_t)lp.oitems.size();
+  D.items16 = upload(A, lp.oitems16, st);
+  D.nitems16 = (int64_t)lp.oitems16.size();
+  D.mem = upload(A, lp.omem, st);
+  const bool cg = &F == &S.levels.back() && F.kind == 1 && !(S.op.flags & DPGMG_FLAG_CG_C128);
+  D.W = A.arr<float2>((size_t)D.ncls * D.stride());
+  if (cg) {
+    D.Wlo = A.arr<float2>((size_t)D.ncls * D.stride());
+    D.ydf = A.arr<float4>((size_t)D.ncell * D.n);
+    D.df_on = true;
+  }
+  D.rflag = A.arr<uint8_t>((size_t)D.ncls);
+  D.ybuf = A.arr<float2>((size_t)D.ncell * D.n);
+  uint8_t* code = nullptr;
+  if (macro) {
+    D.sptr = F.sslot_ptr;
+    D.slots = F.sslots;
+  } else {
+    std::vector<uint8_t> h(F.mesh.loc.size());
+    for (size_t i = 0; i < h.size(); ++i) {
+      const LocFn& f = F.mesh.loc[i];
+      int c = 0, bit = 0;
+      if (f.type == 1) c = f.s;
+      else
+        for (int d = 0; d < 3; ++d)
+          if (f.idx[d] < 2) c |= f.idx[d] << bit++;
+      h[i] = (uint8_t)c;
+    }
+    code = upload(A, h, st);
+    const size_t rows = (size_t)cell_row(D.ndof, D.offE, D.offF);
+    D.tab = A.arr<int32_t>(rows);
+    DPG_CUDA(cudaMemsetAsync(D.tab, 0xff, rows * sizeof(int32_t), st));
+  }
+  const int64_t total = D.ncell * D.n;
+  k_cell_index<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(macro ? F.S_glob : F.dofs, code, total, D.n, D.offE,
+                                                              D.offF, D.idx, D.tab);
+  DPG_CHECK_LAUNCH();
+  if (code) A.release(code);
+  D.on = true;
+}
+
+// Matrices of the classes whose first cell is among cells e0 .. e0 + ne - 1 (E: their matrices).
+template <class TE>
+static void cell_op_matrices(SystemImpl& S, Level& F, const int64_t* rep, const TE* E, int64_t e0, int64_t ne,
+                             cudaStream_t st) {
+  CellOpDev& D = F.A.cell;
+  if (!D.W) return;
+  k_cell_class<TE><<<(unsigned)D.ncls, 256, 0, st>>>(E, e0, ne, rep, D.idx, D.n, D.stride(), D.offU, pack_storage(S),
+                                                    D.W, D.Wlo, D.rflag);
+  DPG_CHECK_LAUNCH();
+}
+
 template <class C>
 static void macro_condense(SystemImpl& S, Level& F, Level& C_, const MacroHost& M, const int32_t* cmap, int* dinfo,
-                           C* Y, C* Ai, cudaStream_t st) {
+                           C* Y, C* Ai, const int64_t* crep, cudaStream_t st) {
   Alloc& A = S.mem;
   std::vector<C> ik(M.IK.size());
   for (size_t i = 0; i < ik.size(); ++i) {
@@ -324,6 +448,7 @@ static void macro_condense(SystemImpl& S, Level& F, Level& C_, const MacroHost& 
     k_macro<C><<<nb, CTA_THREADS, sm, st>>>(a);
     DPG_CHECK_LAUNCH();
     ecsr_add_t<C>(F.A, MK, F.S_glob + K0 * F.nS, nb, F.nS, K0, C_.mesh.n, st);
+    cell_op_matrices<C>(S, F, crep, MK, K0, nb, st);
   }
   A.release(AK);   // stream-ordered frees: after the launches above
   A.release(T1);
@@ -796,9 +921,10 @@ constexpr double CLS_MIN_SHARE = 2.0;
 // Work items of a class product: mem lists the members class by class, items
 // are (first member, members, first output, CLS_* shape), the longest first
 // (sum length times tile size), so that short ones end the launch.
+// most: members per item at most.
 template <class F>
 static void class_items(const std::vector<std::vector<int32_t>>& members, F&& size_of, std::vector<int32_t>& mem,
-                        std::vector<int4>& items) {
+                        std::vector<int4>& items, int most = 32) {
   for (const auto& m : members) {
     const int64_t n = size_of(m[0]), m0 = (int64_t)mem.size();
     const int cnt = (int)m.size();
@@ -806,7 +932,7 @@ static void class_items(const std::vector<std::vector<int32_t>>& members, F&& si
     for (int64_t a = 0; a < n; a += 64) {
       const bool half = n - a <= 32;
       for (int q = 0; q < cnt;) {
-        const int left = cnt - q;
+        const int left = std::min(cnt - q, most);
         const int shape = half ? (left > 16 ? CLS_32x32 : CLS_32x16)
                                : (left > 16 ? CLS_64x32 : (left > 8 ? CLS_64x16 : CLS_64x8));
         const int w = shape == CLS_64x8 ? 8 : (shape == CLS_64x16 || shape == CLS_32x16 ? 16 : 32);
@@ -857,6 +983,27 @@ static void plan_patch_classes(LevelPlan& lp, const std::vector<int32_t>& cells,
   P.val_ptr[np] = off;
   if ((double)lp.sum_sq < CLS_MIN_SHARE * (double)lp.uniq_sq) return;
   class_items(members, size_of, lp.cmem, lp.citems);
+}
+
+// The same for the operator by cells: one matrix per cell class, n local DOFs.
+// Kept when a matrix serves at least CLS_MIN_SHARE cells on average.
+static void plan_cell_classes(LevelPlan& lp, const std::vector<int32_t>& cells, int n) {
+  if (cells.empty()) return;
+  std::vector<std::vector<int32_t>> members;
+  for (size_t e = 0; e < cells.size(); ++e) {
+    if (cells[e] == (int32_t)members.size()) {
+      if ((double)members.size() * CLS_MIN_SHARE > (double)cells.size()) return;
+      members.emplace_back();
+    }
+    members[cells[e]].push_back((int32_t)e);
+  }
+  if ((double)members.size() * CLS_MIN_SHARE > (double)cells.size()) return;
+  lp.ocls = cells;
+  for (const auto& m : members) lp.orep.push_back(m[0]);
+  auto size_of = [&](int64_t) { return (int64_t)n; };
+  class_items(members, size_of, lp.omem, lp.oitems);
+  lp.omem.clear();
+  class_items(members, size_of, lp.omem, lp.oitems16, 16);
 }
 
 // Host index plan of a hierarchy (every level's integer structures); runs on
@@ -928,6 +1075,8 @@ std::shared_ptr<HostPlan> plan_host(const SystemImpl& S) {
       std::stable_sort(ch.begin(), ch.end(), [&](const int2& u, const int2& v) { return size_of(u.x) > size_of(v.x); });
     }
     plan_patch_classes(lp, cells[l > 0 ? l - 1 : 0], C.mesh.n);
+    if (S.op.precision == DPGMG_PREC_MIXED)
+      plan_cell_classes(lp, F.kind == 2 ? cells[l - 1] : cells[l], F.kind == 2 ? lp.M.nS : (int)F.mesh.loc.size());
     for (int64_t j = 0; j < np; ++j)
       if (lp.prep[j] == j) lp.order.push_back(j);
     std::stable_sort(lp.order.begin(), lp.order.end(), [&](int64_t u, int64_t v) { return size_of(u) > size_of(v); });
@@ -1028,6 +1177,12 @@ void build_hierarchy(SystemImpl& S, cudaStream_t st) {
       DPG_CHECK_LAUNCH();
       assemble_ecsr(A, lp.E, F.A, st);
       ecsr_add_elements(F.A, F.E, F.dofs, F.mesh.nelem, F.nloc, 0, F.mesh.n, st);
+      cell_op_begin(S, F, lp, st);
+      if (F.A.cell.W) {
+        int64_t* crep = upload(A, lp.orep, st);
+        cell_op_matrices<double2>(S, F, crep, F.E, 0, F.mesh.nelem, st);
+        A.release(crep);
+      }
     } else {
       const MacroHost& M = lp.M;
       F.nS = M.nS;
@@ -1046,15 +1201,18 @@ void build_hierarchy(SystemImpl& S, cudaStream_t st) {
       F.smask = upload(A, M.smask, st);
       int32_t* cmap = upload(A, M.child_map, st);
       assemble_ecsr(A, lp.E, F.A, st);
+      cell_op_begin(S, F, lp, st);
+      int64_t* crep = upload(A, lp.orep, st);
       if (macro_fp32(S)) {
         F.Y32 = A.arr<float2>((size_t)F.nK * F.nI * F.nS);
         F.Ai32 = A.arr<float2>((size_t)F.nK * F.nI * F.nI);
-        macro_condense<float2>(S, F, C, M, cmap, dinfo, F.Y32, F.Ai32, st);
+        macro_condense<float2>(S, F, C, M, cmap, dinfo, F.Y32, F.Ai32, crep, st);
       } else {
         F.Y64 = A.arr<double2>((size_t)F.nK * F.nI * F.nS);
         F.Ai64 = A.arr<double2>((size_t)F.nK * F.nI * F.nI);
-        macro_condense<double2>(S, F, C, M, cmap, dinfo, F.Y64, F.Ai64, st);
+        macro_condense<double2>(S, F, C, M, cmap, dinfo, F.Y64, F.Ai64, crep, st);
       }
+      A.release(crep);
     }
     if (S.op.flags & DPGMG_FLAG_STORE_COARSE) {
       // "stored" coarse operator (Sec. 3): the DPG system assembled directly on

@@ -25,6 +25,7 @@
 #include "block.cuh"
 #include "smoother.cuh"
 #include "classes.cuh"
+#include "cells.cuh"
 
 namespace dpgmg {
 
@@ -524,6 +525,7 @@ template <> struct SpmvSlot<double2> { static constexpr int v = 1; };
 constexpr int SPMV_PF = 16;
 constexpr int SPMV_RING = 32;   // one row per warp, (value, index) stream prefetched by cp.async
 constexpr int SPMV_HALF = 64;   // one row per half-warp (k_spmv_hw)
+constexpr int SPMV_CELLS = 128; // tuner only: the operator by cells (CellOpDev)
 // complex64 values with packed real entities: every SpMV but the cp.async
 // ring variant reads them
 template <class C> static const uint8_t* packed_rows(const ECSRDev& A) {
@@ -585,11 +587,17 @@ template <class C>
 static void spmv(const ECSRDev& A, const C* vals, const C* x, const C* b, C* y, int mode, cudaStream_t st,
                  SystemImpl* prof = nullptr) {
   int pe = prof_begin(prof, st);
-  spmv_g<C>(A, vals, x, b, y, mode, A.gsel[SpmvSlot<C>::v], st);
+  if constexpr (std::is_same<C, float2>::value) {
+    if (A.cell.on) cell_op_apply(A.cell, x, b, y, mode, st);
+    else spmv_g<C>(A, vals, x, b, y, mode, A.gsel[SpmvSlot<C>::v], st);
+  } else {
+    spmv_g<C>(A, vals, x, b, y, mode, A.gsel[SpmvSlot<C>::v], st);
+  }
   prof_end(prof, pe, st);
 }
 
 // ------------------------------------------------- double-float CG operator
+// (df_add, df_mul: cells.cuh)
 // The CG operator is stored as complex64 high and low parts (a = a_hi + a_lo,
 // exact to ~2^-48) and applied with error-free FP32 transformations
 // (TwoProduct by fma, TwoSum; Ogita, Rump and Oishi, "Accurate sum and dot
@@ -597,20 +605,6 @@ static void spmv(const ECSRDev& A, const C* vals, const C* x, const C* b, C* y, 
 // the cross terms a_hi x_lo + a_lo x_hi are added to the low accumulator.
 // The result carries ~48 significant bits, enough for the FP64 CG recurrence,
 // without the FP64 pipe that bounds a complex128 SpMV on this GPU.
-__device__ __forceinline__ void df_add(float& sh, float& sl, float p, float q) {
-  const float s = sh + p;
-  const float bb = s - sh;
-  const float e = (sh - (s - bb)) + (p - bb);
-  sh = s;
-  sl += e + q;
-}
-__device__ __forceinline__ void df_mul(float ah, float al, float xh, float xl, float& p, float& q) {
-  p = ah * xh;
-  q = fmaf(ah, xh, -p);
-  q = fmaf(ah, xl, q);
-  q = fmaf(al, xh, q);
-}
-
 // Warp sum of double-float values (h, l) with TwoSum on the high parts; every
 // lane ends with the same (h, l) (the exact error of a + b does not depend on
 // the order of the operands).
@@ -921,6 +915,10 @@ __global__ void k_split_vals(const double2* __restrict__ v, float2* __restrict__
 static void spmv_df_g(const ECSRDev& A, const float2* xh, const float2* xl, const double2* b, double2* y, int mode,
                       int G, cudaStream_t st) {
   const int64_t n = A.nrows;
+  if (G == SPMV_CELLS) {
+    cell_op_apply_df(A.cell, xh, xl, b, y, mode, st);
+    return;
+  }
   if (A.rent && G == SPMV_RING) G = SPMV_PF;   // the ring kernel reads complex64 values only
   if (G == SPMV_RING) {
     const int64_t blocks = std::min<int64_t>((n + 7) / 8, 152 * 5);
@@ -958,6 +956,9 @@ static void spmv_df_g(const ECSRDev& A, const float2* xh, const float2* xl, cons
     DPG_CHECK_LAUNCH();
   }
 }
+
+// form of the CG operator in force: by cells, or the assembled rows' tuned group
+static int cg_group(const ECSRDev& A) { return A.cell.df_on ? SPMV_CELLS : A.gsel[2]; }
 
 // Block form of the double-float CG operator: KB vectors (split into FP32
 // pairs xh/xl at stride ld), one warp per row, each stored pair (ah, al) loaded
@@ -1066,7 +1067,7 @@ static void spmv_df(const ECSRDev& A, const double2* x, const double2* b, double
   k_split_vec<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x, xh, xl, n);
   DPG_CHECK_LAUNCH();
   int pe = prof_begin(prof, st);
-  spmv_df_g(A, xh, xl, b, y, mode, A.gsel[2], st);
+  spmv_df_g(A, xh, xl, b, y, mode, cg_group(A), st);
   prof_end(prof, pe, st);
 }
 
@@ -1967,6 +1968,12 @@ template <class C>
 static void spmv_blk(const ECSRDev& A, const C* vals, const C* x, const C* b, C* y, int mode, int K,
                      cudaStream_t st) {
   const int64_t n = A.nrows;
+  if constexpr (std::is_same<C, float2>::value) {
+    if (A.cell.on) {   // shared cell matrices, read from L2 for every vector
+      for (int k = 0; k < K; ++k) cell_op_apply(A.cell, x + k * n, b ? b + k * n : nullptr, y + k * n, mode, st);
+      return;
+    }
+  }
   for (int g = 0; g < K; g += BLK_MAX) {
     const int kb = std::min(BLK_MAX, K - g);
     const C* xg = x + g * n;
@@ -2345,8 +2352,16 @@ void prepare_solve(SystemImpl& S, cudaStream_t st) {
     if (mixed) {
       float2 *x = W.w32[l].x, *y = W.w32[l].t;
       DPG_CUDA(cudaMemsetAsync(x, 0, (size_t)n * sizeof(float2), st));
-      F.A.gsel[0] = pick_group(key, ev, st, [&](int G) { spmv_g<float2>(F.A, F.A.v32, x, nullptr, y, 0, G, st); },
-                               F.A.rent != nullptr);
+      auto rows = [&](int G) { spmv_g<float2>(F.A, F.A.v32, x, nullptr, y, 0, G, st); };
+      F.A.gsel[0] = pick_group(key, ev, st, rows, F.A.rent != nullptr);
+      if (F.A.cell.W) {   // by cells, against the best assembled form
+        TuneKey ck = key;
+        ck.kind += 16 * (1 + log2i(F.A.cell.nitems));
+        F.A.cell.on = pick_variant(ck, ev, st, {SPMV_CELLS, F.A.gsel[0]}, [&](int G) {
+          if (G == SPMV_CELLS) cell_op_apply(F.A.cell, x, nullptr, y, 0, st);
+          else rows(G);
+        }) == SPMV_CELLS;
+      }
       if (F.P.inv32 && F.P.np) {
         // smoother product: shared blocks (classes.cuh), or 1 or 2 columns per lane (32- or 64-column work
         // items), the latter at 8 or 6 CTAs per SM; the block smoother takes
@@ -2381,8 +2396,13 @@ void prepare_solve(SystemImpl& S, cudaStream_t st) {
       Acg.gsel[1] = pick_group(key, ev, st, [&](int G) { spmv_g<double2>(Acg, Acg.v64, W.p, nullptr, W.q, 0, G, st); });
     } else {
       const TuneKey key{2, F.mesh.p, F.kind, log2i(n)};
-      Acg.gsel[2] = pick_group(key, ev, st, [&](int G) { spmv_df_g(Acg, W.xh, W.xl, nullptr, W.q, 0, G, st); },
-                               Acg.rent != nullptr, true);
+      auto run = [&](int G) { spmv_df_g(Acg, W.xh, W.xl, nullptr, W.q, 0, G, st); };
+      Acg.gsel[2] = pick_group(key, ev, st, run, Acg.rent != nullptr, true);
+      if (Acg.cell.Wlo) {
+        TuneKey ck = key;
+        ck.kind += 16 * (1 + log2i(Acg.cell.nitems16));
+        Acg.cell.df_on = pick_variant(ck, ev, st, {SPMV_CELLS, Acg.gsel[2]}, run) == SPMV_CELLS;
+      }
     }
   }
 }
@@ -2438,7 +2458,7 @@ int pcg_solve(SystemImpl& S, cudaStream_t st, double2* xout, dpgmg_stats* stats,
         spmv<double2>(A, A.v64, W.p, nullptr, W.q, 0, st, pcg_prof);
       } else if (presplit) {
         int pe = prof_begin(pcg_prof, st);
-        spmv_df_g(A, W.xh, W.xl, nullptr, W.q, 0, A.gsel[2], st);
+        spmv_df_g(A, W.xh, W.xl, nullptr, W.q, 0, cg_group(A), st);
         prof_end(pcg_prof, pe, st);
       } else {
         spmv_df(A, W.p, nullptr, W.q, 0, W.xh, W.xl, st, pcg_prof);
@@ -2565,6 +2585,12 @@ int pcg_solve_block(SystemImpl& S, cudaStream_t st, int K, const double2* B, dou
     }
     k_split_vec<<<nblk(n * K), 256, 0, st>>>(Xs, XH, XL, n * K);
     DPG_CHECK_LAUNCH();
+    if (A.cell.df_on) {
+      for (int k = 0; k < K; ++k)
+        cell_op_apply_df(A.cell, XH + (size_t)k * n, XL + (size_t)k * n, Bs ? Bs + (size_t)k * n : nullptr,
+                         Ys + (size_t)k * n, mode, st);
+      return;
+    }
     for (int g = 0; g < K; g += BLK_MAX) {
       const int kb = std::min(BLK_MAX, K - g);
       const double2* bg = Bs ? Bs + (size_t)g * n : nullptr;
