@@ -338,21 +338,60 @@ __global__ void __launch_bounds__(CTA_THREADS) k_elem_build(ElemArgs a) {
   (void)n1;
 }
 
+// Work split of the dense steps.  With element classes a mesh has a few dozen
+// representatives, fewer than the SMs, and the FP64 pipe of one SM (2 DFMA a
+// clock) bounds each step: so an element's Cholesky goes to a thread-block
+// cluster (CL), and its triangular solves, products and outputs to blockIdx.y:
+// a strip of right-hand sides, or a share of the output tiles.  Every entry is
+// computed by the same instructions in the same order for any split.
+__device__ __forceinline__ void strip(int total, int* c0, int* cnt) {   // TL-column strips over blockIdx.y
+  const int nt = (total + TL - 1) / TL, per = (nt + gridDim.y - 1) / gridDim.y;
+  *c0 = (int)blockIdx.y * per * TL;
+  *cnt = min(per * TL, total - *c0);
+}
+__device__ __forceinline__ unsigned elem_cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned elem_cluster_size() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+// CTA blockIdx.y's share of the output tiles of a product (no synchronisation
+// between the shares: the operands are complete before the launch)
+__device__ __forceinline__ Team<true> tile_share() {
+  Team<true> tm;
+  tm.rank = blockIdx.y;
+  tm.n = gridDim.y;
+  return tm;
+}
+
+template <bool CL>
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_potrf(ElemArgs a) {
   extern __shared__ double sh[];
-  const int64_t le = blockIdx.x;
+  Team<CL> tm;
+  if constexpr (CL) {
+    tm.rank = (int)elem_cluster_rank();
+    tm.n = (int)elem_cluster_size();
+  }
+  const int64_t le = blockIdx.x / tm.n;
   double* G = a.G + le * (size_t)a.nt * a.nt;
-  int info = cta_potrf<double>(G, a.nt, a.nt, sh);
-  if (threadIdx.x == 0 && info) atomicOr(a.info, 1);
+  int info = cta_potrf<double, CL>(G, a.nt, a.nt, sh, tm);
+  if (threadIdx.x == 0 && info && tm.rank == 0) atomicOr(a.info, 1);
 }
 
 template <class T>
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_trsm(ElemArgs a) {
   extern __shared__ char shc[];
   const int64_t le = blockIdx.x;
+  int c0, cnt;
+  strip(a.m + 1, &c0, &cnt);
+  if (cnt <= 0) return;
   const double* G = a.G + le * (size_t)a.nt * a.nt;
   T* W = reinterpret_cast<T*>(a.W) + le * (size_t)a.nt * (a.m + 1);
-  cta_trsm_lower<double, T>(G, a.nt, a.nt, W, a.m + 1, a.m + 1, shc);
+  cta_trsm_lower<double, T>(G, a.nt, a.nt, W + c0, cnt, a.m + 1, shc);
 }
 
 template <class T>
@@ -363,7 +402,8 @@ __global__ void __launch_bounds__(CTA_THREADS) k_elem_herk(ElemArgs a) {
   const T* W = reinterpret_cast<const T*>(a.W) + le * (size_t)a.nt * ld;
   T* K = reinterpret_cast<T*>(a.K) + le * (size_t)ld * ld;
   // K = W^H W is Hermitian: lower tiles plus their mirror
-  cta_herk_lower<T>(W, a.nt, ld, ld, K, ld, reinterpret_cast<T*>(shraw), false);
+  if (gridDim.y > 1) cta_herk_lower<T, true>(W, a.nt, ld, ld, K, ld, reinterpret_cast<T*>(shraw), false, tile_share());
+  else cta_herk_lower<T>(W, a.nt, ld, ld, K, ld, reinterpret_cast<T*>(shraw), false);
 }
 
 // ---- split path: real TRSM and HERK on [B_r | l' | B_i(p-hat)], then the
@@ -376,7 +416,9 @@ __global__ void __launch_bounds__(CTA_THREADS) k_elem_trsm_split(ElemArgs a) {
   const int ld2 = a.m + 1 + a.nph;
   const double* G = a.G + le * (size_t)a.nt * a.nt;
   double* W = reinterpret_cast<double*>(reinterpret_cast<double2*>(a.W) + le * (size_t)a.nt * (a.m + 1));
-  cta_trsm_lower<double, double>(G, a.nt, a.nt, W, ld2, ld2, shc);
+  int c0, cnt;
+  strip(ld2, &c0, &cnt);
+  if (cnt > 0) cta_trsm_lower<double, double>(G, a.nt, a.nt, W + c0, cnt, ld2, shc);
 }
 
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_herk_split(ElemArgs a) {
@@ -385,7 +427,10 @@ __global__ void __launch_bounds__(CTA_THREADS) k_elem_herk_split(ElemArgs a) {
   const int ld = a.m + 1, ld2 = ld + a.nph;
   const double* W = reinterpret_cast<const double*>(reinterpret_cast<const double2*>(a.W) + le * (size_t)a.nt * ld);
   double* R = reinterpret_cast<double*>(reinterpret_cast<double2*>(a.K) + le * (size_t)ld * ld);
-  cta_herk_lower<double>(W, a.nt, ld2, ld2, R, ld2, reinterpret_cast<double*>(shraw), false);
+  if (gridDim.y > 1)
+    cta_herk_lower<double, true>(W, a.nt, ld2, ld2, R, ld2, reinterpret_cast<double*>(shraw), false, tile_share());
+  else
+    cta_herk_lower<double>(W, a.nt, ld2, ld2, R, ld2, reinterpret_cast<double*>(shraw), false);
 }
 
 // R (real, ld2 x ld2, in the K slot) -> complex K' (ld x ld) in the same slot,
@@ -427,6 +472,32 @@ template <> __device__ __forceinline__ double2 from_c128<double2>(double2 v) { r
 template <> __device__ __forceinline__ double2 out_value<double2, true>(double2 v, int ph) { return phased_c(v, ph); }
 __device__ __forceinline__ int phase_of(bool a_i, bool b_i) { return (a_i && !b_i) ? 1 : ((!a_i && b_i) ? 2 : 0); }
 
+// Field condensation in three steps: K_ff = L L^H; Y = K_ff^-1 [K_ft | F_f] by
+// strips of columns; K_c = K_tt - K_tf Y and F_c by strips of rows, with the
+// strips' outputs (and a share of the recovery data Y).
+template <class T>
+__global__ void __launch_bounds__(CTA_THREADS) k_elem_field_potrf(ElemArgs a) {
+  extern __shared__ unsigned char shraw[];
+  const int64_t le = blockIdx.x;
+  const int ld = a.m + 1;
+  T* K = reinterpret_cast<T*>(a.K) + le * (size_t)ld * ld;
+  int info = cta_potrf<T>(K, a.nf, ld, reinterpret_cast<T*>(shraw));
+  if (threadIdx.x == 0 && info) atomicOr(a.info, 2);
+}
+
+template <class T>
+__global__ void __launch_bounds__(CTA_THREADS) k_elem_field_solve(ElemArgs a) {
+  extern __shared__ unsigned char shraw[];
+  const int64_t le = blockIdx.x;
+  const int ld = a.m + 1, nf = a.nf;
+  int c0, cnt;
+  strip(a.ntr + 1, &c0, &cnt);
+  if (cnt <= 0) return;
+  T* K = reinterpret_cast<T*>(a.K) + le * (size_t)ld * ld;
+  cta_trsm_lower<T, T>(K, nf, ld, K + nf + c0, cnt, ld, reinterpret_cast<char*>(shraw));
+  cta_trsm_lower_h<T>(K, nf, ld, K + nf + c0, cnt, ld, reinterpret_cast<char*>(shraw));
+}
+
 template <class T, bool PH = false>
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_condense(ElemArgs a) {
   extern __shared__ unsigned char shraw[];
@@ -435,21 +506,21 @@ __global__ void __launch_bounds__(CTA_THREADS) k_elem_condense(ElemArgs a) {
   const int64_t e = a.elist[a.e0 + le];
   const int ld = a.m + 1, nf = a.nf, ntr = a.ntr;
   T* K = reinterpret_cast<T*>(a.K) + le * (size_t)ld * ld;
-  int info = cta_potrf<T>(K, nf, ld, sh);
-  if (threadIdx.x == 0 && info) atomicOr(a.info, 2);
-  cta_trsm_lower<T, T>(K, nf, ld, K + nf, ntr + 1, ld, reinterpret_cast<char*>(sh));
-  cta_trsm_lower_h<T>(K, nf, ld, K + nf, ntr + 1, ld, reinterpret_cast<char*>(sh));
-  cta_gemm<T>(false, ntr, ntr + 1, nf, -1.0, K + (size_t)nf * ld, ld, K + nf, ld, 1.0, K + (size_t)nf * ld + nf, ld,
-              sh);
-  double2* E = a.Eout + e * (size_t)ntr * ntr;
-  for (int q = threadIdx.x; q < ntr * ntr; q += blockDim.x) {
-    int i = q / ntr, j = q % ntr;
-    E[q] = out_value<T, PH>(K[(size_t)(nf + i) * ld + nf + j], phase_of(a.tr[i].x == 0, a.tr[j].x == 0));
+  int r0, rows;
+  strip(ntr, &r0, &rows);
+  if (rows > 0) {
+    cta_gemm<T>(false, rows, ntr + 1, nf, -1.0, K + (size_t)(nf + r0) * ld, ld, K + nf, ld, 1.0,
+                K + (size_t)(nf + r0) * ld + nf, ld, sh);
+    double2* E = a.Eout + e * (size_t)ntr * ntr;
+    for (int q = threadIdx.x; q < rows * ntr; q += blockDim.x) {
+      int i = r0 + q / ntr, j = q % ntr;
+      E[(size_t)i * ntr + j] = out_value<T, PH>(K[(size_t)(nf + i) * ld + nf + j], phase_of(a.tr[i].x == 0, a.tr[j].x == 0));
+    }
+    for (int i = r0 + threadIdx.x; i < r0 + rows; i += blockDim.x)
+      a.Fc[e * ntr + i] = out_value<T, PH>(K[(size_t)(nf + i) * ld + a.m], a.tr[i].x == 0 ? 1 : 0);
   }
-  for (int i = threadIdx.x; i < ntr; i += blockDim.x)
-    a.Fc[e * ntr + i] = out_value<T, PH>(K[(size_t)(nf + i) * ld + a.m], a.tr[i].x == 0 ? 1 : 0);
   double2* Y = a.Yrec + e * (size_t)nf * (ntr + 1);
-  for (int q = threadIdx.x; q < nf * (ntr + 1); q += blockDim.x) {
+  for (int q = blockIdx.y * blockDim.x + threadIdx.x; q < nf * (ntr + 1); q += gridDim.y * blockDim.x) {
     int i = q / (ntr + 1), j = q % (ntr + 1);
     const bool fi = a.ff[i].x == 0;
     const int ph = (j < ntr) ? phase_of(fi, a.tr[j].x == 0) : (fi ? 1 : 0);
@@ -623,6 +694,64 @@ static size_t smem_bytes_dense(size_t elt) { return (size_t)(NB * NB + 2 * TL * 
 // operators) they are scratch.
 static void element_core(SystemImpl& S, Level& L, const std::vector<double>& cvals, bool finest, cudaStream_t st);
 
+// CTAs per element of a dense step with at most `most` shares: enough for two
+// CTAs on every SM (nb elements), one where the elements alone are that many.
+static unsigned elem_split(int nb, int most) {
+  int dev = 0, nsm = 0;
+  DPG_CUDA(cudaGetDevice(&dev));
+  DPG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  return (unsigned)std::max(1, std::min(most, (2 * nsm + nb - 1) / std::max(nb, 1)));
+}
+
+// Gram Cholesky of nb elements: clusters of 2, 4 or 8 CTAs while they all fit
+// the SMs at once
+static void launch_elem_potrf(const ElemArgs& a, int nb, size_t sm, cudaStream_t st) {
+  int dev = 0, nsm = 0;
+  DPG_CUDA(cudaGetDevice(&dev));
+  DPG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  int team = 1;
+  while (team < 8 && nb * team * 2 <= nsm && a.nt >= 64 * team) team *= 2;
+  if (team > 1) {
+    DPG_CUDA(cudaFuncSetAttribute(k_elem_potrf<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)team;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(nb * team));
+    cfg.blockDim = dim3(CTA_THREADS);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int ncl = 0;
+    if (cudaOccupancyMaxActiveClusters(&ncl, k_elem_potrf<true>, &cfg) == cudaSuccess && ncl >= 1) {
+      DPG_CUDA(cudaLaunchKernelEx(&cfg, k_elem_potrf<true>, a));
+      count_launch();
+      return;
+    }
+    (void)cudaGetLastError();
+  }
+  k_elem_potrf<false><<<nb, CTA_THREADS, sm, st>>>(a);
+  DPG_CHECK_LAUNCH();
+}
+
+// field condensation of nb elements (T, PH as k_elem_condense)
+template <class T, bool PH>
+static void launch_elem_condense(const ElemArgs& a, int nb, size_t sm, cudaStream_t st) {
+  const unsigned sp = elem_split(nb, (a.ntr + 1 + TL - 1) / TL);
+  DPG_CUDA(cudaFuncSetAttribute(k_elem_field_potrf<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  DPG_CUDA(cudaFuncSetAttribute(k_elem_field_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  DPG_CUDA(cudaFuncSetAttribute(k_elem_condense<T, PH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  k_elem_field_potrf<T><<<nb, CTA_THREADS, sm, st>>>(a);
+  DPG_CHECK_LAUNCH();
+  k_elem_field_solve<T><<<dim3(nb, sp), CTA_THREADS, sm, st>>>(a);
+  DPG_CHECK_LAUNCH();
+  k_elem_condense<T, PH><<<dim3(nb, sp), CTA_THREADS, sm, st>>>(a);
+  DPG_CHECK_LAUNCH();
+}
+
 void element_stage(SystemImpl& S, cudaStream_t st) { element_core(S, S.levels.back(), S.wavespeed, true, st); }
 
 void element_stage_level(SystemImpl& S, Level& L, cudaStream_t st) {
@@ -732,20 +861,15 @@ static void element_core(SystemImpl& S, Level& L, const std::vector<double>& cva
   const size_t sm_cplx = smem_bytes_dense(16);
   DPG_CUDA(cudaFuncSetAttribute(k_elem_build<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_build_max));
   DPG_CUDA(cudaFuncSetAttribute(k_elem_build<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_build_max));
-  DPG_CUDA(cudaFuncSetAttribute(k_elem_potrf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_real));
+  DPG_CUDA(cudaFuncSetAttribute(k_elem_potrf<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_real));
   DPG_CUDA(cudaFuncSetAttribute(k_elem_trsm<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_cplx));
   DPG_CUDA(cudaFuncSetAttribute(k_elem_trsm<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_cplx));
   DPG_CUDA(cudaFuncSetAttribute(k_elem_herk<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_cplx));
   DPG_CUDA(cudaFuncSetAttribute(k_elem_herk<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_cplx));
-  DPG_CUDA(cudaFuncSetAttribute(k_elem_condense<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_cplx));
-  DPG_CUDA(cudaFuncSetAttribute(k_elem_condense<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_cplx));
   DPG_CUDA(cudaFuncSetAttribute(k_elem_build<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)sm_build_max));
   DPG_CUDA(cudaFuncSetAttribute(k_elem_trsm_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_cplx));
   DPG_CUDA(cudaFuncSetAttribute(k_elem_herk_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_cplx));
-  DPG_CUDA(cudaFuncSetAttribute(k_elem_condense<double2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)sm_cplx));
-  // element lists: real path (no impedance face, real source) and complex path
   // element lists: real path (no impedance face, real source), split path
   // (impedance faces, Gaussian source: the only complex entries are the
   // impedance terms of the p-hat columns) and complex path (other sources)
@@ -763,6 +887,7 @@ static void element_core(SystemImpl& S, Level& L, const std::vector<double>& cva
     else if (split_ok) lsplit.push_back(e);
     else lcplx.push_back(e);
   }
+  const int nt1 = (int)((ld1 + TL - 1) / TL), nt2 = (int)((ld2 + TL - 1) / TL);   // tiles of the columns
   int64_t* dreal = upload(A, lreal, st);
   int64_t* dsplit = upload(A, lsplit, st);
   int64_t* dcplx = upload(A, lcplx, st);
@@ -773,16 +898,14 @@ static void element_core(SystemImpl& S, Level& L, const std::vector<double>& cva
       const int nb = (int)std::min<int64_t>(chunk, cnt - e0);
       k_elem_build<double, true><<<nb, CTA_THREADS, sm_build, st>>>(a);
       DPG_CHECK_LAUNCH();
-      k_elem_potrf<<<nb, CTA_THREADS, sm_real, st>>>(a);
+      launch_elem_potrf(a, nb, sm_real, st);
+      k_elem_trsm_split<<<dim3(nb, elem_split(nb, nt2)), CTA_THREADS, sm_cplx, st>>>(a);
       DPG_CHECK_LAUNCH();
-      k_elem_trsm_split<<<nb, CTA_THREADS, sm_cplx, st>>>(a);
-      DPG_CHECK_LAUNCH();
-      k_elem_herk_split<<<nb, CTA_THREADS, sm_cplx, st>>>(a);
+      k_elem_herk_split<<<dim3(nb, elem_split(nb, nt2 * (nt2 + 1) / 2)), CTA_THREADS, sm_cplx, st>>>(a);
       DPG_CHECK_LAUNCH();
       k_elem_split_assemble<<<nb, CTA_THREADS, 0, st>>>(a);
       DPG_CHECK_LAUNCH();
-      k_elem_condense<double2, true><<<nb, CTA_THREADS, sm_cplx, st>>>(a);
-      DPG_CHECK_LAUNCH();
+      launch_elem_condense<double2, true>(a, nb, sm_cplx, st);
     }
   };
   auto run_list = [&](const int64_t* dl, int64_t cnt, bool real) {
@@ -793,17 +916,16 @@ static void element_core(SystemImpl& S, Level& L, const std::vector<double>& cva
       if (real) k_elem_build<double><<<nb, CTA_THREADS, sm_build, st>>>(a);
       else k_elem_build<double2><<<nb, CTA_THREADS, sm_build, st>>>(a);
       DPG_CHECK_LAUNCH();
-      k_elem_potrf<<<nb, CTA_THREADS, sm_real, st>>>(a);
+      launch_elem_potrf(a, nb, sm_real, st);
+      const dim3 gt(nb, elem_split(nb, nt1)), gh(nb, elem_split(nb, nt1 * (nt1 + 1) / 2));
+      if (real) k_elem_trsm<double><<<gt, CTA_THREADS, sm_cplx, st>>>(a);
+      else k_elem_trsm<double2><<<gt, CTA_THREADS, sm_cplx, st>>>(a);
       DPG_CHECK_LAUNCH();
-      if (real) k_elem_trsm<double><<<nb, CTA_THREADS, sm_cplx, st>>>(a);
-      else k_elem_trsm<double2><<<nb, CTA_THREADS, sm_cplx, st>>>(a);
+      if (real) k_elem_herk<double><<<gh, CTA_THREADS, sm_cplx, st>>>(a);
+      else k_elem_herk<double2><<<gh, CTA_THREADS, sm_cplx, st>>>(a);
       DPG_CHECK_LAUNCH();
-      if (real) k_elem_herk<double><<<nb, CTA_THREADS, sm_cplx, st>>>(a);
-      else k_elem_herk<double2><<<nb, CTA_THREADS, sm_cplx, st>>>(a);
-      DPG_CHECK_LAUNCH();
-      if (real) k_elem_condense<double><<<nb, CTA_THREADS, sm_cplx, st>>>(a);
-      else k_elem_condense<double2><<<nb, CTA_THREADS, sm_cplx, st>>>(a);
-      DPG_CHECK_LAUNCH();
+      if (real) launch_elem_condense<double, false>(a, nb, sm_cplx, st);
+      else launch_elem_condense<double2, false>(a, nb, sm_cplx, st);
     }
   };
   // Element classes (Gaussian source: real loads, no boundary loads): the key
@@ -896,15 +1018,13 @@ static void element_core(SystemImpl& S, Level& L, const std::vector<double>& cva
       int64_t* de = nm ? upload(A, rmem, st) : nullptr;
       k_elem_build<double><<<nb, CTA_THREADS, sm_build, st>>>(a);
       DPG_CHECK_LAUNCH();
-      k_elem_potrf<<<nb, CTA_THREADS, sm_real, st>>>(a);
+      launch_elem_potrf(a, nb, sm_real, st);
+      k_elem_trsm<double><<<dim3(nb, elem_split(nb, nt1)), CTA_THREADS, sm_cplx, st>>>(a);
       DPG_CHECK_LAUNCH();
-      k_elem_trsm<double><<<nb, CTA_THREADS, sm_cplx, st>>>(a);
-      DPG_CHECK_LAUNCH();
-      k_elem_herk<double><<<nb, CTA_THREADS, sm_cplx, st>>>(a);
+      k_elem_herk<double><<<dim3(nb, elem_split(nb, nt1 * (nt1 + 1) / 2)), CTA_THREADS, sm_cplx, st>>>(a);
       DPG_CHECK_LAUNCH();
       if (nm) member_loads(rch, de, false);
-      k_elem_condense<double><<<nb, CTA_THREADS, sm_cplx, st>>>(a);
-      DPG_CHECK_LAUNCH();
+      launch_elem_condense<double, false>(a, nb, sm_cplx, st);
       if (nm) {
         int4* dch = upload(A, rch, st);
         k_elem_member_condense<double, false><<<(unsigned)rch.size(), CTA_THREADS, sm_cplx, st>>>(a, de, dch, Ub, Cb,
@@ -923,17 +1043,15 @@ static void element_core(SystemImpl& S, Level& L, const std::vector<double>& cva
       int64_t* de = nm ? upload(A, smem, st) : nullptr;
       k_elem_build<double, true><<<nb, CTA_THREADS, sm_build, st>>>(a);
       DPG_CHECK_LAUNCH();
-      k_elem_potrf<<<nb, CTA_THREADS, sm_real, st>>>(a);
+      launch_elem_potrf(a, nb, sm_real, st);
+      k_elem_trsm_split<<<dim3(nb, elem_split(nb, nt2)), CTA_THREADS, sm_cplx, st>>>(a);
       DPG_CHECK_LAUNCH();
-      k_elem_trsm_split<<<nb, CTA_THREADS, sm_cplx, st>>>(a);
-      DPG_CHECK_LAUNCH();
-      k_elem_herk_split<<<nb, CTA_THREADS, sm_cplx, st>>>(a);
+      k_elem_herk_split<<<dim3(nb, elem_split(nb, nt2 * (nt2 + 1) / 2)), CTA_THREADS, sm_cplx, st>>>(a);
       DPG_CHECK_LAUNCH();
       if (nm) member_loads(sch, de, true);   // before the assembly below reuses the W slots
       k_elem_split_assemble<<<nb, CTA_THREADS, 0, st>>>(a);
       DPG_CHECK_LAUNCH();
-      k_elem_condense<double2, true><<<nb, CTA_THREADS, sm_cplx, st>>>(a);
-      DPG_CHECK_LAUNCH();
+      launch_elem_condense<double2, true>(a, nb, sm_cplx, st);
       if (nm) {
         int4* dch = upload(A, sch, st);
         k_elem_member_condense<double2, true><<<(unsigned)sch.size(), CTA_THREADS, sm_cplx, st>>>(a, de, dch, Ub, Cb,
@@ -1079,8 +1197,7 @@ void error_indicator(SystemImpl& S, const double2* x, double* eta2, cudaStream_t
     const int nb = (int)std::min<int64_t>(chunk, nel - e0);
     k_elem_build<double2><<<nb, CTA_THREADS, sm_build, st>>>(a);
     DPG_CHECK_LAUNCH();
-    k_elem_potrf<<<nb, CTA_THREADS, sm_real, st>>>(a);
-    DPG_CHECK_LAUNCH();
+    launch_elem_potrf(a, nb, sm_real, st);
     k_elem_eta<<<nb, CTA_THREADS, sm_eta, st>>>(a, fields, L.dofs, x, eta2);
     DPG_CHECK_LAUNCH();
   }
