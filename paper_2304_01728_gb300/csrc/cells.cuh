@@ -10,7 +10,7 @@ namespace dpgmg {
 
 // The operator by cells: ybuf[cell][a] = (A_K R_K x)_a of every cell, then
 // k_cell_sum adds the cells of each DOF.
-static __global__ void __launch_bounds__(CLS_THREADS, 4) k_class_cell(const int32_t* __restrict__ idx,
+static __global__ void __launch_bounds__(CLS_THREADS, CLS_CTAS) k_class_cell(const int32_t* __restrict__ idx,
                                                             const int32_t* __restrict__ cls, int n, int64_t stride,
                                                             const int4* __restrict__ items,
                                                             const int32_t* __restrict__ mem,

@@ -33,6 +33,8 @@ namespace dpgmg {
 constexpr int CLS_K = 16;       // rows of W per stage
 constexpr int CLS_STAGES = 3;   // stages of W in flight
 constexpr int CLS_THREADS = 128;
+constexpr int CLS_MEM = 32;     // members per item at most
+constexpr int CLS_CTAS = 4;     // resident per SM at least (registers)
 
 typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 pack2(float a, float b) {
@@ -60,11 +62,13 @@ __device__ __forceinline__ void cp_async16_zfill(void* smem, const void* gmem, b
 
 struct ClassSmem {
   __align__(16) unsigned char w[CLS_STAGES][CLS_K * 64 * sizeof(float2)];
-  __align__(16) float2 r[2][CLS_K][32 + 2];   // + 2: 2-way conflicts on the stores, 16-byte rows
-  int64_t base[32];                           // members' first positions in the index list and in the output
+  __align__(16) float2 r[2][CLS_K][CLS_MEM + 2];   // + 2: 2-way conflicts on the stores, 16-byte rows
+  int64_t base[CLS_MEM];                            // members' first positions in the index list and in the output
 };
 
-// One work item: outputs a0 .. a0 + 4 TX - 1, members 0 .. cnt - 1 (cnt <= (128 / TX) MPT).
+// One work item: outputs a0 .. a0 + 4 TX - 1, members 0 .. cnt - 1 (cnt <= (128 / TX) MPT);
+// a thread owns 4 outputs x MPT members: 16-byte pieces of a row of W, neighbouring
+// threads' pieces next to each other (no bank conflicts).
 // W: row k at W + k ld (reals, or complex numbers for CX), n x n.
 // CX:  y_a = sum_k conj(W[k][a]) r_k;
 // !CX: y_a = i^(s_a) sum_k W[k][a] i^(-s_k) r_k, s = 1 on DOFs below offU (smoother.cuh).
@@ -78,6 +82,7 @@ __device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict
   constexpr int EL = CX ? 8 : 4;                      // bytes per stored entry
   constexpr int ROW16 = TM * EL / 16;                 // 16-byte pieces per row of a stage
   constexpr int NW = CLS_K * ROW16 / CLS_THREADS;     // of them per thread
+  constexpr int PW = 16 / EL;                         // outputs of a thread's 16-byte pieces, TX pieces apart
   const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
   const int gk = tid % CLS_K, gm = tid / CLS_K;       // gather: row in the chunk, first member (then + 8)
   const char* W = reinterpret_cast<const char*>(Wv) + (int64_t)a0 * EL;
@@ -141,18 +146,18 @@ __device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict
     load_w(c + CLS_STAGES - 1);
     load_val();                        // chunk c + 1 (indices loaded one chunk earlier)
     load_idx(c + 2);
-    const unsigned char* ws = sm.w[c % CLS_STAGES] + tx * (4 * EL);
+    const unsigned char* ws = sm.w[c % CLS_STAGES] + tx * 16;
     const float2* rs = &sm.r[c & 1][0][ty * MPT];
 #pragma unroll
     for (int k = 0; k < CLS_K; ++k) {
       f32x2 rv[MPT];
       if constexpr (MPT == 1) {
-        const float2 t = rs[k * (32 + 2)];
+        const float2 t = rs[k * (CLS_MEM + 2)];
         rv[0] = pack2(t.x, t.y);
       } else {
 #pragma unroll
         for (int m = 0; m < MPT; m += 2) {
-          const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(rs + k * (32 + 2) + m);
+          const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(rs + k * (CLS_MEM + 2) + m);
           rv[m] = t.x;
           rv[m + 1] = t.y;
         }
@@ -166,7 +171,7 @@ __device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict
           for (int u = 0; u < 4; ++u) acc[m][u] = fma2(w2[u], rv[m], acc[m][u]);
       } else {
         const float4 wa = *reinterpret_cast<const float4*>(ws + k * (TM * EL));
-        const float4 wb = *reinterpret_cast<const float4*>(ws + k * (TM * EL) + 16);
+        const float4 wb = *reinterpret_cast<const float4*>(ws + k * (TM * EL) + 16 * TX);
         const f32x2 wr[4] = {pack2(wa.x, wa.x), pack2(wa.z, wa.z), pack2(wb.x, wb.x), pack2(wb.z, wb.z)};
         const f32x2 wi[4] = {pack2(wa.y, wa.y), pack2(wa.w, wa.w), pack2(wb.y, wb.y), pack2(wb.w, wb.w)};
 #pragma unroll
@@ -182,7 +187,7 @@ __device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict
   }
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
-    const int a = a0 + 4 * tx + u;
+    const int a = a0 + (u / PW) * (PW * TX) + PW * tx + u % PW;
     if (a >= n) continue;
     const int s = !CX && rep_idx[a] < offU ? 1 : 0;
 #pragma unroll
@@ -198,7 +203,7 @@ __device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict
 // patches class by class and a class's first patch in mem[] order owns the
 // stored block (vptr, rflag of any member give the same).  blockIdx.y: vector.
 template <class TIN>
-__global__ void __launch_bounds__(CLS_THREADS, 4) k_class_apply(const int64_t* __restrict__ ptr,
+__global__ void __launch_bounds__(CLS_THREADS, CLS_CTAS) k_class_apply(const int64_t* __restrict__ ptr,
                                                              const int32_t* __restrict__ dofs,
                                                              const int64_t* __restrict__ vptr,
                                                              const int4* __restrict__ items,
