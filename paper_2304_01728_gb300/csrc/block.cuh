@@ -268,8 +268,7 @@ __global__ void k_slot_sum_blk(const int64_t* __restrict__ sptr, const int32_t* 
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (g >= n) return;
   const C* pb = pbuf + blockIdx.y * ldp;
-  C acc = Ops<C>::zero();
-  for (int64_t s = sptr[g]; s < sptr[g + 1]; ++s) acc = Ops<C>::add(acc, pb[slots[s]]);
+  C acc = sum_slots<C>(sptr, slots, pb, g);
   acc = Ops<C>::scale(acc, (typename Ops<C>::R)theta);
   C* yk = y + blockIdx.y * ld;
   yk[g] = accumulate ? Ops<C>::add(yk[g], acc) : acc;

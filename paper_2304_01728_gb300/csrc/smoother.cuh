@@ -289,14 +289,36 @@ inline void launch_patch_apply_c64(const PatchDev& P, int variant, const float2*
   DPG_CHECK_LAUNCH();
 }
 
+// sum over the slots of g in list order, four slots at a time: their indices,
+// then their values, are loaded together, so a DOF waits for two memory
+// latencies per four slots and not per slot (the sum's only cost: 5.5 us of a
+// 6.4 us launch on 1,241 DOFs before)
+template <class C>
+__device__ __forceinline__ C sum_slots(const int64_t* __restrict__ sptr, const int32_t* __restrict__ slots,
+                                       const C* __restrict__ v, int64_t g) {
+  C acc = Ops<C>::zero();
+  const int64_t s1 = sptr[g + 1];
+  for (int64_t s = sptr[g]; s < s1; s += 4) {
+    int32_t i[4];
+    C t[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) i[u] = s + u < s1 ? slots[s + u] : -1;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) t[u] = i[u] >= 0 ? v[i[u]] : Ops<C>::zero();
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i[u] >= 0) acc = Ops<C>::add(acc, t[u]);
+  }
+  return acc;
+}
+
 // y[g] = (accumulate ? y[g] : 0) + theta * sum_{slots of g} pbuf[slot]
 template <class C, class TOUT>
 __global__ void k_slot_sum(const int64_t* __restrict__ sptr, const int32_t* __restrict__ slots,
                            const C* __restrict__ pbuf, TOUT* __restrict__ y, int64_t n, double theta, int accumulate) {
   int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (g >= n) return;
-  C acc = Ops<C>::zero();
-  for (int64_t s = sptr[g]; s < sptr[g + 1]; ++s) acc = Ops<C>::add(acc, pbuf[slots[s]]);
+  C acc = sum_slots<C>(sptr, slots, pbuf, g);
   acc = Ops<C>::scale(acc, (typename Ops<C>::R)theta);
   TOUT o = cvt_in<TOUT>(acc);
   y[g] = accumulate ? Ops<TOUT>::add(y[g], o) : o;

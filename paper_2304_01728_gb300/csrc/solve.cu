@@ -1388,9 +1388,7 @@ __global__ void k_condense_sum(const int64_t* __restrict__ sptr, const int32_t* 
   int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (g >= n) return;
   if (!smask[g]) { rs[g] = Ops<C>::zero(); return; }
-  C acc = r[g];
-  for (int64_t s = sptr[g]; s < sptr[g + 1]; ++s) acc = Ops<C>::sub(acc, cbuf[slots[s]]);
-  rs[g] = acc;
+  rs[g] = Ops<C>::sub(r[g], sum_slots<C>(sptr, slots, cbuf, g));
 }
 
 // x_I = A_II^-1 r_I - Y x_S, one CTA per coarse element, one warp per row
@@ -1430,11 +1428,24 @@ __global__ void k_csr_real(const int64_t* __restrict__ ptr, const int32_t* __res
   if (i >= n) return;
   using R = typename Ops<C>::R;
   C acc = Ops<C>::zero();
-  for (int64_t k = ptr[i]; k < ptr[i + 1]; ++k) {
-    R v = (R)val[k];
-    C xv = x[col[k]];
-    acc.x += v * xv.x;
-    acc.y += v * xv.y;
+  const int64_t k1 = ptr[i + 1];
+  for (int64_t k = ptr[i]; k < k1; k += 4) {   // four entries' loads in flight; summed in order
+    int32_t c[4];
+    R v[4];
+    C xv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      c[u] = k + u < k1 ? col[k + u] : -1;
+      v[u] = k + u < k1 ? (R)val[k + u] : R(0);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) xv[u] = c[u] >= 0 ? x[c[u]] : Ops<C>::zero();
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c[u] >= 0) {
+        acc.x += v[u] * xv[u].x;
+        acc.y += v[u] * xv[u].y;
+      }
   }
   y[i] = accumulate ? Ops<C>::add(y[i], acc) : acc;
 }
@@ -1465,7 +1476,11 @@ __global__ void k_widen(const float2* a, double2* b, int64_t n) {
   if (i < n) b[i] = make_double2(a[i].x, a[i].y);
 }
 
-constexpr int RED_BLOCKS = 608;
+constexpr int RED_BLOCKS = 608;   // blocks of a reduction at most (4 per SM)
+// blocks of a reduction over n entries: one entry per thread until the cap.  A
+// block without entries only adds to the last block's work (n = 1,241: 11 us a
+// dot product with 608 blocks).
+static unsigned red_blocks(int64_t n) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>(RED_BLOCKS, (n + 255) / 256)); }
 
 // scalar slots of the CG state
 enum { SC_RHO = 0, SC_PQ, SC_ALPHA, SC_BETA, SC_RR, SC_RHONEW, SC_COUNT };
@@ -2124,7 +2139,7 @@ static std::vector<BlockLevel<C>> alloc_block_levels(Alloc& M, const SystemImpl&
 }
 
 static void dot(WS& W, const double2* u, const double2* v, int64_t n, int which, cudaStream_t st) {
-  k_dot_fused<double2><<<RED_BLOCKS, 256, 0, st>>>(u, v, n, W.part, W.sc, which, W.ticket);
+  k_dot_fused<double2><<<red_blocks(n), 256, 0, st>>>(u, v, n, W.part, W.sc, which, W.ticket);
   DPG_CHECK_LAUNCH();
 }
 
@@ -2464,7 +2479,7 @@ int pcg_solve(SystemImpl& S, cudaStream_t st, double2* xout, dpgmg_stats* stats,
         spmv_df(A, W.p, nullptr, W.q, 0, W.xh, W.xl, st, pcg_prof);
       }
       dot(W, W.p, W.q, n, 0, st);   // pq = p^H q
-      k_cg_update_fused<<<RED_BLOCKS, 256, 0, st>>>(W.x, W.r, W.p, W.q, W.sc, n, W.part, W.ticket, r32);
+      k_cg_update_fused<<<red_blocks(n), 256, 0, st>>>(W.x, W.r, W.p, W.q, W.sc, n, W.part, W.ticket, r32);
       DPG_CHECK_LAUNCH();
       DPG_CUDA(cudaMemcpyAsync(W.sc_host, W.sc, SC_COUNT * sizeof(double2), cudaMemcpyDeviceToHost, st));
     };
@@ -2474,14 +2489,14 @@ int pcg_solve(SystemImpl& S, cudaStream_t st, double2* xout, dpgmg_stats* stats,
         // r's complex64 copy comes from the CG update; z stays in complex64 and is widened on load
         precondition(S, W, W.r, nullptr, st, true);
         const float2* z32 = W.w32[Lf].x;
-        k_dot_fused<float2><<<RED_BLOCKS, 256, 0, st>>>(z32, W.r, n, W.part, W.sc, 2, W.ticket);
+        k_dot_fused<float2><<<red_blocks(n), 256, 0, st>>>(z32, W.r, n, W.part, W.sc, 2, W.ticket);
         DPG_CHECK_LAUNCH();
-        k_cg_dir<float2><<<RED_BLOCKS, 256, 0, st>>>(W.p, z32, W.sc, n, W.xh, W.xl);
+        k_cg_dir<float2><<<red_blocks(n), 256, 0, st>>>(W.p, z32, W.sc, n, W.xh, W.xl);
         DPG_CHECK_LAUNCH();
       } else {
         precondition(S, W, W.r, W.z, st);
         dot(W, W.z, W.r, n, 2, st);
-        k_cg_dir<double2><<<RED_BLOCKS, 256, 0, st>>>(W.p, W.z, W.sc, n, W.xh, W.xl);
+        k_cg_dir<double2><<<red_blocks(n), 256, 0, st>>>(W.p, W.z, W.sc, n, W.xh, W.xl);
         DPG_CHECK_LAUNCH();
       }
     };
@@ -2625,7 +2640,7 @@ int pcg_solve_block(SystemImpl& S, cudaStream_t st, int K, const double2* B, dou
       vcycle_blk<double2>(S, W, V64, L, R, Z, K, st);
     }
   };
-  const dim3 rgrid(RED_BLOCKS, (unsigned)K);
+  const dim3 rgrid(red_blocks(n), (unsigned)K);
   auto dot_blk = [&](const double2* U, const double2* Vv, int which, unsigned long long mask) {
     k_dot_fused_blk<double2><<<rgrid, 256, 0, st>>>(U, Vv, n, part, sc, which, ticket, mask);
     DPG_CHECK_LAUNCH();
@@ -2788,9 +2803,9 @@ __global__ void k_scale(C* x, int64_t n, const double2* sc, int slot) {
 
 template <class C>
 static void dot_t(WS& W, const C* u, const C* v, int64_t n, int which, cudaStream_t st) {
-  k_dot_partial_t<C><<<RED_BLOCKS, 256, 0, st>>>(u, v, n, W.part);
+  k_dot_partial_t<C><<<red_blocks(n), 256, 0, st>>>(u, v, n, W.part);
   DPG_CHECK_LAUNCH();
-  k_dot_finish<<<1, 256, 0, st>>>(W.part, RED_BLOCKS, W.sc, which);
+  k_dot_finish<<<1, 256, 0, st>>>(W.part, (int)red_blocks(n), W.sc, which);
   DPG_CHECK_LAUNCH();
 }
 
@@ -2828,13 +2843,13 @@ static void estimate_theta_c64(SystemImpl& S, Level& F, double* out, cudaStream_
   k_start_vector<float2><<<nblk(n), 256, 0, st>>>(x, n, F.P.slot_ptr);
   DPG_CHECK_LAUNCH();
   dot_t<float2>(W, x, x, n, 1, st);
-  k_scale<float2><<<RED_BLOCKS, 256, 0, st>>>(x, n, W.sc, SC_RR);
+  k_scale<float2><<<red_blocks(n), 256, 0, st>>>(x, n, W.sc, SC_RR);
   DPG_CHECK_LAUNCH();
   for (int k = 0; k < 30; ++k) {
     spmv<float2>(F.A, F.A.v32, x, nullptr, t, 0, st);
     smooth<float2>(F, t, y, 1.0, 0, pbuf, st);
     dot_t<float2>(W, y, y, n, 1, st);
-    k_scale<float2><<<RED_BLOCKS, 256, 0, st>>>(y, n, W.sc, SC_RR);
+    k_scale<float2><<<red_blocks(n), 256, 0, st>>>(y, n, W.sc, SC_RR);
     DPG_CHECK_LAUNCH();
     std::swap(x, y);
   }
@@ -2877,13 +2892,13 @@ static void estimate_theta_fp(SystemImpl& S, Level& F, const float2* plo, double
   k_start_vector<double2><<<nblk(n), 256, 0, st>>>(x, n, F.P.slot_ptr);
   DPG_CHECK_LAUNCH();
   dot_t<double2>(W, x, x, n, 1, st);
-  k_scale<double2><<<RED_BLOCKS, 256, 0, st>>>(x, n, W.sc, SC_RR);
+  k_scale<double2><<<red_blocks(n), 256, 0, st>>>(x, n, W.sc, SC_RR);
   DPG_CHECK_LAUNCH();
   for (int k = 0; k < 30; ++k) {
     op(x, t);
     sm(t, y);
     dot_t<double2>(W, y, y, n, 1, st);
-    k_scale<double2><<<RED_BLOCKS, 256, 0, st>>>(y, n, W.sc, SC_RR);
+    k_scale<double2><<<red_blocks(n), 256, 0, st>>>(y, n, W.sc, SC_RR);
     DPG_CHECK_LAUNCH();
     std::swap(x, y);
   }
