@@ -22,15 +22,16 @@ static __global__ void __launch_bounds__(CLS_THREADS, CLS_CTAS) k_class_cell(con
   const int4 it = items[blockIdx.x];
   const int cnt = it.y, a0 = it.z;
   const int e = mem[it.x], c = cls[e];
-  if ((int)threadIdx.x < cnt) sm.base[threadIdx.x] = (int64_t)mem[it.x + threadIdx.x] * n;
+  if ((int)threadIdx.x < cnt)
+    sm.base[threadIdx.x] = sm.obase[threadIdx.x] = (int64_t)mem[it.x + threadIdx.x] * n;
   __syncthreads();
   const float2* W = Wall + c * stride;
   const int32_t* rep = idx + (int64_t)e * n;
 #define DPG_ITEM(TX, MPT)                                                                                \
   if (rflag[c] != 0)                                                                                     \
-    class_item<float2, TX, MPT, false>(sm, W, patch_ldr(n), n, a0, cnt, idx, x, ybuf, rep, offU);        \
+    class_item<float2, TX, MPT, false>(sm, W, patch_ldr(n), n, n, a0, cnt, idx, x, x, n, ybuf, nullptr, rep, offU);  \
   else                                                                                                   \
-    class_item<float2, TX, MPT, true>(sm, W, patch_ld(n), n, a0, cnt, idx, x, ybuf, rep, offU)
+    class_item<float2, TX, MPT, true>(sm, W, patch_ld(n), n, n, a0, cnt, idx, x, x, n, ybuf, nullptr, rep, offU)
   switch (it.w) {
     case CLS_64x32: DPG_ITEM(16, 4); break;
     case CLS_64x16: DPG_ITEM(16, 2); break;
@@ -236,29 +237,37 @@ static __global__ void __launch_bounds__(CLS_THREADS, 4) k_class_cell_df(const i
 #undef DPG_ITEM
 }
 
-// slots of DOF g: a fixed-pitch row of tab, or a CSR row
-template <class F>
+// calls f(value) for the slots of DOF g in list order (a fixed-pitch row of
+// tab, or a CSR row); indices and then values are loaded up to four at a time
+template <class V, class F>
 __device__ __forceinline__ void for_slots(const int32_t* __restrict__ tab, const int64_t* __restrict__ sptr,
-                                          const int32_t* __restrict__ slots, int64_t offE, int64_t offF, int64_t g,
-                                          F&& f) {
+                                          const int32_t* __restrict__ slots, int64_t offE, int64_t offF,
+                                          const V* __restrict__ v, int64_t g, F&& f) {
+  auto four = [&](int4 t) {
+    V a, b, c, d;
+    if (t.x >= 0) a = v[t.x];
+    if (t.y >= 0) b = v[t.y];
+    if (t.z >= 0) c = v[t.z];
+    if (t.w >= 0) d = v[t.w];
+    if (t.x >= 0) f(a);
+    if (t.y >= 0) f(b);
+    if (t.z >= 0) f(c);
+    if (t.w >= 0) f(d);
+  };
   if (tab) {
     const int32_t* row = tab + cell_row(g, offE, offF);
-    if (g >= offF) {   // faces: the two sides in one load
+    if (g >= offF) {   // faces: the two sides
       const int2 t = *reinterpret_cast<const int2*>(row);
-      if (t.x >= 0) f(t.x);
-      if (t.y >= 0) f(t.y);
+      four(make_int4(t.x, t.y, -1, -1));
     } else {
-      const int cnt = g < offE ? 8 : 4;
-      for (int q = 0; q < cnt; q += 4) {
-        const int4 t = *reinterpret_cast<const int4*>(row + q);
-        if (t.x >= 0) f(t.x);
-        if (t.y >= 0) f(t.y);
-        if (t.z >= 0) f(t.z);
-        if (t.w >= 0) f(t.w);
-      }
+      four(*reinterpret_cast<const int4*>(row));
+      if (g < offE) four(*reinterpret_cast<const int4*>(row + 4));
     }
   } else {
-    for (int64_t s = sptr[g]; s < sptr[g + 1]; ++s) f(slots[s]);
+    const int64_t s1 = sptr[g + 1];
+    for (int64_t s = sptr[g]; s < s1; s += 4)
+      four(make_int4(slots[s], s + 1 < s1 ? slots[s + 1] : -1, s + 2 < s1 ? slots[s + 2] : -1,
+                     s + 3 < s1 ? slots[s + 3] : -1));
   }
 }
 
@@ -270,7 +279,7 @@ static __global__ void k_cell_sum(const int32_t* __restrict__ tab, const int64_t
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (g >= n) return;
   float2 acc = make_float2(0.f, 0.f);
-  for_slots(tab, sptr, slots, offE, offF, g, [&](int s) { acc = Ops<float2>::add(acc, ybuf[s]); });
+  for_slots(tab, sptr, slots, offE, offF, ybuf, g, [&](float2 v) { acc = Ops<float2>::add(acc, v); });
   y[g] = mode ? Ops<float2>::sub(b[g], acc) : acc;
 }
 
@@ -283,8 +292,7 @@ static __global__ void k_cell_sum_df(const int32_t* __restrict__ tab, const int6
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (g >= n) return;
   float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-  for_slots(tab, sptr, slots, offE, offF, g, [&](int s) {
-    const float4 v = ybuf[s];
+  for_slots(tab, sptr, slots, offE, offF, ybuf, g, [&](float4 v) {
     df_add(rh, rl, v.x, v.y);
     df_add(ih, il, v.z, v.w);
   });
@@ -309,6 +317,105 @@ inline void cell_op_apply(const CellOpDev& D, const float2* x, const float2* b, 
   DPG_CHECK_LAUNCH();
   k_cell_sum<<<(unsigned)((D.ndof + 255) / 256), 256, 0, st>>>(D.tab, D.sptr, D.slots, D.offE, D.offF, D.ybuf, b, y,
                                                               D.ndof, mode);
+  DPG_CHECK_LAUNCH();
+}
+
+// ---- macro-grid transfers with shared class matrices ----
+// BACK:  x_I = A_II^-1 r_I - Y x_S          (rows: I then S; outputs: I, scattered)
+// !BACK: cbuf[K][a] = sum_i conj(Y[i][a]) r_i (rows: I; outputs: S)
+// idx: [nK][nI + nS] DOFs, I then S.
+template <bool BACK>
+static __global__ void __launch_bounds__(CLS_THREADS, CLS_CTAS) k_class_macro(
+    const int32_t* __restrict__ idx, const int32_t* __restrict__ cls, int nI, int nS, int64_t stride,
+    const int4* __restrict__ items, const int32_t* __restrict__ mem, const float2* __restrict__ Wall,
+    const uint8_t* __restrict__ rflag, const float2* r, float2* out, int64_t offU) {
+  __shared__ ClassSmem sm;
+  const int4 it = items[blockIdx.x];
+  const int cnt = it.y, a0 = it.z;
+  const int K = mem[it.x], c = cls[K];
+  if ((int)threadIdx.x < cnt) {
+    const int64_t m = mem[it.x + threadIdx.x];
+    sm.base[threadIdx.x] = m * (nI + nS);
+    sm.obase[threadIdx.x] = BACK ? m * (nI + nS) : m * nS;
+  }
+  __syncthreads();
+  const float2* W = Wall + c * stride;
+  const int n = BACK ? nI + nS : nI, nout = BACK ? nI : nS;
+  const int32_t* rep = idx + (int64_t)K * (nI + nS) + (BACK ? 0 : nI);
+  const int32_t* oidx = BACK ? idx : nullptr;
+#define DPG_ITEM(TX, MPT)                                                                                            \
+  if (rflag[c] != 0)                                                                                                 \
+    class_item<float2, TX, MPT, false, BACK>(sm, W, patch_ldr(nout), n, nout, a0, cnt, idx, r, out, nI, out, oidx,   \
+                                             rep, offU);                                                             \
+  else                                                                                                               \
+    class_item<float2, TX, MPT, true, BACK>(sm, W, patch_ld(nout), n, nout, a0, cnt, idx, r, out, nI, out, oidx, rep, \
+                                            offU)
+  switch (it.w) {
+    case CLS_64x32: DPG_ITEM(16, 4); break;
+    case CLS_64x16: DPG_ITEM(16, 2); break;
+    case CLS_64x8: DPG_ITEM(16, 1); break;
+    case CLS_32x32: DPG_ITEM(8, 2); break;
+    default: DPG_ITEM(8, 1); break;
+  }
+#undef DPG_ITEM
+}
+
+// class matrices of both transfers from the first cell of every class (one CTA
+// per class): as reals when every entry is real once the unit phases are taken out
+static __global__ void k_macro_class(const int32_t* __restrict__ idx, const int64_t* __restrict__ rep, int nI, int nS,
+                                     int64_t offU, bool pack, const float2* __restrict__ Y,
+                                     const float2* __restrict__ Ai, float2* __restrict__ Wb, int64_t bstride,
+                                     float2* __restrict__ Wc, int64_t cstride, uint8_t* __restrict__ rflag) {
+  const int64_t c = blockIdx.x, K = rep[c];
+  const int32_t* g = idx + K * (nI + nS);
+  const float2 *Yk = Y + K * (int64_t)nI * nS, *Ak = Ai + K * (int64_t)nI * nI;
+  const int n = nI + nS;
+  auto phat = [&](int q) { return g[q] >= 0 && g[q] < offU ? 1 : 0; };
+  // entry (row i of I, column q of [I, S]) of [A_II^-1, -Y]
+  auto entry = [&](int i, int q) {
+    if (q < nI) return Ak[i * nI + q];
+    const float2 y = Yk[(int64_t)i * nS + q - nI];
+    return make_float2(-y.x, -y.y);
+  };
+  bool cplx = !pack;
+  if (pack)
+    for (int t = threadIdx.x; t < nI * n; t += blockDim.x)
+      if (mul_i(entry(t / n, t % n), phat(t % n) - phat(t / n)).y != 0.f) cplx = true;
+  cplx = __syncthreads_or(cplx) != 0;
+  float2 *B = Wb + c * bstride, *Cc = Wc + c * cstride;
+  const int lb = (int)(cplx ? patch_ld(nI) : patch_ldr(nI)), lc = (int)(cplx ? patch_ld(nS) : patch_ldr(nS));
+  for (int t = threadIdx.x; t < n * lb; t += blockDim.x) {   // B[k][a] = conj([A_II^-1, -Y][a][k])
+    const int k = t / lb, a = t % lb;
+    const float2 v = a < nI ? entry(a, k) : make_float2(0.f, 0.f);
+    if (cplx) B[t] = make_float2(v.x, -v.y);
+    else reinterpret_cast<float*>(B)[t] = a < nI ? mul_i(v, phat(k) - phat(a)).x : 0.f;
+  }
+  for (int t = threadIdx.x; t < nI * lc; t += blockDim.x) {  // C[i][a] = Y[i][a]
+    const int i = t / lc, a = t % lc;
+    const float2 v = a < nS ? Yk[(int64_t)i * nS + a] : make_float2(0.f, 0.f);
+    if (cplx) Cc[t] = v;
+    else reinterpret_cast<float*>(Cc)[t] = a < nS ? mul_i(v, phat(nI + a) - phat(i)).x : 0.f;
+  }
+  if (threadIdx.x == 0) rflag[c] = cplx ? 0 : 1;
+}
+
+static __global__ void k_macro_index(const int64_t* __restrict__ Ig, const int64_t* __restrict__ Sg, int nI, int nS,
+                                     int64_t nK, int32_t* __restrict__ idx) {
+  const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (q >= nK * (nI + nS)) return;
+  const int64_t K = q / (nI + nS);
+  const int i = (int)(q % (nI + nS));
+  idx[q] = (int32_t)(i < nI ? Ig[K * nI + i] : Sg[K * nS + i - nI]);
+}
+
+inline void macro_backsub(const MacroOpDev& D, const float2* r, float2* x, cudaStream_t st) {
+  k_class_macro<true><<<(unsigned)D.nbitems, CLS_THREADS, 0, st>>>(D.idx, D.cls, D.nI, D.nS, D.bstride(), D.bitems,
+                                                                  D.mem, D.Wb, D.rflag, r, x, D.offU);
+  DPG_CHECK_LAUNCH();
+}
+inline void macro_condense_apply(const MacroOpDev& D, const float2* r, float2* cbuf, cudaStream_t st) {
+  k_class_macro<false><<<(unsigned)D.ncitems, CLS_THREADS, 0, st>>>(D.idx, D.cls, D.nI, D.nS, D.cstride(), D.citems,
+                                                                   D.mem, D.Wc, D.rflag, r, cbuf, D.offU);
   DPG_CHECK_LAUNCH();
 }
 

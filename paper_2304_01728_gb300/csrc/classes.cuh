@@ -63,20 +63,22 @@ __device__ __forceinline__ void cp_async16_zfill(void* smem, const void* gmem, b
 struct ClassSmem {
   __align__(16) unsigned char w[CLS_STAGES][CLS_K * 64 * sizeof(float2)];
   __align__(16) float2 r[2][CLS_K][CLS_MEM + 2];   // + 2: 2-way conflicts on the stores, 16-byte rows
-  int64_t base[CLS_MEM];                            // members' first positions in the index list and in the output
+  int64_t base[CLS_MEM];                            // members' first positions in the index list
+  int64_t obase[CLS_MEM];                           // and in the output (or its index list)
 };
 
 // One work item: outputs a0 .. a0 + 4 TX - 1, members 0 .. cnt - 1 (cnt <= (128 / TX) MPT);
 // a thread owns 4 outputs x MPT members: 16-byte pieces of a row of W, neighbouring
 // threads' pieces next to each other (no bank conflicts).
-// W: row k at W + k ld (reals, or complex numbers for CX), n x n.
+// W: row k at W + k ld (reals, or complex numbers for CX), n x nout.  TWO: rows
+// from nsplit on gather from r2.  oidx: output positions by index list, or null.
 // CX:  y_a = sum_k conj(W[k][a]) r_k;
 // !CX: y_a = i^(s_a) sum_k W[k][a] i^(-s_k) r_k, s = 1 on DOFs below offU (smoother.cuh).
-template <class TIN, int TX, int MPT, bool CX>
-__device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict__ Wv, int64_t ld, int n, int a0,
-                                           int cnt, const int32_t* __restrict__ idx, const TIN* __restrict__ r,
-                                           float2* __restrict__ out, const int32_t* __restrict__ rep_idx,
-                                           int64_t offU) {
+template <class TIN, int TX, int MPT, bool CX, bool TWO = false>
+__device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict__ Wv, int64_t ld, int n, int nout,
+                                           int a0, int cnt, const int32_t* __restrict__ idx, const TIN* r,
+                                           const TIN* r2, int nsplit, float2* out, const int32_t* __restrict__ oidx,
+                                           const int32_t* __restrict__ rep_idx, int64_t offU) {
   constexpr int TM = 4 * TX, TN = (CLS_THREADS / TX) * MPT;
   constexpr int NG = TN / 8;                          // gathered values per thread and chunk
   constexpr int EL = CX ? 8 : 4;                      // bytes per stored entry
@@ -112,12 +114,13 @@ __device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict
       gi[q] = (k < n && m < cnt) ? __ldg(idx + sm.base[m] + k) : -1;
     }
   };
-  auto load_val = [&]() {
+  auto load_val = [&](int c) {
+    const TIN* src = TWO && c * CLS_K + gk >= nsplit ? r2 : r;
 #pragma unroll
     for (int q = 0; q < NG; ++q) {
       float2 v = make_float2(0.f, 0.f);
       if (gi[q] >= 0) {
-        v = cvt_in<float2>(r[gi[q]]);
+        v = cvt_in<float2>(src[gi[q]]);
         if (!CX) v = mul_i(v, gi[q] < offU ? -1 : 0);
       }
       gv[q] = v;
@@ -137,14 +140,14 @@ __device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict
 #pragma unroll
   for (int c = 0; c < CLS_STAGES - 1; ++c) load_w(c);
   load_idx(0);
-  load_val();
+  load_val(0);
   store_val(0);
   load_idx(1);
   for (int c = 0; c < nch; ++c) {
     cp_async_wait<CLS_STAGES - 2>();   // this thread's pieces of stage c have landed
     __syncthreads();                   // everybody's have, and everybody is done with chunk c - 1
     load_w(c + CLS_STAGES - 1);
-    load_val();                        // chunk c + 1 (indices loaded one chunk earlier)
+    load_val(c + 1);                   // chunk c + 1 (indices loaded one chunk earlier)
     load_idx(c + 2);
     const unsigned char* ws = sm.w[c % CLS_STAGES] + tx * 16;
     const float2* rs = &sm.r[c & 1][0][ty * MPT];
@@ -188,12 +191,12 @@ __device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int a = a0 + (u / PW) * (PW * TX) + PW * tx + u % PW;
-    if (a >= n) continue;
+    if (a >= nout) continue;
     const int s = !CX && rep_idx[a] < offU ? 1 : 0;
 #pragma unroll
     for (int m = 0; m < MPT; ++m) {
       const int q = ty * MPT + m;
-      if (q < cnt) out[sm.base[q] + a] = mul_i(unpack2(acc[m][u]), s);
+      if (q < cnt) out[oidx ? (int64_t)oidx[sm.obase[q] + a] : sm.obase[q] + a] = mul_i(unpack2(acc[m][u]), s);
     }
   }
 }
@@ -220,15 +223,15 @@ __global__ void __launch_bounds__(CLS_THREADS, CLS_CTAS) k_class_apply(const int
   const int j = mem[it.x];
   const int64_t b = ptr[j];
   const int n = (int)(ptr[j + 1] - b);
-  if ((int)threadIdx.x < cnt) sm.base[threadIdx.x] = ptr[mem[it.x + threadIdx.x]];
+  if ((int)threadIdx.x < cnt) sm.base[threadIdx.x] = sm.obase[threadIdx.x] = ptr[mem[it.x + threadIdx.x]];
   __syncthreads();
   const float2* W = inv + vptr[j];
   const int32_t* rep = dofs + b;
 #define DPG_ITEM(TX, MPT)                                                                                         \
   if (rflag != nullptr && rflag[j] != 0)                                                                          \
-    class_item<TIN, TX, MPT, false>(sm, W, patch_ldr(n), n, a0, cnt, dofs, r, pbuf, rep, offU);                   \
+    class_item<TIN, TX, MPT, false>(sm, W, patch_ldr(n), n, n, a0, cnt, dofs, r, r, n, pbuf, nullptr, rep, offU);   \
   else                                                                                                            \
-    class_item<TIN, TX, MPT, true>(sm, W, patch_ld(n), n, a0, cnt, dofs, r, pbuf, rep, offU)
+    class_item<TIN, TX, MPT, true>(sm, W, patch_ld(n), n, n, a0, cnt, dofs, r, r, n, pbuf, nullptr, rep, offU)
   switch (it.w) {   // CLS_SHAPE_*: outputs x members of the item
     case CLS_64x32: DPG_ITEM(16, 4); break;
     case CLS_64x16: DPG_ITEM(16, 2); break;

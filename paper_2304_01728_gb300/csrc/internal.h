@@ -95,6 +95,23 @@ inline int64_t cell_row(int64_t g, int64_t offE, int64_t offF) {
   return g < offE ? 8 * g : (g < offF ? 8 * offE + 4 * (g - offE) : 8 * offE + 4 * (offF - offE) + 2 * (g - offF));
 }
 
+// Macro-grid transfers with one stored matrix per macro class (cells.cuh)
+struct MacroOpDev {
+  bool back = false, cond = false;   // back-substitution, condensation by classes (tuned)
+  int nI = 0, nS = 0;
+  int64_t offU = 0;
+  int32_t* idx = nullptr;      // [nK][nI + nS] DOFs, I then S
+  int32_t* cls = nullptr;      // [nK] class
+  float2* Wb = nullptr;        // per class conj([A_II^-1, -Y])^T, (nI + nS) rows of nI
+  float2* Wc = nullptr;        // per class Y, nI rows of nS
+  uint8_t* rflag = nullptr;    // per class: stored as reals
+  int4 *bitems = nullptr, *citems = nullptr;
+  int64_t nbitems = 0, ncitems = 0;
+  int32_t* mem = nullptr;
+  int64_t bstride() const { return (nI + nS) * patch_ld(nI); }
+  int64_t cstride() const { return nI * patch_ld(nS); }
+};
+
 struct ECSRDev {
   int64_t nrows = 0, nent = 0, nnz = 0, max_nnz_row = 0;
   int64_t nnz_alg = 0;     // operator entries (algorithmic bytes count these)
@@ -202,6 +219,7 @@ struct Level {
   double2* Ai64 = nullptr;   // [nK][nI][nI]   A_II^-1
   float2* Y32 = nullptr;
   float2* Ai32 = nullptr;
+  MacroOpDev mop;            // mixed path, shared macro classes: when mop.back / mop.cond
   int64_t *P_ptr = nullptr, *PT_ptr = nullptr, *sslot_ptr = nullptr;
   int32_t *P_col = nullptr, *PT_col = nullptr, *sslots = nullptr;
   double *P_val = nullptr, *PT_val = nullptr;
@@ -251,6 +269,7 @@ struct LevelPlan {
   std::vector<int64_t> orep;       // first cell of each class
   std::vector<int4> oitems, oitems16;
   std::vector<int32_t> omem;
+  std::vector<int4> mbitems, mcitems;   // macro transfers: outputs I, outputs S
   int64_t max_n = 0, sum_sq = 0;
 };
 struct HostPlan {
@@ -363,6 +382,8 @@ void spmv64(const ECSRDev& A, const double2* x, double2* y, cudaStream_t st);
 // (the level's operator must carry its double-float split v32 + vlo, its patch
 // inverses their high parts in P.inv32 and low parts in plo)
 void estimate_theta(SystemImpl& S, int level, double* rayleigh, const float2* plo, cudaStream_t st);
+// class matrices and work items of an h level's macro transfers (mixed path; needs Y32 and Ai32)
+void macro_op_setup(SystemImpl& S, Level& F, const LevelPlan& lp, cudaStream_t st);
 // double-float split of an operator's values: v32 (kept if already set) + vlo
 void split_operator(Alloc& M, ECSRDev& A, int64_t offU, bool pack, cudaStream_t st);
 void operator_c64(Alloc& M, ECSRDev& A, int64_t offU, bool pack, cudaStream_t st);

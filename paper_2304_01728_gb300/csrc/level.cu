@@ -987,7 +987,8 @@ static void plan_patch_classes(LevelPlan& lp, const std::vector<int32_t>& cells,
 
 // The same for the operator by cells: one matrix per cell class, n local DOFs.
 // Kept when a matrix serves at least CLS_MIN_SHARE cells on average.
-static void plan_cell_classes(LevelPlan& lp, const std::vector<int32_t>& cells, int n) {
+// nI: macro-interior DOFs on an h level (its transfers share the classes), 0 on a p level.
+static void plan_cell_classes(LevelPlan& lp, const std::vector<int32_t>& cells, int n, int nI) {
   if (cells.empty()) return;
   std::vector<std::vector<int32_t>> members;
   for (size_t e = 0; e < cells.size(); ++e) {
@@ -1004,6 +1005,13 @@ static void plan_cell_classes(LevelPlan& lp, const std::vector<int32_t>& cells, 
   class_items(members, size_of, lp.omem, lp.oitems);
   lp.omem.clear();
   class_items(members, size_of, lp.omem, lp.oitems16, 16);
+  if (nI > 0) {
+    lp.omem.clear();
+    class_items(members, size_of, lp.omem, lp.mcitems);   // outputs S
+    auto in_of = [&](int64_t) { return (int64_t)nI; };
+    lp.omem.clear();
+    class_items(members, in_of, lp.omem, lp.mbitems);     // outputs I
+  }
 }
 
 // Host index plan of a hierarchy (every level's integer structures); runs on
@@ -1076,7 +1084,8 @@ std::shared_ptr<HostPlan> plan_host(const SystemImpl& S) {
     }
     plan_patch_classes(lp, cells[l > 0 ? l - 1 : 0], C.mesh.n);
     if (S.op.precision == DPGMG_PREC_MIXED)
-      plan_cell_classes(lp, F.kind == 2 ? cells[l - 1] : cells[l], F.kind == 2 ? lp.M.nS : (int)F.mesh.loc.size());
+      plan_cell_classes(lp, F.kind == 2 ? cells[l - 1] : cells[l], F.kind == 2 ? lp.M.nS : (int)F.mesh.loc.size(),
+                        F.kind == 2 ? lp.M.nI : 0);
     for (int64_t j = 0; j < np; ++j)
       if (lp.prep[j] == j) lp.order.push_back(j);
     std::stable_sort(lp.order.begin(), lp.order.end(), [&](int64_t u, int64_t v) { return size_of(u) > size_of(v); });
@@ -1254,6 +1263,7 @@ void build_hierarchy(SystemImpl& S, cudaStream_t st) {
       split_df(Pd.inv64, Pd.inv32, plo, Pd.nvals, st);
       if (!F.A.vlo) split_operator(A, F.A, F.mesh.offU, pack_storage(S), st);
     }
+    if (F.kind == 2 && F.Y32) macro_op_setup(S, F, lp, st);
     estimate_theta(S, l, dtheta + 2 * l, plo, st);
     if (plo) A.release(plo);
     if (F.A.vlo && !keep_split) {
@@ -1293,6 +1303,7 @@ void build_hierarchy(SystemImpl& S, cudaStream_t st) {
       if (F.kind == 2 && !F.Y32) {
         F.Y32 = to_c64(A, F.Y64, F.nK * F.nI * F.nS, st);
         F.Ai32 = to_c64(A, F.Ai64, F.nK * F.nI * F.nI, st);
+        macro_op_setup(S, F, lp, st);
       }
     }
   }

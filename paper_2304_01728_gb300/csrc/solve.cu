@@ -1461,6 +1461,34 @@ __global__ void k_scatter_add(const int32_t* __restrict__ idx, const C* __restri
   if (i < n) y[idx[i]] = Ops<C>::add(y[idx[i]], x[i]);
 }
 
+void macro_op_setup(SystemImpl& S, Level& F, const LevelPlan& lp, cudaStream_t st) {
+  if (lp.mbitems.empty() || !F.Y32) return;
+  Alloc& A = S.mem;
+  MacroOpDev& D = F.mop;
+  D.nI = F.nI;
+  D.nS = F.nS;
+  D.offU = F.mesh.offU;
+  const int64_t ncls = (int64_t)lp.orep.size(), total = F.nK * (F.nI + F.nS);
+  D.idx = A.arr<int32_t>((size_t)total);
+  D.cls = F.A.cell.cls;
+  D.mem = F.A.cell.mem;
+  D.Wb = A.arr<float2>((size_t)(ncls * D.bstride()));
+  D.Wc = A.arr<float2>((size_t)(ncls * D.cstride()));
+  D.rflag = A.arr<uint8_t>((size_t)ncls);
+  D.bitems = upload(A, lp.mbitems, st);
+  D.nbitems = (int64_t)lp.mbitems.size();
+  D.citems = upload(A, lp.mcitems, st);
+  D.ncitems = (int64_t)lp.mcitems.size();
+  k_macro_index<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(F.I_glob, F.S_glob, F.nI, F.nS, F.nK, D.idx);
+  DPG_CHECK_LAUNCH();
+  int64_t* rep = upload(A, lp.orep, st);
+  k_macro_class<<<(unsigned)ncls, 256, 0, st>>>(D.idx, rep, F.nI, F.nS, D.offU, pack_storage(S), F.Y32, F.Ai32, D.Wb,
+                                               D.bstride(), D.Wc, D.cstride(), D.rflag);
+  DPG_CHECK_LAUNCH();
+  A.release(rep);
+  D.back = D.cond = true;   // until setup has timed them
+}
+
 // ------------------------------------------------------------- vector ops
 template <class C>
 __global__ void k_zero(C* y, int64_t n) {
@@ -1793,15 +1821,28 @@ static void prolong_add(const Level& F, const Level& Cl, const C* ec, C* x, cuda
 
 template <class C>
 static void condense(const Level& F, const C* r, C* rs, C* cbuf, cudaStream_t st) {
-  size_t sm = (size_t)F.nI * sizeof(C) + 16;
-  k_condense_apply<C><<<(unsigned)F.nK, 256, sm, st>>>(F.nS, F.nI, F.I_glob, Prec<C>::Y(F), r, cbuf);
-  DPG_CHECK_LAUNCH();
+  bool done = false;
+  if constexpr (std::is_same<C, float2>::value)
+    if (F.mop.cond) {
+      macro_condense_apply(F.mop, r, cbuf, st);
+      done = true;
+    }
+  if (!done) {
+    size_t sm = (size_t)F.nI * sizeof(C) + 16;
+    k_condense_apply<C><<<(unsigned)F.nK, 256, sm, st>>>(F.nS, F.nI, F.I_glob, Prec<C>::Y(F), r, cbuf);
+    DPG_CHECK_LAUNCH();
+  }
   k_condense_sum<C><<<nblk(F.mesh.ndof), 256, 0, st>>>(F.sslot_ptr, F.sslots, cbuf, F.smask, r, rs, F.mesh.ndof);
   DPG_CHECK_LAUNCH();
 }
 
 template <class C>
 static void backsub(const Level& F, const C* r, C* x, cudaStream_t st) {
+  if constexpr (std::is_same<C, float2>::value)
+    if (F.mop.back) {
+      macro_backsub(F.mop, r, x, st);
+      return;
+    }
   size_t sm = (size_t)(F.nI + F.nS) * sizeof(C) + 16;
   k_backsub<C><<<(unsigned)F.nK, 256, sm, st>>>(F.nS, F.nI, F.S_glob, F.I_glob, Prec<C>::Ai(F), Prec<C>::Y(F), r, x);
   DPG_CHECK_LAUNCH();
@@ -2017,8 +2058,8 @@ template <class C> static int blk_group(int64_t per_vec) {
 template <class C>
 static void condense_blk(const Level& F, const C* r, C* rs, C* cbuf, int K, cudaStream_t st) {
   const int64_t n = F.mesh.ndof, ldc = (int64_t)F.nK * F.nS;
-  const int cap = blk_group<C>(F.nI);
-  if (cap < 1) {
+  const int cap = F.mop.cond ? 0 : blk_group<C>(F.nI);
+  if (cap < 1) {   // shared classes, or too large a block: one vector at a time
     for (int k = 0; k < K; ++k) condense<C>(F, r + k * n, rs + k * n, cbuf, st);
     return;
   }
@@ -2046,7 +2087,7 @@ static void condense_blk(const Level& F, const C* r, C* rs, C* cbuf, int K, cuda
 template <class C>
 static void backsub_blk(const Level& F, const C* r, C* x, int K, cudaStream_t st) {
   const int64_t n = F.mesh.ndof;
-  const int cap = blk_group<C>((int64_t)F.nI + F.nS);
+  const int cap = F.mop.back ? 0 : blk_group<C>((int64_t)F.nI + F.nS);
   if (cap < 1) {
     for (int k = 0; k < K; ++k) backsub<C>(F, r + k * n, x + k * n, st);
     return;
@@ -2376,6 +2417,18 @@ void prepare_solve(SystemImpl& S, cudaStream_t st) {
           if (G == SPMV_CELLS) cell_op_apply(F.A.cell, x, nullptr, y, 0, st);
           else rows(G);
         }) == SPMV_CELLS;
+      }
+      if (F.mop.Wb) {   // macro transfers by classes, or one CTA per coarse element
+        const TuneKey bk{5 + 16 * (1 + log2i(F.mop.nbitems)), F.mesh.p, F.kind, log2i(F.nK)};
+        const TuneKey ckk{6 + 16 * (1 + log2i(F.mop.ncitems)), F.mesh.p, F.kind, log2i(F.nK)};
+        F.mop.back = pick_variant(bk, ev, st, {1, 0}, [&](int v) {
+          F.mop.back = v == 1;
+          backsub<float2>(F, x, y, st);
+        }) == 1;
+        F.mop.cond = pick_variant(ckk, ev, st, {1, 0}, [&](int v) {
+          F.mop.cond = v == 1;
+          condense<float2>(F, x, y, W.w32[l].cbuf, st);
+        }) == 1;
       }
       if (F.P.inv32 && F.P.np) {
         // smoother product: shared blocks (classes.cuh), or 1 or 2 columns per lane (32- or 64-column work
