@@ -13,6 +13,8 @@
 // dependency between rows (one warp per row, coalesced row reads).
 #include <algorithm>
 #include <cmath>
+#include <map>
+#include <mutex>
 
 #include "common.cuh"
 #include "internal.h"
@@ -20,6 +22,7 @@
 namespace dpgmg {
 
 constexpr int CNB = 64;   // block width of the dense kernels
+constexpr int SMALL_TILES = 76;   // 64 x 64 tiles up to which a product runs on 32 x 32 tiles (half the SMs)
 
 template <class C> __device__ __forceinline__ C warp_sum_c(C v) {
   for (int o = 16; o > 0; o >>= 1) {
@@ -104,7 +107,7 @@ __global__ void __launch_bounds__(CTA_THREADS) k_dense_diag(C* A, int64_t N, int
   if (tid < kb) rdiag[tid] = R(1) / O::re(D[tid * LD + tid]);
   __syncthreads();
   // X = L_kk^-1 row by row: X[r][c] = (delta_rc - sum_{c<=t<r} L[r][t] X[t][c]) / L[r][r];
-  // four lanes per column split the sum
+  // four lanes of one warp per column split the sum, so rows need no CTA barrier
   const int col = tid / 4, part = tid % 4;
   for (int r = 0; r < kb; ++r) {
     C acc = O::zero();
@@ -116,8 +119,9 @@ __global__ void __launch_bounds__(CTA_THREADS) k_dense_diag(C* A, int64_t N, int
     }
     if (part == 0 && col <= r && col < kb)
       X[r * LD + col] = O::scale(O::sub(r == col ? O::from_re(R(1)) : O::zero(), acc), rdiag[r]);
-    __syncthreads();
+    __syncwarp();
   }
+  __syncthreads();
   C* Dk = Dinv + (size_t)(k0 / CNB) * CNB * CNB;
   for (int q = tid; q < CNB * CNB; q += blockDim.x) {
     const int r = q / CNB, c = q % CNB;
@@ -127,9 +131,9 @@ __global__ void __launch_bounds__(CTA_THREADS) k_dense_diag(C* A, int64_t N, int
 }
 
 // Panel: rows i >= k0 + kb, A[i, k0:k0+kb] <- A[i, k0:k0+kb] L_kk^-H, as the
-// product with the stored inverse (one CTA per 64 rows; thread (tx, ty) owns
-// rows ty*4 + a and columns tx + 16 b).
-template <class C>
+// product with the stored inverse (one CTA per 16 Q rows; thread (tx, ty) owns
+// rows ty*Q + a and columns tx + 16 b).
+template <class C, int Q>
 __global__ void __launch_bounds__(CTA_THREADS) k_dense_panel(C* A, int64_t N, int64_t ld, int k0,
                                                              const C* __restrict__ Dinv) {
   extern __shared__ unsigned char shraw[];
@@ -138,38 +142,42 @@ __global__ void __launch_bounds__(CTA_THREADS) k_dense_panel(C* A, int64_t N, in
   C* Pa = reinterpret_cast<C*>(shraw);   // [CNB][LD] Pa[r][t] = A[i0 + r][k0 + t]
   C* Bt = Pa + CNB * LD;                 // [CNB][LD] Bt[t][j] = conj(L_kk^-1[j][t])
   const int kb = (int)(N - k0 < CNB ? N - k0 : CNB);
-  const int64_t i0 = (int64_t)k0 + kb + (int64_t)blockIdx.x * CNB;
+  const int64_t i0 = (int64_t)k0 + kb + (int64_t)blockIdx.x * (16 * Q);
   const C* Dk = Dinv + (size_t)(k0 / CNB) * CNB * CNB;
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
   for (int q = tid; q < CNB * CNB; q += blockDim.x) {
     const int r = q / CNB, t = q % CNB;
-    Pa[r * LD + t] = (i0 + r < N && t < kb) ? A[(size_t)(i0 + r) * ld + k0 + t] : O::zero();
+    if (r < 16 * Q) Pa[r * LD + t] = (i0 + r < N && t < kb) ? A[(size_t)(i0 + r) * ld + k0 + t] : O::zero();
     Bt[t * LD + r] = O::conj(Dk[q]);
   }
   __syncthreads();
-  C acc[4][4];
-  for (int a = 0; a < 4; ++a)
+  C acc[Q][4];
+  for (int a = 0; a < Q; ++a)
     for (int b = 0; b < 4; ++b) acc[a][b] = O::zero();
   for (int t = 0; t < kb; ++t) {
-    C av[4], bv[4];
-    for (int a = 0; a < 4; ++a) av[a] = Pa[(ty * 4 + a) * LD + t];
+    C av[Q], bv[4];
+    for (int a = 0; a < Q; ++a) av[a] = Pa[(ty * Q + a) * LD + t];
     for (int b = 0; b < 4; ++b) bv[b] = Bt[t * LD + tx + 16 * b];
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < Q; ++a)
       for (int b = 0; b < 4; ++b) acc[a][b] = O::fma(av[a], bv[b], acc[a][b]);
   }
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < Q; ++a)
     for (int b = 0; b < 4; ++b) {
-      const int64_t i = i0 + ty * 4 + a;
+      const int64_t i = i0 + ty * Q + a;
       const int j = tx + 16 * b;
       if (i < N && j < kb) A[(size_t)i * ld + k0 + j] = acc[a][b];
     }
 }
 
-// trailing update of one lower 64x64 tile pair: A[i][j] -= sum_t L[i][t] conj(L[j][t])
-template <class C>
+// trailing update of one lower T x T tile pair: A[i][j] -= sum_t L[i][t] conj(L[j][t]).
+// T = 64 where the tiles fill the SMs; T = 32 for the few tiles of a small
+// trailing block, which otherwise run as a dependent chain of launches on a
+// handful of SMs.  Same sums in the same order.
+template <class C, int T>
 __global__ void __launch_bounds__(CTA_THREADS) k_dense_herk(C* A, int64_t N, int64_t ld, int k0) {
-  __shared__ C Pi[CNB][17];
-  __shared__ C Pj[CNB][17];
+  constexpr int Q = T / 16;
+  __shared__ C Pi[T][17];
+  __shared__ C Pj[T][17];
   using O = Ops<C>;
   const int kb = (int)(N - k0 < CNB ? N - k0 : CNB);
   const int64_t k1 = k0 + kb;
@@ -178,33 +186,33 @@ __global__ void __launch_bounds__(CTA_THREADS) k_dense_herk(C* A, int64_t N, int
   while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
   while (bi * (bi + 1) / 2 > t) --bi;
   const int64_t bj = t - bi * (bi + 1) / 2;
-  const int64_t i0 = k1 + bi * CNB, j0 = k1 + bj * CNB;
+  const int64_t i0 = k1 + bi * T, j0 = k1 + bj * T;
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  C acc[4][4];
-  for (int a = 0; a < 4; ++a)
-    for (int b = 0; b < 4; ++b) acc[a][b] = O::zero();
+  C acc[Q][Q];
+  for (int a = 0; a < Q; ++a)
+    for (int b = 0; b < Q; ++b) acc[a][b] = O::zero();
   for (int t0 = 0; t0 < kb; t0 += 16) {
-    for (int q = threadIdx.x; q < CNB * 16; q += blockDim.x) {
+    for (int q = threadIdx.x; q < T * 16; q += blockDim.x) {
       int r = q / 16, c = q % 16;
       int64_t ii = i0 + r, jj = j0 + r;
       Pi[r][c] = (ii < N && t0 + c < kb) ? A[ii * ld + k0 + t0 + c] : O::zero();
       Pj[r][c] = (jj < N && t0 + c < kb) ? A[jj * ld + k0 + t0 + c] : O::zero();
     }
     __syncthreads();
-    // thread (tx, ty) owns rows ty*4 + a and columns tx + 16 b: the 16 lanes of
+    // thread (tx, ty) owns rows ty*Q + a and columns tx + 16 b: the 16 lanes of
     // a half-warp read 16 consecutive rows of Pj (row stride 17: distinct banks)
     for (int c = 0; c < 16; ++c) {
-      C av[4], bv[4];
-      for (int a = 0; a < 4; ++a) av[a] = Pi[ty * 4 + a][c];
-      for (int b = 0; b < 4; ++b) bv[b] = Pj[tx + 16 * b][c];
-      for (int a = 0; a < 4; ++a)
-        for (int b = 0; b < 4; ++b) acc[a][b] = O::fmac(av[a], bv[b], acc[a][b]);
+      C av[Q], bv[Q];
+      for (int a = 0; a < Q; ++a) av[a] = Pi[ty * Q + a][c];
+      for (int b = 0; b < Q; ++b) bv[b] = Pj[tx + 16 * b][c];
+      for (int a = 0; a < Q; ++a)
+        for (int b = 0; b < Q; ++b) acc[a][b] = O::fmac(av[a], bv[b], acc[a][b]);
     }
     __syncthreads();
   }
-  for (int a = 0; a < 4; ++a)
-    for (int b = 0; b < 4; ++b) {
-      int64_t i = i0 + ty * 4 + a, j = j0 + tx + 16 * b;
+  for (int a = 0; a < Q; ++a)
+    for (int b = 0; b < Q; ++b) {
+      int64_t i = i0 + ty * Q + a, j = j0 + tx + 16 * b;
       if (i < N && j <= i) {
         C& o = A[i * ld + j];
         o = O::sub(o, acc[a][b]);
@@ -219,24 +227,33 @@ template <class C>
 static void dense_cholesky(C* A, int64_t n, int64_t ld, C* Dinv, int* info, cudaStream_t st) {
   const size_t sm = (size_t)2 * CNB * (CNB + 1) * sizeof(C);
   DPG_CUDA(cudaFuncSetAttribute(k_dense_diag<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  DPG_CUDA(cudaFuncSetAttribute(k_dense_panel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  DPG_CUDA(cudaFuncSetAttribute(k_dense_panel<C, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  DPG_CUDA(cudaFuncSetAttribute(k_dense_panel<C, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   for (int64_t k0 = 0; k0 < n; k0 += CNB) {
     int kb = (int)std::min<int64_t>(CNB, n - k0);
     k_dense_diag<C><<<1, CTA_THREADS, sm, st>>>(A, n, ld, (int)k0, Dinv, info);
     DPG_CHECK_LAUNCH();
     int64_t rows = n - k0 - kb;
     if (rows <= 0) break;
-    k_dense_panel<C><<<(unsigned)((rows + CNB - 1) / CNB), CTA_THREADS, sm, st>>>(A, n, ld, (int)k0, Dinv);
+    if (rows <= (int64_t)16 * SMALL_TILES)
+      k_dense_panel<C, 1><<<(unsigned)((rows + 15) / 16), CTA_THREADS, sm, st>>>(A, n, ld, (int)k0, Dinv);
+    else
+      k_dense_panel<C, 4><<<(unsigned)((rows + CNB - 1) / CNB), CTA_THREADS, sm, st>>>(A, n, ld, (int)k0, Dinv);
     DPG_CHECK_LAUNCH();
     int64_t nt = (rows + CNB - 1) / CNB;
-    k_dense_herk<C><<<(unsigned)(nt * (nt + 1) / 2), CTA_THREADS, 0, st>>>(A, n, ld, (int)k0);
+    if (nt * (nt + 1) / 2 <= SMALL_TILES) {
+      nt = (rows + 31) / 32;
+      k_dense_herk<C, 32><<<(unsigned)(nt * (nt + 1) / 2), CTA_THREADS, 0, st>>>(A, n, ld, (int)k0);
+    } else {
+      k_dense_herk<C, 64><<<(unsigned)(nt * (nt + 1) / 2), CTA_THREADS, 0, st>>>(A, n, ld, (int)k0);
+    }
     DPG_CHECK_LAUNCH();
   }
 }
 
 // ---------------------------------------------------------- L^-1 (blocked)
-// X[kb rows, tile cols] <- Dinv_kb * X[kb rows, tile cols], one CTA per 64-column tile
-template <class C>
+// X[kb rows, tile cols] <- Dinv_kb * X[kb rows, tile cols], one CTA per W-column tile
+template <class C, int W>
 __global__ void __launch_bounds__(CTA_THREADS) k_trinv_scale(C* X, const C* Dinv, int64_t N, int64_t ld, int kb) {
   extern __shared__ unsigned char shraw[];
   C* D = reinterpret_cast<C*>(shraw);
@@ -244,60 +261,61 @@ __global__ void __launch_bounds__(CTA_THREADS) k_trinv_scale(C* X, const C* Dinv
   using O = Ops<C>;
   const int64_t k0 = (int64_t)kb * CNB;
   const int kw = (int)(N - k0 < CNB ? N - k0 : CNB);
-  const int64_t c0 = (int64_t)blockIdx.x * CNB;
-  const int cw = (int)(N - c0 < CNB ? N - c0 : CNB);
+  const int64_t c0 = (int64_t)blockIdx.x * W;
+  const int cw = (int)(N - c0 < W ? N - c0 : W);
   const C* Dk = Dinv + (size_t)kb * CNB * CNB;
-  for (int q = threadIdx.x; q < CNB * CNB; q += blockDim.x) {
-    D[q] = Dk[q];
-    int r = q / CNB, c = q % CNB;
+  for (int q = threadIdx.x; q < CNB * CNB; q += blockDim.x) D[q] = Dk[q];
+  for (int q = threadIdx.x; q < CNB * W; q += blockDim.x) {
+    int r = q / W, c = q % W;
     T[q] = (r < kw && c < cw) ? X[(k0 + r) * ld + c0 + c] : O::zero();
   }
   __syncthreads();
-  for (int q = threadIdx.x; q < CNB * CNB; q += blockDim.x) {
-    int r = q / CNB, c = q % CNB;
+  for (int q = threadIdx.x; q < CNB * W; q += blockDim.x) {
+    int r = q / W, c = q % W;
     if (r >= kw || c >= cw) continue;
     C acc = O::zero();
-    for (int t = 0; t <= r; ++t) acc = O::fma(D[r * CNB + t], T[t * CNB + c], acc);
+    for (int t = 0; t <= r; ++t) acc = O::fma(D[r * CNB + t], T[t * W + c], acc);
     X[(k0 + r) * ld + c0 + c] = acc;
   }
 }
 
-// X[ib, jb] -= L[ib, kb] X[kb, jb] for ib > kb, jb <= kb (64x64 tiles)
-template <class C>
+// X[ib, jb] -= L[ib, kb] X[kb, jb] for ib > kb, jb <= kb (T x T tiles of those
+// blocks; T as k_dense_herk)
+template <class C, int T>
 __global__ void __launch_bounds__(CTA_THREADS) k_trinv_update(C* X, const C* L, int64_t N, int64_t ld, int kb) {
-  __shared__ C La[CNB][17];
-  __shared__ C Xb[16][CNB + 1];
+  constexpr int Q = T / 16;
+  __shared__ C La[T][17];
+  __shared__ C Xb[16][T + 1];
   using O = Ops<C>;
   const int64_t k0 = (int64_t)kb * CNB;
   const int kw = (int)(N - k0 < CNB ? N - k0 : CNB);
-  const int ncol = kb + 1;
-  const int64_t ib = kb + 1 + blockIdx.x / ncol;
-  const int64_t jb = blockIdx.x % ncol;
-  const int64_t i0 = ib * CNB, j0 = jb * CNB;
+  const int ncol = (kb + 1) * (CNB / T);
+  const int64_t i0 = (int64_t)(kb + 1) * CNB + (int64_t)(blockIdx.x / ncol) * T;
+  const int64_t j0 = (int64_t)(blockIdx.x % ncol) * T;
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  C acc[4][4];
-  for (int a = 0; a < 4; ++a)
-    for (int b = 0; b < 4; ++b) acc[a][b] = O::zero();
+  C acc[Q][Q];
+  for (int a = 0; a < Q; ++a)
+    for (int b = 0; b < Q; ++b) acc[a][b] = O::zero();
   for (int t0 = 0; t0 < kw; t0 += 16) {
-    for (int q = threadIdx.x; q < CNB * 16; q += blockDim.x) {
+    for (int q = threadIdx.x; q < T * 16; q += blockDim.x) {
       int r = q / 16, c = q % 16;
       La[r][c] = (i0 + r < N && t0 + c < kw) ? L[(i0 + r) * ld + k0 + t0 + c] : O::zero();
-      int t = q / CNB, cc = q % CNB;
+      int t = q / T, cc = q % T;
       Xb[t][cc] = (t0 + t < kw && j0 + cc < N) ? X[(k0 + t0 + t) * ld + j0 + cc] : O::zero();
     }
     __syncthreads();
     for (int c = 0; c < 16; ++c) {
-      C av[4], bv[4];
-      for (int a = 0; a < 4; ++a) av[a] = La[ty * 4 + a][c];
-      for (int b = 0; b < 4; ++b) bv[b] = Xb[c][tx + 16 * b];   // consecutive columns: distinct banks
-      for (int a = 0; a < 4; ++a)
-        for (int b = 0; b < 4; ++b) acc[a][b] = O::fma(av[a], bv[b], acc[a][b]);
+      C av[Q], bv[Q];
+      for (int a = 0; a < Q; ++a) av[a] = La[ty * Q + a][c];
+      for (int b = 0; b < Q; ++b) bv[b] = Xb[c][tx + 16 * b];   // consecutive columns: distinct banks
+      for (int a = 0; a < Q; ++a)
+        for (int b = 0; b < Q; ++b) acc[a][b] = O::fma(av[a], bv[b], acc[a][b]);
     }
     __syncthreads();
   }
-  for (int a = 0; a < 4; ++a)
-    for (int b = 0; b < 4; ++b) {
-      int64_t i = i0 + ty * 4 + a, j = j0 + tx + 16 * b;
+  for (int a = 0; a < Q; ++a)
+    for (int b = 0; b < Q; ++b) {
+      int64_t i = i0 + ty * Q + a, j = j0 + tx + 16 * b;
       if (i < N && j < N) {
         C& o = X[i * ld + j];
         o = O::sub(o, acc[a][b]);
@@ -332,13 +350,18 @@ static void dense_trinv(const C* L, C* X, int64_t n, int64_t ld, const C* Dinv, 
   k_identity_lower<C><<<(unsigned)std::min<int64_t>(1216, (n * n + 255) / 256), 256, 0, st>>>(X, n, ld);
   DPG_CHECK_LAUNCH();
   const size_t sms = (size_t)2 * CNB * CNB * sizeof(C);
-  DPG_CUDA(cudaFuncSetAttribute(k_trinv_scale<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sms));
+  DPG_CUDA(cudaFuncSetAttribute(k_trinv_scale<C, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sms));
+  DPG_CUDA(cudaFuncSetAttribute(k_trinv_scale<C, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sms));
   for (int kb = 0; kb < nb; ++kb) {
-    k_trinv_scale<C><<<kb + 1, CTA_THREADS, sms, st>>>(X, Dinv, n, ld, kb);
+    if (kb + 1 <= SMALL_TILES / 4) k_trinv_scale<C, 16><<<4 * (kb + 1), CTA_THREADS, sms, st>>>(X, Dinv, n, ld, kb);
+    else k_trinv_scale<C, 64><<<kb + 1, CTA_THREADS, sms, st>>>(X, Dinv, n, ld, kb);
     DPG_CHECK_LAUNCH();
     const int rows = nb - kb - 1;
     if (rows > 0) {
-      k_trinv_update<C><<<(unsigned)(rows * (kb + 1)), CTA_THREADS, 0, st>>>(X, L, n, ld, kb);
+      if (rows * (kb + 1) <= SMALL_TILES)
+        k_trinv_update<C, 32><<<(unsigned)(4 * rows * (kb + 1)), CTA_THREADS, 0, st>>>(X, L, n, ld, kb);
+      else
+        k_trinv_update<C, 64><<<(unsigned)(rows * (kb + 1)), CTA_THREADS, 0, st>>>(X, L, n, ld, kb);
       DPG_CHECK_LAUNCH();
     }
   }
@@ -355,6 +378,24 @@ enum { TC_A_NH = 0, TC_A_NN = 1, TC_B = 2, TC_B_TRANS = 3 };
 // Panel width of the tensor-core factorisation (a multiple of 64 and of 16).
 static int64_t tc_panel(int64_t N) { return N >= 4096 ? 512 : (N >= 1024 ? 256 : 128); }
 
+// Stream of the diagonal-block factorisations that run ahead of a coarsest
+// factorisation's stream (one per device and stream, kept for the life of the
+// process like the side streams of the setup).
+static cudaStream_t lookahead_stream_for(cudaStream_t st) {
+  static std::mutex mu;
+  static std::map<std::pair<int, cudaStream_t>, cudaStream_t> streams;
+  int dev = 0;
+  DPG_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lk(mu);
+  cudaStream_t& s = streams[{dev, st}];
+  if (!s) {
+    int least = 0, greatest = 0;
+    DPG_CUDA(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+    DPG_CUDA(cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, greatest));
+  }
+  return s;
+}
+
 // Mixed path: A = L L^H and X = L^-1 (complex64, N x N, row-major, lower
 // halves) by panels of width W, right-looking.  Per panel K (rows and
 // columns K0 .. K0 + W - 1), with the rows below it "2":
@@ -364,7 +405,13 @@ static int64_t tc_panel(int64_t N) { return N >= 4096 ? 512 : (N >= 1024 ? 256 :
 //   A_22 -= L_2K L_2K^H          tensor cores, lower tiles only
 //   T_2,<=K += L_2K X_K,<=K      tensor cores
 // which gives X_IJ = -L_II^-1 sum_{J<=K<I} L_IK X_KJ for every block below
-// the diagonal.  fault (tests): the first product issues no MMA.
+// the diagonal.  The diagonal factorisation is a chain of small dependent
+// launches (1.2 ms a panel of 512, most SMs idle; 24 of 71 ms on N = 9,777
+// when it ran between the products), so it runs one panel ahead on its own
+// stream: the update of A_22 starts with the next panel's diagonal block, and
+// the factorisation of that block overlaps the rest of the panel's products.
+// Every entry gets the same operations in the same order.
+// fault (tests): the first product issues no MMA.
 static void tc_cholesky_inverse(Alloc& Al, float2* A, float2* X, int64_t N, float2* Dinv, int* info, int fault,
                                 cudaStream_t st) {
   tc_configure();
@@ -372,38 +419,71 @@ static void tc_cholesky_inverse(Alloc& Al, float2* A, float2* X, int64_t N, floa
   void* Aimg = Al.get(tc_image_bytes(N, W, true));
   void* Bimg = Al.get(tc_image_bytes(N, W, false));
   DPG_CUDA(cudaMemsetAsync(X, 0, (size_t)N * N * sizeof(float2), st));
+  const cudaStream_t sf = lookahead_stream_for(st);
+  struct Events {   // destroyed on every exit path, after sf's work has been joined into st
+    cudaEvent_t ready = nullptr, done = nullptr;
+    cudaStream_t sf, st;
+    Events(cudaStream_t f, cudaStream_t s) : sf(f), st(s) {
+      DPG_CUDA(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
+      DPG_CUDA(cudaEventCreateWithFlags(&done, cudaEventDisableTiming));
+    }
+    ~Events() {
+      if (done && cudaEventRecord(done, sf) == cudaSuccess) cudaStreamWaitEvent(st, done, 0);
+      if (ready) cudaEventDestroy(ready);
+      if (done) cudaEventDestroy(done);
+    }
+  } ev(sf, st);
+  // L_KK and L_KK^-1 of the panel at K0, after everything recorded on st so far
+  auto factor = [&](int64_t K0) {
+    const int64_t kb = std::min<int64_t>(W, N - K0);
+    float2* Dk = Dinv + (K0 / CNB) * CNB * CNB;
+    DPG_CUDA(cudaEventRecord(ev.ready, st));
+    DPG_CUDA(cudaStreamWaitEvent(sf, ev.ready, 0));
+    dense_cholesky<float2>(A + K0 * N + K0, kb, N, Dk, info, sf);
+    dense_trinv<float2>(A + K0 * N + K0, X + K0 * N + K0, kb, N, Dk, sf);
+    DPG_CUDA(cudaEventRecord(ev.done, sf));
+  };
   int first = fault;
-  auto gemm = [&](int64_t M, int64_t Nc, int64_t kc, float2* C, float alpha, float beta, int lower) {
-    tc_gemm(Aimg, Bimg, M, Nc, kc, C, N, alpha, beta, lower, info, first, st);
+  auto gemm = [&](const void* Ai, const void* Bi, int64_t M, int64_t Nc, int64_t kc, float2* C, float alpha,
+                  float beta, int lower) {
+    tc_gemm(Ai, Bi, M, Nc, kc, C, N, alpha, beta, lower, info, first, st);
     first = 0;
   };
+  factor(0);
   for (int64_t K0 = 0; K0 < N; K0 += W) {
     const int64_t kb = std::min<int64_t>(W, N - K0);
-    float2* Akk = A + K0 * N + K0;
     float2* Xkk = X + K0 * N + K0;
-    float2* Dk = Dinv + (K0 / CNB) * CNB * CNB;
-    dense_cholesky<float2>(Akk, kb, N, Dk, info, st);
-    dense_trinv<float2>(Akk, Xkk, kb, N, Dk, st);
+    DPG_CUDA(cudaStreamWaitEvent(st, ev.done, 0));   // L_KK and L_KK^-1
     if (K0 > 0) {   // X_K,<K = -L_KK^-1 T_K,<K (T read into the image before it is overwritten)
       tc_pack(Aimg, Xkk, N, kb, kb, TC_A_NN, st);
       tc_pack(Bimg, X + K0 * N, N, K0, kb, TC_B_TRANS, st);
-      gemm(kb, K0, kb, X + K0 * N, -1.f, 0.f, 0);
+      gemm(Aimg, Bimg, kb, K0, kb, X + K0 * N, -1.f, 0.f, 0);
     }
     const int64_t rows = N - K0 - kb;
     if (rows <= 0) break;
     float2* A2 = A + (K0 + kb) * N + K0;   // rows below the panel, panel columns
+    float2* A22 = A + (K0 + kb) * N + K0 + kb;
     // L_2K = A_2K L_KK^-H
     tc_pack(Aimg, A2, N, rows, kb, TC_A_NH, st);
     tc_pack(Bimg, Xkk, N, kb, kb, TC_B, st);
-    gemm(rows, kb, kb, A2, 1.f, 0.f, 0);
-    // A_22 -= L_2K L_2K^H
+    gemm(Aimg, Bimg, rows, kb, kb, A2, 1.f, 0.f, 0);
+    // A_22 -= L_2K L_2K^H: the next panel's diagonal block, which its factorisation waits for,
+    // then the rows below it (images advance by whole tiles: W is a multiple of 128)
     tc_pack(Aimg, A2, N, rows, kb, TC_A_NH, st);
     tc_pack(Bimg, A2, N, rows, kb, TC_B, st);
-    gemm(rows, rows, kb, A + (K0 + kb) * N + K0 + kb, -1.f, 1.f, 1);
+    const int64_t nw = std::min<int64_t>(W, rows), rest = rows - nw;
+    gemm(Aimg, Bimg, nw, nw, kb, A22, -1.f, 1.f, 1);
+    factor(K0 + kb);
+    if (rest > 0) {
+      const void* Ar = reinterpret_cast<const char*>(Aimg) + tc_image_bytes(nw, kb, true);
+      const void* Br = reinterpret_cast<const char*>(Bimg) + tc_image_bytes(nw, kb, false);
+      gemm(Ar, Bimg, rest, nw, kb, A22 + nw * N, -1.f, 1.f, 0);
+      gemm(Ar, Br, rest, rest, kb, A22 + nw * N + nw, -1.f, 1.f, 1);
+    }
     // T_2,<=K += L_2K X_K,<=K
     tc_pack(Aimg, A2, N, rows, kb, TC_A_NN, st);
     tc_pack(Bimg, X + K0 * N, N, K0 + kb, kb, TC_B_TRANS, st);
-    gemm(rows, K0 + kb, kb, X + (K0 + kb) * N, 1.f, 1.f, 0);
+    gemm(Aimg, Bimg, rows, K0 + kb, kb, X + (K0 + kb) * N, 1.f, 1.f, 0);
   }
   Al.release(Bimg);
   Al.release(Aimg);

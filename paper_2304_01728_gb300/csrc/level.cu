@@ -1108,11 +1108,11 @@ static cudaStream_t side_stream_for(cudaStream_t st) {
   std::lock_guard<std::mutex> lk(mu);
   cudaStream_t& s = streams[{dev, st}];
   if (!s) {
-    // highest priority: the factorisation is a chain of small dependent
-    // launches, the patch work it overlaps is many independent CTAs
+    // above the patch work it overlaps (many independent CTAs), below the
+    // diagonal blocks that run ahead of it (lookahead_stream_for, coarse.cu)
     int least = 0, greatest = 0;
     DPG_CUDA(cudaDeviceGetStreamPriorityRange(&least, &greatest));
-    DPG_CUDA(cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, greatest));
+    DPG_CUDA(cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, std::min(greatest + 1, least)));
   }
   return s;
 }
