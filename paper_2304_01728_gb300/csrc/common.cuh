@@ -136,6 +136,196 @@ struct Team {
   }
 };
 
+// ------------------------------------------------- 32 x 32 x 32 tile products
+// acc[q] += sum_t A[r][t] B[t][c] for the thread's outputs r = w + 8 q, c = lane
+// (warp w of 8, q < 4), the inner step of every blocked routine below.  The
+// operands come in registers: a[i] = A[4 w + i][lane], and b[i] = B[4 w + i][lane];
+// with BT, b[i] = B[lane][4 w + i] (rows of the transpose).  At, Bt: TL x NB
+// elements of shared memory each.  All 256 threads call it; it synchronises
+// before it writes shared memory and before it reads it.
+//
+// FP32 types: FMA chains in increasing t, continued from acc.
+//
+// FP64 types: this GPU's FP64 pipe runs 1.7 FMAs per clock and SM, its integer
+// pipe 59 32 x 32 -> 64-bit multiply-adds.  A row of A and a column of B are
+// taken as fixed-point numbers with the exponent of their largest entry, 57
+// bits each in two 28-bit limbs, and multiplied exactly on the integer pipe:
+// hi hi, and hi lo + lo hi in a second 64-bit sum (lo lo is below 2^-58 of the
+// largest product and dropped), three multiply-adds per product.  |hi| <= 2^28
+// and |lo| <= 2^27, so 64 products (32 complex ones) stay below 2^62.  The sum
+// is rounded once per chunk.  Element matrices of random (p, h, omega, c), p = 1
+// to 4, carry the same error against 128-bit arithmetic as with FP64 FMA chains
+// (geometric means of the two within 7%, either way; unchanged with 60-bit
+// operands, so what is left comes from the FP64 panels).  Tiles with an
+// infinity, a NaN or an exponent at the top of the range take the FP64 chain.
+// Measured (GB300): element stage of 800 elements of order 3 with distinct
+// wavespeeds 88 -> 45 ms, 64 of order 5 1,107 -> 174 ms; complex128 setup on
+// 8^3 p = 3 78 -> 50 ms.
+__device__ __forceinline__ int fx_exponent(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+__device__ __forceinline__ int fx_exponent(double2 v) { return max(fx_exponent(v.x), fx_exponent(v.y)); }
+
+// round(v 2^(1078 - E)) for a biased exponent E >= v's: |v| < 2^(E - 1022) maps below 2^56 (zero and
+// denormals to 0); hi, lo: limbs with v = hi 2^28 + lo
+__device__ __forceinline__ void fx_limbs(double v, int E, int& hi, int& lo) {
+  const int e = fx_exponent(v);
+  const int sh = E - e - 3;   // shift right (left when negative) of the 53-bit mantissa
+  const long long m = ((long long)((__double2hiint(v) & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
+  long long f = 0;
+  if (e != 0 && sh < 60) f = sh <= 0 ? m << -sh : (m + (1ll << (sh - 1))) >> sh;
+  if (__double2hiint(v) < 0) f = -f;
+  hi = (int)((f + (1ll << 27)) >> 28);
+  lo = (int)(f - ((long long)hi << 28));
+}
+
+// 2^k t, rounded once
+__device__ __forceinline__ double fx_value(long long hh, long long x, int k) {
+  const double t = (double)(hh + ((x + (1ll << 27)) >> 28));
+  if (k >= -1000 && k <= 960) return t * __hiloint2double((k + 1023) << 20, 0);
+  return ldexp(t, k);
+}
+
+__device__ __forceinline__ void fx_store(double* p, double v, int E) {
+  int2 f;
+  fx_limbs(v, E, f.x, f.y);
+  *reinterpret_cast<int2*>(p) = f;
+}
+__device__ __forceinline__ void fx_store(double2* p, double2 v, int E) {
+  int4 f;
+  fx_limbs(v.x, E, f.x, f.y);
+  fx_limbs(v.y, E, f.z, f.w);
+  *reinterpret_cast<int4*>(p) = f;
+}
+
+// column c of row t of Bt: swizzled with BT, so that stores along t do not conflict
+template <bool BT>
+__device__ __forceinline__ int fx_col(int t, int c) { return t * TL + (BT ? c ^ t : c); }
+
+// column t of row r of At: swizzled by even numbers with AT (pairs of t stay together)
+template <bool AT>
+__device__ __forceinline__ int fx_row(int r, int t) { return r * NB + (AT ? t ^ (r & ~1) : t); }
+
+template <class T> struct IsFp64 { static constexpr bool v = false; };
+template <> struct IsFp64<double> { static constexpr bool v = true; };
+template <> struct IsFp64<double2> { static constexpr bool v = true; };
+
+template <class T, bool BT, bool AT = false>
+__device__ void tile_product(const T a[4], const T b[4], T* At, T* Bt, int kb, T acc[4]) {
+  using O = Ops<T>;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  // place of a[i] and b[i]
+  auto pa = [&](int i) { return AT ? fx_row<AT>(lane, 4 * w + i) : fx_row<AT>(4 * w + i, lane); };
+  auto pb = [&](int i) { return BT ? fx_col<BT>(lane, 4 * w + i) : fx_col<BT>(4 * w + i, lane); };
+  auto plain = [&]() {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      At[pa(i)] = a[i];
+      Bt[pb(i)] = b[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      T s = acc[q];
+#pragma unroll 8
+      for (int t = 0; t < kb; ++t) s = O::fma(At[fx_row<AT>(w + 8 * q, t)], Bt[fx_col<BT>(t, lane)], s);
+      acc[q] = s;
+    }
+  };
+  if constexpr (!IsFp64<T>::v) {
+    __syncthreads();   // the last product's readers are done
+    plain();
+  } else {
+    __shared__ int s_ea[TL], s_eb[TL], s_pa[8][TL], s_pb[8][TL];
+    int ea[4], eb[4], ma = 0, mb = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      ea[i] = fx_exponent(a[i]);
+      eb[i] = fx_exponent(b[i]);
+      if (!AT) ea[i] = __reduce_max_sync(0xffffffffu, ea[i]);   // over the row's t
+      if (BT) eb[i] = __reduce_max_sync(0xffffffffu, eb[i]);
+      ma = max(ma, ea[i]);
+      mb = max(mb, eb[i]);
+    }
+    if (__syncthreads_or(max(ma, mb) >= 0x7fe)) {   // uniform over the CTA; also: the last product's readers are done
+      plain();
+      return;
+    }
+    if (AT || !BT) {   // exponents of the rows or columns that run across the warps
+      if (AT) s_pa[w][lane] = ma;
+      if (!BT) s_pb[w][lane] = mb;
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (AT) ma = max(ma, s_pa[u][lane]);
+        if (!BT) mb = max(mb, s_pb[u][lane]);
+      }
+      if (AT && w == 0) s_ea[lane] = ma;
+      if (!BT && w == 0) s_eb[lane] = mb;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      fx_store(&At[pa(i)], a[i], AT ? ma : ea[i]);
+      fx_store(&Bt[pb(i)], b[i], BT ? eb[i] : mb);
+      if (lane == 0) {
+        if (!AT) s_ea[4 * w + i] = ea[i];
+        if (BT) s_eb[4 * w + i] = eb[i];
+      }
+    }
+    __syncthreads();
+    const int ec = s_eb[lane];
+    if constexpr (sizeof(T) == sizeof(double)) {
+      const int2* Af = reinterpret_cast<const int2*>(At);
+      const int2* Bf = reinterpret_cast<const int2*>(Bt);
+      long long hh[4] = {0, 0, 0, 0}, x[4] = {0, 0, 0, 0};
+#pragma unroll 4
+      for (int t = 0; t < NB; t += 2) {
+        const int2 b0 = Bf[fx_col<BT>(t, lane)], b1 = Bf[fx_col<BT>(t + 1, lane)];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int4 u = *reinterpret_cast<const int4*>(&Af[fx_row<AT>(w + 8 * q, t)]);
+          hh[q] += (long long)u.x * b0.x;
+          x[q] += (long long)u.x * b0.y;
+          x[q] += (long long)u.y * b0.x;
+          hh[q] += (long long)u.z * b1.x;
+          x[q] += (long long)u.z * b1.y;
+          x[q] += (long long)u.w * b1.x;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[q] += fx_value(hh[q], x[q], s_ea[w + 8 * q] + ec - 2100);
+    } else {
+      const int4* Af = reinterpret_cast<const int4*>(At);
+      const int4* Bf = reinterpret_cast<const int4*>(Bt);
+      long long rh[4] = {0, 0, 0, 0}, rx[4] = {0, 0, 0, 0}, ih[4] = {0, 0, 0, 0}, ix[4] = {0, 0, 0, 0};
+#pragma unroll 2
+      for (int t = 0; t < NB; ++t) {
+        const int4 v = Bf[fx_col<BT>(t, lane)];   // (re hi, re lo, im hi, im lo)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int4 u = Af[fx_row<AT>(w + 8 * q, t)];
+          rh[q] += (long long)u.x * v.x;
+          rh[q] -= (long long)u.z * v.z;
+          rx[q] += (long long)u.x * v.y;
+          rx[q] += (long long)u.y * v.x;
+          rx[q] -= (long long)u.z * v.w;
+          rx[q] -= (long long)u.w * v.z;
+          ih[q] += (long long)u.x * v.z;
+          ih[q] += (long long)u.z * v.x;
+          ix[q] += (long long)u.x * v.w;
+          ix[q] += (long long)u.y * v.z;
+          ix[q] += (long long)u.z * v.y;
+          ix[q] += (long long)u.w * v.x;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int k = s_ea[w + 8 * q] + ec - 2100;
+        acc[q].x += fx_value(rh[q], rx[q], k);
+        acc[q].y += fx_value(ih[q], ix[q], k);
+      }
+    }
+  }
+}
+
 // In-place lower Cholesky A = L L^H of an n x n Hermitian matrix (row-major,
 // leading dimension lda).  The strict upper triangle is not referenced and
 // is left unchanged.  Returns 0 or k+1 if the k-th pivot is not positive.
@@ -149,7 +339,7 @@ __device__ int cta_potrf(T* A, int n, int lda, T* smem, Team<CL> tm = Team<CL>()
   T* Pj = Pi + TL * NB;
   __shared__ int info;
   __shared__ R rdiag[NB];   // 1 / L[j][j] of the current diagonal block
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   if (tid == 0) info = 0;
   __syncthreads();
   for (int k0 = 0; k0 < n; k0 += NB) {
@@ -209,26 +399,26 @@ __device__ int cta_potrf(T* A, int n, int lda, T* smem, Team<CL> tm = Team<CL>()
       for (int bj = 0; bj <= bi; ++bj) {
         const int i0 = k1 + bi * TL, j0 = k1 + bj * TL;
         if (!tm.own2(i0 / TL, j0 / TL)) continue;
-        for (int e = tid; e < TL * NB; e += blockDim.x) {
-          int r = e / NB, t = e % NB;
-          Pi[e] = (i0 + r < n && t < kb) ? tm.ld(&A[(size_t)(i0 + r) * lda + k0 + t]) : O::zero();
-          Pj[e] = (j0 + r < n && t < kb) ? tm.ld(&A[(size_t)(j0 + r) * lda + k0 + t]) : O::zero();
+        T a[4], b[4], acc[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int r = 4 * w + u;
+          a[u] = (i0 + r < n && lane < kb) ? tm.ld(&A[(size_t)(i0 + r) * lda + k0 + lane]) : O::zero();
+          b[u] = (j0 + r < n && lane < kb) ? O::conj(tm.ld(&A[(size_t)(j0 + r) * lda + k0 + lane])) : O::zero();
+          acc[u] = O::zero();
         }
-        __syncthreads();
-        for (int e = tid; e < TL * TL; e += blockDim.x) {
-          int r = e / TL, c = e % TL;
-          int i = i0 + r, j = j0 + c;
+        tile_product<T, true>(a, b, Pi, Pj, kb, acc);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int i = i0 + w + 8 * q, j = j0 + lane;
           if (i < n && j <= i) {
-            T acc = O::zero();
-            for (int t = 0; t < kb; ++t) acc = O::fmac(Pi[r * NB + t], Pj[c * NB + t], acc);
             size_t o = (size_t)i * lda + j;
-            A[o] = O::sub(tm.ld(&A[o]), acc);
+            A[o] = O::sub(tm.ld(&A[o]), acc[q]);
           }
         }
-        __syncthreads();
       }
     }
-    if constexpr (CL) tm.sync();
+    tm.sync();   // the next block reads what every thread (and CTA) updated
   }
   __syncthreads();
   return info;
@@ -240,22 +430,27 @@ __device__ __forceinline__ double2 lmul(double l, double2 b) { return make_doubl
 __device__ __forceinline__ double2 lmul(double2 l, double2 b) { return Ops<double2>::mul(l, b); }
 __device__ __forceinline__ float2 lmul(float l, float2 b) { return make_float2(l * b.x, l * b.y); }
 __device__ __forceinline__ float2 lmul(float2 l, float2 b) { return Ops<float2>::mul(l, b); }
+// a factor entry in the right-hand sides' type
+template <class TB, class TLt> __device__ __forceinline__ TB as_type(TLt l) {
+  if constexpr (sizeof(TB) == sizeof(TLt)) return l;
+  else return Ops<TB>::mk(l, 0);
+}
 __device__ __forceinline__ double lmul(double l, double b) { return l * b; }
 __device__ __forceinline__ float lmul(float l, float b) { return l * b; }
 
 // Solve L X = B in place (L lower triangular n x n of type TLt, B n x nrhs
 // of type TB; TLt may be the real type of TB).  smem (bytes): room for
-// NB*NB + TL*NB elements of TLt followed by NB*TL elements of TB.
+// NB*NB elements of TLt followed by 2*NB*TL elements of TB.
 template <class TLt, class TB>
 __device__ void cta_trsm_lower(const TLt* L, int n, int ldl, TB* B, int nrhs, int ldb, char* smem) {
   using OL = Ops<TLt>;
   using OB = Ops<TB>;
   using RB = typename OB::R;
   TLt* D = reinterpret_cast<TLt*>(smem);
-  TLt* Lt = D + NB * NB;
-  TB* Xt = reinterpret_cast<TB*>(Lt + TL * NB);
+  TB* Lt = reinterpret_cast<TB*>(D + NB * NB);
+  TB* Xt = Lt + TL * NB;
   __shared__ RB rdiag[NB];
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   for (int k0 = 0; k0 < n; k0 += NB) {
     const int kb = min(NB, n - k0);
     for (int e = tid; e < kb * kb; e += blockDim.x) {
@@ -278,29 +473,32 @@ __device__ void cta_trsm_lower(const TLt* L, int n, int ldl, TB* B, int nrhs, in
     // update rows below: B[i][c] -= sum_t L[i][k0+t] X[k0+t][c]
     const int k1 = k0 + kb;
     for (int i0 = k1; i0 < n; i0 += TL) {
-      for (int e = tid; e < TL * NB; e += blockDim.x) {
-        int r = e / NB, t = e % NB;
-        Lt[e] = (i0 + r < n && t < kb) ? L[(size_t)(i0 + r) * ldl + k0 + t] : OL::zero();
+      TB a[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = i0 + 4 * w + u;
+        a[u] = (r < n && lane < kb) ? as_type<TB>(L[(size_t)r * ldl + k0 + lane]) : OB::zero();
       }
       for (int c0 = 0; c0 < nrhs; c0 += TL) {
-        for (int e = tid; e < NB * TL; e += blockDim.x) {
-          int t = e / TL, c = e % TL;
-          Xt[e] = (t < kb && c0 + c < nrhs) ? B[(size_t)(k0 + t) * ldb + c0 + c] : OB::zero();
+        TB b[4], acc[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int t = 4 * w + u;
+          b[u] = (t < kb && c0 + lane < nrhs) ? B[(size_t)(k0 + t) * ldb + c0 + lane] : OB::zero();
+          acc[u] = OB::zero();
         }
-        __syncthreads();
-        for (int e = tid; e < TL * TL; e += blockDim.x) {
-          int r = e / TL, c = e % TL;
-          int i = i0 + r, cc = c0 + c;
+        tile_product<TB, false>(a, b, Lt, Xt, kb, acc);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int i = i0 + w + 8 * q, cc = c0 + lane;
           if (i < n && cc < nrhs) {
-            TB acc = OB::zero();
-            for (int t = 0; t < kb; ++t) acc = OB::add(acc, lmul(Lt[r * NB + t], Xt[t * TL + c]));
             size_t o = (size_t)i * ldb + cc;
-            B[o] = OB::sub(B[o], acc);
+            B[o] = OB::sub(B[o], acc[q]);
           }
         }
-        __syncthreads();
       }
     }
+    __syncthreads();
   }
   __syncthreads();
 }
@@ -315,7 +513,7 @@ __device__ void cta_trsm_lower_h(const T* L, int n, int ldl, T* B, int nrhs, int
   T* Lt = D + NB * NB;
   T* Xt = Lt + TL * NB;
   __shared__ R rdiag[NB];
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int nblk = (n + NB - 1) / NB;
   for (int kbI = nblk - 1; kbI >= 0; --kbI) {
     const int k0 = kbI * NB;
@@ -339,29 +537,32 @@ __device__ void cta_trsm_lower_h(const T* L, int n, int ldl, T* B, int nrhs, int
     __syncthreads();
     // update rows above: B[i][c] -= sum_t conj(L[k0+t][i]) X[k0+t][c], i < k0
     for (int i0 = 0; i0 < k0; i0 += TL) {
-      for (int e = tid; e < TL * NB; e += blockDim.x) {
-        int r = e / NB, t = e % NB;     // Lt[r][t] = conj(L[k0+t][i0+r])
-        Lt[e] = (i0 + r < k0 && t < kb) ? O::conj(L[(size_t)(k0 + t) * ldl + i0 + r]) : O::zero();
+      T a[4];   // rows of L^H: row r of the transpose of L's rows k0 + t (loaded along r, placed by BT below)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int t = 4 * w + u;
+        a[u] = (t < kb && i0 + lane < k0) ? O::conj(L[(size_t)(k0 + t) * ldl + i0 + lane]) : O::zero();
       }
       for (int c0 = 0; c0 < nrhs; c0 += TL) {
-        for (int e = tid; e < NB * TL; e += blockDim.x) {
-          int t = e / TL, c = e % TL;
-          Xt[e] = (t < kb && c0 + c < nrhs) ? B[(size_t)(k0 + t) * ldb + c0 + c] : O::zero();
+        T b[4], acc[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int t = 4 * w + u;
+          b[u] = (t < kb && c0 + lane < nrhs) ? B[(size_t)(k0 + t) * ldb + c0 + lane] : O::zero();
+          acc[u] = O::zero();
         }
-        __syncthreads();
-        for (int e = tid; e < TL * TL; e += blockDim.x) {
-          int r = e / TL, c = e % TL;
-          int i = i0 + r, cc = c0 + c;
+        tile_product<T, false, true>(a, b, Lt, Xt, kb, acc);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int i = i0 + w + 8 * q, cc = c0 + lane;
           if (i < k0 && cc < nrhs) {
-            T acc = O::zero();
-            for (int t = 0; t < kb; ++t) acc = O::fma(Lt[r * NB + t], Xt[t * TL + c], acc);
             size_t o = (size_t)i * ldb + cc;
-            B[o] = O::sub(B[o], acc);
+            B[o] = O::sub(B[o], acc[q]);
           }
         }
-        __syncthreads();
       }
     }
+    __syncthreads();
   }
   __syncthreads();
 }
@@ -374,36 +575,25 @@ __device__ void cta_gemm(bool transA, int m, int n, int k, typename Ops<T>::R al
                          const T* A, int lda, const T* B, int ldb,
                          typename Ops<T>::R beta, T* C, int ldc, T* smem) {
   using O = Ops<T>;
-  T* At = smem;               // At[r][t]: op(A)[i0+r][k0+t]
-  T* Bt = smem + TL * NB;     // Bt[t][c]: B[k0+t][j0+c]
-  const int tid = threadIdx.x;
+  T* At = smem;
+  T* Bt = smem + TL * NB;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   constexpr int PER = TL * TL / CTA_THREADS;   // outputs per thread
   for (int i0 = 0; i0 < m; i0 += TL) {
     for (int j0 = 0; j0 < n; j0 += TL) {
       T acc[PER];
       for (int q = 0; q < PER; ++q) acc[q] = O::zero();
       for (int k0 = 0; k0 < k; k0 += NB) {
-        for (int e = tid; e < TL * NB; e += blockDim.x) {
-          int r = e / NB, t = e % NB;
-          T v = O::zero();
-          if (i0 + r < m && k0 + t < k)
-            v = transA ? O::conj(A[(size_t)(k0 + t) * lda + i0 + r]) : A[(size_t)(i0 + r) * lda + k0 + t];
-          At[e] = v;
+        T a[4], b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int v = 4 * w + u;
+          if (transA) a[u] = (i0 + lane < m && k0 + v < k) ? O::conj(A[(size_t)(k0 + v) * lda + i0 + lane]) : O::zero();
+          else a[u] = (i0 + v < m && k0 + lane < k) ? A[(size_t)(i0 + v) * lda + k0 + lane] : O::zero();
+          b[u] = (k0 + v < k && j0 + lane < n) ? B[(size_t)(k0 + v) * ldb + j0 + lane] : O::zero();
         }
-        for (int e = tid; e < NB * TL; e += blockDim.x) {
-          int t = e / TL, c = e % TL;
-          Bt[e] = (k0 + t < k && j0 + c < n) ? B[(size_t)(k0 + t) * ldb + j0 + c] : O::zero();
-        }
-        __syncthreads();
-        for (int q = 0; q < PER; ++q) {
-          int e = tid + q * CTA_THREADS;
-          int r = e / TL, c = e % TL;
-          T a = acc[q];
-#pragma unroll 8
-          for (int t = 0; t < NB; ++t) a = O::fma(At[r * NB + t], Bt[t * TL + c], a);
-          acc[q] = a;
-        }
-        __syncthreads();
+        if (transA) tile_product<T, false, true>(a, b, At, Bt, NB, acc);
+        else tile_product<T, false>(a, b, At, Bt, NB, acc);
       }
       for (int q = 0; q < PER; ++q) {
         int e = tid + q * CTA_THREADS;
@@ -431,7 +621,7 @@ __device__ void cta_trinv_lower(const T* L, int n, int ldl, T* X, int ldx, char*
   T* Lt = D + NB * NB;
   T* Xt = Lt + TL * NB;
   __shared__ R rdiag[NB];
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   for (int k0 = 0; k0 < n; k0 += NB) {
     const int kb = min(NB, n - k0);
     const int k1 = k0 + kb;
@@ -453,30 +643,33 @@ __device__ void cta_trinv_lower(const T* L, int n, int ldl, T* X, int ldx, char*
     }
     __syncthreads();
     for (int i0 = k1; i0 < n; i0 += TL) {
-      for (int e = tid; e < TL * NB; e += blockDim.x) {
-        int r = e / NB, t = e % NB;
-        Lt[e] = (i0 + r < n && t < kb) ? tm.ld(&L[(size_t)(i0 + r) * ldl + k0 + t]) : O::zero();
+      T a[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = i0 + 4 * w + u;
+        a[u] = (r < n && lane < kb) ? tm.ld(&L[(size_t)r * ldl + k0 + lane]) : O::zero();
       }
       for (int c0 = 0; c0 < k1; c0 += TL) {
         if (!tm.own_col(c0 / TL)) continue;
-        for (int e = tid; e < NB * TL; e += blockDim.x) {
-          int t = e / TL, c = e % TL;
-          Xt[e] = (t < kb && c0 + c < k1) ? tm.ld(&X[(size_t)(k0 + t) * ldx + c0 + c]) : O::zero();
+        T b[4], acc[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int t = 4 * w + u;
+          b[u] = (t < kb && c0 + lane < k1) ? tm.ld(&X[(size_t)(k0 + t) * ldx + c0 + lane]) : O::zero();
+          acc[u] = O::zero();
         }
-        __syncthreads();
-        for (int e = tid; e < TL * TL; e += blockDim.x) {
-          int r = e / TL, c = e % TL;
-          int i = i0 + r, cc = c0 + c;
+        tile_product<T, false>(a, b, Lt, Xt, kb, acc);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int i = i0 + w + 8 * q, cc = c0 + lane;
           if (i < n && cc < k1) {
-            T acc = O::zero();
-            for (int t = 0; t < kb; ++t) acc = O::fma(Lt[r * NB + t], Xt[t * TL + c], acc);
             size_t o = (size_t)i * ldx + cc;
-            X[o] = O::sub(tm.ld(&X[o]), acc);
+            X[o] = O::sub(tm.ld(&X[o]), acc[q]);
           }
         }
-        __syncthreads();
       }
     }
+    __syncthreads();
   }
   __syncthreads();
 }
@@ -492,7 +685,7 @@ __device__ void cta_herk_lower(const T* X, int kdim, int n, int ldx, T* M, int l
   using O = Ops<T>;
   T* At = smem;
   T* Bt = smem + TL * NB;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   constexpr int PER = TL * TL / CTA_THREADS;
   for (int i0 = 0; i0 < n; i0 += TL) {
     for (int j0 = 0; j0 <= i0; j0 += TL) {
@@ -500,24 +693,14 @@ __device__ void cta_herk_lower(const T* X, int kdim, int n, int ldx, T* M, int l
       T acc[PER];
       for (int q = 0; q < PER; ++q) acc[q] = O::zero();
       for (int k0 = tri ? i0 : 0; k0 < kdim; k0 += NB) {
-        for (int e = tid; e < TL * NB; e += blockDim.x) {
-          int r = e / NB, t = e % NB;
-          At[e] = (i0 + r < n && k0 + t < kdim) ? O::conj(tm.ld(&X[(size_t)(k0 + t) * ldx + i0 + r])) : O::zero();
+        T a[4], b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int t = 4 * w + u;
+          a[u] = (i0 + lane < n && k0 + t < kdim) ? O::conj(tm.ld(&X[(size_t)(k0 + t) * ldx + i0 + lane])) : O::zero();
+          b[u] = (k0 + t < kdim && j0 + lane < n) ? tm.ld(&X[(size_t)(k0 + t) * ldx + j0 + lane]) : O::zero();
         }
-        for (int e = tid; e < NB * TL; e += blockDim.x) {
-          int t = e / TL, c = e % TL;
-          Bt[e] = (k0 + t < kdim && j0 + c < n) ? tm.ld(&X[(size_t)(k0 + t) * ldx + j0 + c]) : O::zero();
-        }
-        __syncthreads();
-        for (int q = 0; q < PER; ++q) {
-          int e = tid + q * CTA_THREADS;
-          int r = e / TL, c = e % TL;
-          T a = acc[q];
-#pragma unroll 8
-          for (int t = 0; t < NB; ++t) a = O::fma(At[r * NB + t], Bt[t * TL + c], a);
-          acc[q] = a;
-        }
-        __syncthreads();
+        tile_product<T, false, true>(a, b, At, Bt, NB, acc);
       }
       for (int q = 0; q < PER; ++q) {
         int e = tid + q * CTA_THREADS;
