@@ -270,6 +270,8 @@ struct LevelPlan {
   std::vector<int4> oitems, oitems16;
   std::vector<int32_t> omem;
   std::vector<int4> mbitems, mcitems;   // macro transfers: outputs I, outputs S
+  std::vector<int32_t> kcls;       // h-transition: classes of the macro elements and each class's
+  std::vector<int64_t> krep;       // first one, or empty (every macro element condensed)
   int64_t max_n = 0, sum_sq = 0;
 };
 struct HostPlan {

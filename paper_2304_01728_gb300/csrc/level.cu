@@ -123,14 +123,14 @@ __device__ __forceinline__ double2 widen(double2 a) { return a; }
 __device__ __forceinline__ double2 widen(float2 a) { return make_double2(a.x, a.y); }   // exact
 
 // block (e, s): slice s of element e's entries (the slices of one element are
-// disjoint); TE = double2, or float2 for the mixed path's complex64 macro
+// disjoint); with cls, E holds one matrix per class and cls[e] is element e's; TE = double2, or float2 for the mixed path's complex64 macro
 // element matrices (widened exactly)
 template <class TE>
-__global__ void k_ecsr_add(ECSRDev A, const TE* E, const int64_t* dofs, int64_t nel, int nloc, int64_t e0,
-                           int n0, int n1, int color) {
+__global__ void k_ecsr_add(ECSRDev A, const TE* E, const int32_t* cls, const int64_t* dofs, int64_t nel, int nloc,
+                           int64_t e0, int n0, int n1, int color) {
   const int64_t e = blockIdx.x;
   if (elem_color(e0 + e, n0, n1) != color) return;
-  const TE* Ee = E + e * (size_t)nloc * nloc;
+  const TE* Ee = E + (cls ? cls[e] : e) * (size_t)nloc * nloc;
   const int64_t* g = dofs + e * nloc;
   for (int q = blockIdx.y * blockDim.x + threadIdx.x; q < nloc * nloc; q += gridDim.y * blockDim.x) {
     int i = q / nloc, j = q % nloc;
@@ -145,20 +145,20 @@ __global__ void k_ecsr_add(ECSRDev A, const TE* E, const int64_t* dofs, int64_t 
 }
 
 template <class TE>
-static void ecsr_add_t(ECSRDev& D, const TE* E, const int64_t* dofs, int64_t nel, int nloc, int64_t e0,
-                       const int ext[3], cudaStream_t st) {
+static void ecsr_add_t(ECSRDev& D, const TE* E, const int32_t* cls, const int64_t* dofs, int64_t nel, int nloc,
+                       int64_t e0, const int ext[3], cudaStream_t st) {
   if (nel == 0) return;
   // one colour holds ~nel / 8 elements: slices of ~2048 entries per block keep the passes wide
   const unsigned slices = (unsigned)std::max<int64_t>(1, std::min<int64_t>(64, ((int64_t)nloc * nloc + 2047) / 2048));
   for (int c = 0; c < 8; ++c) {
-    k_ecsr_add<TE><<<dim3((unsigned)nel, slices), 256, 0, st>>>(D, E, dofs, nel, nloc, e0, ext[0], ext[1], c);
+    k_ecsr_add<TE><<<dim3((unsigned)nel, slices), 256, 0, st>>>(D, E, cls, dofs, nel, nloc, e0, ext[0], ext[1], c);
     DPG_CHECK_LAUNCH();
   }
 }
 
 void ecsr_add_elements(ECSRDev& D, const double2* E, const int64_t* dofs, int64_t nel, int nloc, int64_t e0,
                        const int ext[3], cudaStream_t st) {
-  ecsr_add_t<double2>(D, E, dofs, nel, nloc, e0, ext, st);
+  ecsr_add_t<double2>(D, E, nullptr, dofs, nel, nloc, e0, ext, st);
 }
 
 std::vector<std::vector<int64_t>> element_groups(const MeshL& m) {
@@ -212,6 +212,7 @@ template <class C>
 struct MacroArgs {
   int nS, nI, nlf, nlc;
   int64_t K0;
+  const int64_t* rep;         // macro elements of the launch, or null: K0, K0 + 1, ...
   const double2* Ef;          // fine element matrices
   const int64_t* fdofs;       // fine element DOFs
   const int32_t* child_map;   // [8][nlf]
@@ -235,7 +236,7 @@ __global__ void __launch_bounds__(CTA_THREADS) k_macro(MacroArgs<C> a) {
   using O = Ops<C>;
   using R = typename O::R;
   const int64_t lk = blockIdx.x;
-  const int64_t K = a.K0 + lk;
+  const int64_t K = a.rep ? a.rep[lk] : a.K0 + lk;
   const int nS = a.nS, nI = a.nI, n = nS + nI;
   C* AK = a.AK + lk * (size_t)n * n;
   for (int64_t q = threadIdx.x; q < (int64_t)n * n; q += blockDim.x) AK[q] = O::zero();
@@ -293,10 +294,23 @@ __global__ void __launch_bounds__(CTA_THREADS) k_macro(MacroArgs<C> a) {
   }
 }
 
+// Outputs of macro element K from those of its class's representative.
+template <class C>
+__global__ void k_macro_copy(MacroArgs<C> a, const int32_t* __restrict__ cls) {
+  const int64_t K = blockIdx.x, r = a.rep[cls[K]];
+  if (r == K) return;
+  auto copy = [&](auto* p, size_t n) {
+    for (size_t q = threadIdx.x; q < n; q += blockDim.x) p[K * n + q] = p[r * n + q];
+  };
+  copy(a.Y, (size_t)a.nI * a.nS);
+  copy(a.Ai, (size_t)a.nI * a.nI);
+  copy(a.EcOut, (size_t)a.nlc * a.nlc);
+}
+
 // ------------------------------------------------------- operator by cells
 // Class matrices: one CTA per class c, from the matrix of its first cell
 // (E + (rep[c] - e0) n^2; classes whose first cell is outside e0 .. e0 + ne - 1
-// are skipped): W[k][a] = conj(A[a][k]) (classes.cuh), as reals when every
+// are skipped; ne = 0: E holds one matrix per class): W[k][a] = conj(A[a][k]) (classes.cuh), as reals when every
 // entry is real once the unit phases are taken out (pack; exact test, as
 // k_pack_ops), with low parts when Wlo is given (TE = double2).
 template <class TE>
@@ -304,8 +318,8 @@ __global__ void k_cell_class(const TE* __restrict__ E, int64_t e0, int64_t ne, c
                              const int32_t* __restrict__ idx, int n, int64_t stride, int64_t offU, bool pack,
                              float2* __restrict__ W, float2* __restrict__ Wlo, uint8_t* __restrict__ rflag) {
   const int64_t c = blockIdx.x, e = rep[c];
-  if (e < e0 || e >= e0 + ne) return;
-  const TE* A = E + (e - e0) * (size_t)n * n;
+  if (ne > 0 && (e < e0 || e >= e0 + ne)) return;
+  const TE* A = E + (ne > 0 ? e - e0 : c) * (size_t)n * n;
   const int32_t* g = idx + e * n;
   auto phat = [&](int q) { return g[q] >= 0 && g[q] < offU ? 1 : 0; };
   bool cplx = !pack;
@@ -406,7 +420,8 @@ static void cell_op_begin(SystemImpl& S, Level& F, const LevelPlan& lp, cudaStre
   D.on = true;
 }
 
-// Matrices of the classes whose first cell is among cells e0 .. e0 + ne - 1 (E: their matrices).
+// Matrices of the classes whose first cell is among cells e0 .. e0 + ne - 1
+// (E: their matrices), or of all classes (ne = 0; E: one matrix per class).
 template <class TE>
 static void cell_op_matrices(SystemImpl& S, Level& F, const int64_t* rep, const TE* E, int64_t e0, int64_t ne,
                              cudaStream_t st) {
@@ -417,10 +432,21 @@ static void cell_op_matrices(SystemImpl& S, Level& F, const int64_t* rep, const 
   DPG_CHECK_LAUNCH();
 }
 
+// Macro elements of one class (macro_classes) have the same matrices, bit for
+// bit: the class's first one is condensed and the others get copies.  The 2,048
+// macro elements of a layered 32 x 32 x 16 mesh (p = 2) took 9.6 ms one by one;
+// by classes the operator phase ends 7 ms earlier.  Any sharing gains, since a
+// copy only moves what the condensation writes as well.  Not taken for more
+// classes than MACRO_CHUNK: their matrices are held at once, in the scratch of
+// one chunk.
+constexpr int64_t MACRO_CHUNK = 2048;
+
 template <class C>
-static void macro_condense(SystemImpl& S, Level& F, Level& C_, const MacroHost& M, const int32_t* cmap, int* dinfo,
+static void macro_condense(SystemImpl& S, Level& F, Level& C_, const LevelPlan& lp, const int32_t* cmap, int* dinfo,
                            C* Y, C* Ai, const int64_t* crep, cudaStream_t st) {
   Alloc& A = S.mem;
+  const MacroHost& M = lp.M;
+  const bool shared = !lp.krep.empty();
   std::vector<C> ik(M.IK.size());
   for (size_t i = 0; i < ik.size(); ++i) {
     ik[i].x = (typename Ops<C>::R)M.IK[i];
@@ -428,7 +454,8 @@ static void macro_condense(SystemImpl& S, Level& F, Level& C_, const MacroHost& 
   }
   C* dIK = upload(A, ik, st);
   const int n = F.nS + F.nI;
-  int64_t chunk = std::min<int64_t>(F.nK, 2048);
+  const int64_t nrun = shared ? (int64_t)lp.krep.size() : F.nK;   // macro elements that are condensed
+  const int64_t chunk = std::min<int64_t>(nrun, MACRO_CHUNK);
   C* AK = A.arr<C>((size_t)chunk * n * n);
   C* T1 = A.arr<C>((size_t)chunk * F.nS * C_.nloc);
   C* MK = A.arr<C>((size_t)chunk * F.nS * F.nS);
@@ -442,12 +469,24 @@ static void macro_condense(SystemImpl& S, Level& F, Level& C_, const MacroHost& 
   a.Y = Y; a.Ai = Ai; a.Ec = Ec; a.EcOut = C_.E; a.info = dinfo;
   const size_t sm = (size_t)(NB * NB + 2 * TL * NB) * sizeof(C) + 64;
   DPG_CUDA(cudaFuncSetAttribute(k_macro<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  for (int64_t K0 = 0; K0 < F.nK; K0 += chunk) {
+  if (shared) {
+    int64_t* rep = upload(A, lp.krep, st);
+    int32_t* cls = upload(A, lp.kcls, st);
+    a.rep = rep;
+    k_macro<C><<<(unsigned)nrun, CTA_THREADS, sm, st>>>(a);
+    DPG_CHECK_LAUNCH();
+    k_macro_copy<C><<<(unsigned)F.nK, CTA_THREADS, 0, st>>>(a, cls);
+    DPG_CHECK_LAUNCH();
+    ecsr_add_t<C>(F.A, MK, cls, F.S_glob, F.nK, F.nS, 0, C_.mesh.n, st);
+    cell_op_matrices<C>(S, F, crep, MK, 0, 0, st);
+    A.release(rep);
+    A.release(cls);
+  } else for (int64_t K0 = 0; K0 < F.nK; K0 += chunk) {
     a.K0 = K0;
     int nb = (int)std::min<int64_t>(chunk, F.nK - K0);
     k_macro<C><<<nb, CTA_THREADS, sm, st>>>(a);
     DPG_CHECK_LAUNCH();
-    ecsr_add_t<C>(F.A, MK, F.S_glob + K0 * F.nS, nb, F.nS, K0, C_.mesh.n, st);
+    ecsr_add_t<C>(F.A, MK, nullptr, F.S_glob + K0 * F.nS, nb, F.nS, K0, C_.mesh.n, st);
     cell_op_matrices<C>(S, F, crep, MK, K0, nb, st);
   }
   A.release(AK);   // stream-ordered frees: after the launches above
@@ -1066,6 +1105,11 @@ std::shared_ptr<HostPlan> plan_host(const SystemImpl& S) {
       lp.E = prep_ecsr(F.mesh, lp.M.groups);
       lp.smask.assign(lp.M.smask.begin(), lp.M.smask.end());
       lp.H = 4;
+      const std::vector<int32_t>& mc = cells[l - 1];
+      for (size_t K = 0; K < mc.size(); ++K)
+        if (mc[K] == (int32_t)lp.krep.size()) lp.krep.push_back((int64_t)K);
+      if (lp.krep.size() < mc.size() && (int64_t)lp.krep.size() <= MACRO_CHUNK) lp.kcls = mc;
+      else lp.krep.clear();
     }
     lp.P = build_patches(F.mesh, lp.smask, lp.H, C.mesh.n, (S.op.flags & DPGMG_FLAG_PATCH_R2) != 0);
     const Patches& P = lp.P;
@@ -1215,11 +1259,11 @@ void build_hierarchy(SystemImpl& S, cudaStream_t st) {
       if (macro_fp32(S)) {
         F.Y32 = A.arr<float2>((size_t)F.nK * F.nI * F.nS);
         F.Ai32 = A.arr<float2>((size_t)F.nK * F.nI * F.nI);
-        macro_condense<float2>(S, F, C, M, cmap, dinfo, F.Y32, F.Ai32, crep, st);
+        macro_condense<float2>(S, F, C, lp, cmap, dinfo, F.Y32, F.Ai32, crep, st);
       } else {
         F.Y64 = A.arr<double2>((size_t)F.nK * F.nI * F.nS);
         F.Ai64 = A.arr<double2>((size_t)F.nK * F.nI * F.nI);
-        macro_condense<double2>(S, F, C, M, cmap, dinfo, F.Y64, F.Ai64, crep, st);
+        macro_condense<double2>(S, F, C, lp, cmap, dinfo, F.Y64, F.Ai64, crep, st);
       }
       A.release(crep);
     }
