@@ -694,13 +694,14 @@ static size_t smem_bytes_dense(size_t elt) { return (size_t)(NB * NB + 2 * TL * 
 // operators) they are scratch.
 static void element_core(SystemImpl& S, Level& L, const std::vector<double>& cvals, bool finest, cudaStream_t st);
 
-// CTAs per element of a dense step with at most `most` shares: enough for two
-// CTAs on every SM (nb elements), one where the elements alone are that many.
+// CTAs per element of a dense step with at most `most` shares: enough for eight
+// CTAs on every SM (nb elements; their barriers and panel solves leave the
+// pipes idle otherwise), one where the elements alone are that many.
 static unsigned elem_split(int nb, int most) {
   int dev = 0, nsm = 0;
   DPG_CUDA(cudaGetDevice(&dev));
   DPG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  return (unsigned)std::max(1, std::min(most, (2 * nsm + nb - 1) / std::max(nb, 1)));
+  return (unsigned)std::max(1, std::min(most, (8 * nsm + nb - 1) / std::max(nb, 1)));
 }
 
 // Gram Cholesky of nb elements: clusters of 2, 4 or 8 CTAs while they all fit
@@ -899,9 +900,9 @@ static void element_core(SystemImpl& S, Level& L, const std::vector<double>& cva
       k_elem_build<double, true><<<nb, CTA_THREADS, sm_build, st>>>(a);
       DPG_CHECK_LAUNCH();
       launch_elem_potrf(a, nb, sm_real, st);
-      k_elem_trsm_split<<<dim3(nb, elem_split(nb, nt2)), CTA_THREADS, sm_cplx, st>>>(a);
+      k_elem_trsm_split<<<dim3(nb, elem_split(nb, nt2)), CTA_THREADS, sm_real, st>>>(a);
       DPG_CHECK_LAUNCH();
-      k_elem_herk_split<<<dim3(nb, elem_split(nb, nt2 * (nt2 + 1) / 2)), CTA_THREADS, sm_cplx, st>>>(a);
+      k_elem_herk_split<<<dim3(nb, elem_split(nb, nt2 * (nt2 + 1) / 2)), CTA_THREADS, sm_real, st>>>(a);
       DPG_CHECK_LAUNCH();
       k_elem_split_assemble<<<nb, CTA_THREADS, 0, st>>>(a);
       DPG_CHECK_LAUNCH();
@@ -918,13 +919,13 @@ static void element_core(SystemImpl& S, Level& L, const std::vector<double>& cva
       DPG_CHECK_LAUNCH();
       launch_elem_potrf(a, nb, sm_real, st);
       const dim3 gt(nb, elem_split(nb, nt1)), gh(nb, elem_split(nb, nt1 * (nt1 + 1) / 2));
-      if (real) k_elem_trsm<double><<<gt, CTA_THREADS, sm_cplx, st>>>(a);
+      if (real) k_elem_trsm<double><<<gt, CTA_THREADS, sm_real, st>>>(a);
       else k_elem_trsm<double2><<<gt, CTA_THREADS, sm_cplx, st>>>(a);
       DPG_CHECK_LAUNCH();
-      if (real) k_elem_herk<double><<<gh, CTA_THREADS, sm_cplx, st>>>(a);
+      if (real) k_elem_herk<double><<<gh, CTA_THREADS, sm_real, st>>>(a);
       else k_elem_herk<double2><<<gh, CTA_THREADS, sm_cplx, st>>>(a);
       DPG_CHECK_LAUNCH();
-      if (real) launch_elem_condense<double, false>(a, nb, sm_cplx, st);
+      if (real) launch_elem_condense<double, false>(a, nb, sm_real, st);
       else launch_elem_condense<double2, false>(a, nb, sm_cplx, st);
     }
   };
@@ -1019,12 +1020,12 @@ static void element_core(SystemImpl& S, Level& L, const std::vector<double>& cva
       k_elem_build<double><<<nb, CTA_THREADS, sm_build, st>>>(a);
       DPG_CHECK_LAUNCH();
       launch_elem_potrf(a, nb, sm_real, st);
-      k_elem_trsm<double><<<dim3(nb, elem_split(nb, nt1)), CTA_THREADS, sm_cplx, st>>>(a);
+      k_elem_trsm<double><<<dim3(nb, elem_split(nb, nt1)), CTA_THREADS, sm_real, st>>>(a);
       DPG_CHECK_LAUNCH();
-      k_elem_herk<double><<<dim3(nb, elem_split(nb, nt1 * (nt1 + 1) / 2)), CTA_THREADS, sm_cplx, st>>>(a);
+      k_elem_herk<double><<<dim3(nb, elem_split(nb, nt1 * (nt1 + 1) / 2)), CTA_THREADS, sm_real, st>>>(a);
       DPG_CHECK_LAUNCH();
       if (nm) member_loads(rch, de, false);
-      launch_elem_condense<double, false>(a, nb, sm_cplx, st);
+      launch_elem_condense<double, false>(a, nb, sm_real, st);
       if (nm) {
         int4* dch = upload(A, rch, st);
         k_elem_member_condense<double, false><<<(unsigned)rch.size(), CTA_THREADS, sm_cplx, st>>>(a, de, dch, Ub, Cb,
@@ -1044,9 +1045,9 @@ static void element_core(SystemImpl& S, Level& L, const std::vector<double>& cva
       k_elem_build<double, true><<<nb, CTA_THREADS, sm_build, st>>>(a);
       DPG_CHECK_LAUNCH();
       launch_elem_potrf(a, nb, sm_real, st);
-      k_elem_trsm_split<<<dim3(nb, elem_split(nb, nt2)), CTA_THREADS, sm_cplx, st>>>(a);
+      k_elem_trsm_split<<<dim3(nb, elem_split(nb, nt2)), CTA_THREADS, sm_real, st>>>(a);
       DPG_CHECK_LAUNCH();
-      k_elem_herk_split<<<dim3(nb, elem_split(nb, nt2 * (nt2 + 1) / 2)), CTA_THREADS, sm_cplx, st>>>(a);
+      k_elem_herk_split<<<dim3(nb, elem_split(nb, nt2 * (nt2 + 1) / 2)), CTA_THREADS, sm_real, st>>>(a);
       DPG_CHECK_LAUNCH();
       if (nm) member_loads(sch, de, true);   // before the assembly below reuses the W slots
       k_elem_split_assemble<<<nb, CTA_THREADS, 0, st>>>(a);
