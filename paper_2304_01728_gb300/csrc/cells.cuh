@@ -5,6 +5,7 @@
 // cells, so the FP32 pipe and the gathers set the time.
 #pragma once
 #include "classes.cuh"
+#include "digits.cuh"
 
 namespace dpgmg {
 
@@ -42,7 +43,7 @@ static __global__ void __launch_bounds__(CLS_THREADS, CLS_CTAS) k_class_cell(con
 #undef DPG_ITEM
 }
 
-// ---- double-float form (CG operator) ----
+// ---- CG operator ----
 __device__ __forceinline__ void df_add(float& sh, float& sl, float p, float q) {
   const float s = sh + p;
   const float bb = s - sh;
@@ -57,184 +58,203 @@ __device__ __forceinline__ void df_mul(float ah, float al, float xh, float xl, f
   q = fmaf(al, xh, q);
 }
 
-// The same product for the CG operator in double-float (solve.cu): matrices as
-// FP32 high and low parts (W + Wl), x likewise, products and sums with
-// error-free FP32 transformations.  12 FP32 instructions per real product, so
-// the FP32 pipe bounds it; a thread owns 4 outputs x MPT members, 16 bytes of
-// accumulator each.  ybuf: (re hi, re lo, im hi, im lo).
-constexpr int CDF_K = 8;        // rows per stage
-constexpr int CDF_STAGES = 3;
-struct ClassDfSmem {
-  __align__(16) unsigned char w[CDF_STAGES][2][CDF_K * 64 * sizeof(float2)];   // high, low parts
-  __align__(16) float4 r[2][CDF_K][16 + 1];
-  int64_t base[16];
-};
+// The same product for the CG operator: 56-bit fixed point on the tensor cores.
+// A row a of a class matrix is 2^ea times integers of 55 bits, the DOFs of a
+// cell are 2^ex times such integers, and both are written as DG_S = 7 signed
+// digits of 8 bits (-128 .. 127), which bf16 holds exactly.  Digit products of
+// equal weight s + t = o share one FP32 accumulator per output: at most
+// 7 DG_KC products of at most 2^14 each, an integer below 2^24, so every
+// accumulator is exact (error-free splitting as in Mukunoki, Ozaki, Ogita and
+// Imamura, "DGEMM using tensor cores", 2020).  Pairs with o > 6 lie below the
+// operands' own rounding and are left out.  The seven accumulators are joined
+// with error-free FP32 sums into high and low parts.
+//
+// Bound: 28 bf16 products per entry and real column on mma.sync (m16n8k16,
+// 0.5 a clock and SM: 50 us on a layered 32 x 32 x 16 mesh, p = 3), where the
+// double-float form took 12 FP32 instructions per real product.  Operator there
+// 281 -> 158 us, on 16^3, p = 3, 88 -> 66 us, and half the error against
+// complex128 (2.6e-15 to 5e-15 in norm, before 5.5e-15 to 8.8e-15).  Tried:
+// the next tile's digits prefetched into L1, no change; the conversions are
+// half of the instructions, but twice as many only cost 4%.  A CTA turns the DOFs of up to 32 cells (64 real columns,
+// DG_KC rows) into digits once, in shared memory; a warp owns 16 outputs x 8
+// cells, with the matrix's digits read from L2 in fragment order (512 bytes a
+// warp and tile).
+constexpr int DG_LD = DG_KC + 8;   // row length in shared memory: 240 bytes, 8 rows on distinct banks
+constexpr int DG_COLS = 64;
+constexpr int DG_THREADS = 256;
+constexpr int DG_SMEM = DG_S * DG_COLS * DG_LD * 2;
 
-template <int TX, int MPT, bool CX>
-__device__ __forceinline__ void class_item_df(ClassDfSmem& sm, const float2* __restrict__ Wh,
-                                              const float2* __restrict__ Wl, int64_t ld, int n, int a0, int cnt,
-                                              const int32_t* __restrict__ idx, const float2* __restrict__ xh,
-                                              const float2* __restrict__ xl, float4* __restrict__ out,
-                                              const int32_t* __restrict__ rep_idx, int64_t offU) {
-  constexpr int TM = 4 * TX, TN = (CLS_THREADS / TX) * MPT;
-  constexpr int EL = CX ? 8 : 4;
-  constexpr int ROW16 = TM * EL / 16;
-  constexpr int NP = 2 * CDF_K * ROW16;                            // 16-byte pieces per stage, high then low
-  constexpr int NW = (NP + CLS_THREADS - 1) / CLS_THREADS;
-  constexpr int NG = (CDF_K * TN + CLS_THREADS - 1) / CLS_THREADS; // gathered values per thread and chunk
-  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
-  const int gk = tid % CDF_K, gm = tid / CDF_K;                    // gather: row, first member (then + 16)
-  const char* W[2] = {reinterpret_cast<const char*>(Wh) + (int64_t)a0 * EL,
-                      reinterpret_cast<const char*>(Wl) + (int64_t)a0 * EL};
-  const int wcols = (int)(ld - a0);
-  const int nch = (n + CDF_K - 1) / CDF_K;
-
-  auto load_w = [&](int c) {
-    if (c < nch) {
-#pragma unroll
-      for (int q = 0; q < NW; ++q) {
-        const int p = tid + q * CLS_THREADS;
-        if (NP % CLS_THREADS == 0 || p < NP) {
-          const int part = p / (CDF_K * ROW16), pp = p % (CDF_K * ROW16), row = pp / ROW16, col = pp % ROW16;
-          const int k = c * CDF_K + row;
-          const bool in = k < n && col * (16 / EL) < wcols;
-          cp_async16_zfill(sm.w[c % CDF_STAGES][part] + row * (TM * EL) + col * 16,
-                           in ? W[part] + (int64_t)k * ld * EL + col * 16 : W[part], in);
-        }
-      }
-    }
-    cp_async_commit();
-  };
-  int gi[NG];
-  float4 gv[NG];
-  auto load_idx = [&](int c) {
-    const int k = c * CDF_K + gk;
-#pragma unroll
-    for (int q = 0; q < NG; ++q) {
-      const int m = gm + 16 * q;
-      gi[q] = (k < n && m < cnt) ? __ldg(idx + sm.base[m] + k) : -1;
-    }
-  };
-  auto load_val = [&]() {
-#pragma unroll
-    for (int q = 0; q < NG; ++q) {
-      float2 h = make_float2(0.f, 0.f), l = h;
-      if (gi[q] >= 0) {
-        h = xh[gi[q]];
-        l = xl[gi[q]];
-        if (!CX) {
-          const int s = gi[q] < offU ? -1 : 0;
-          h = mul_i(h, s);
-          l = mul_i(l, s);
-        }
-      }
-      gv[q] = make_float4(h.x, l.x, h.y, l.y);
-    }
-  };
-  auto store_val = [&](int c) {
-#pragma unroll
-    for (int q = 0; q < NG; ++q)
-      if (gm + 16 * q < TN) sm.r[c & 1][gk][gm + 16 * q] = gv[q];
-  };
-  float rh[MPT][4], rl[MPT][4], ih[MPT][4], il[MPT][4];
-#pragma unroll
-  for (int m = 0; m < MPT; ++m)
-#pragma unroll
-    for (int u = 0; u < 4; ++u) rh[m][u] = rl[m][u] = ih[m][u] = il[m][u] = 0.f;
-#pragma unroll
-  for (int c = 0; c < CDF_STAGES - 1; ++c) load_w(c);
-  load_idx(0);
-  load_val();
-  store_val(0);
-  load_idx(1);
-  for (int c = 0; c < nch; ++c) {
-    cp_async_wait<CDF_STAGES - 2>();
-    __syncthreads();
-    load_w(c + CDF_STAGES - 1);
-    load_val();
-    load_idx(c + 2);
-    const unsigned char* wh = sm.w[c % CDF_STAGES][0] + tx * (4 * EL);
-    const unsigned char* wl = sm.w[c % CDF_STAGES][1] + tx * (4 * EL);
-    const float4* rs = &sm.r[c & 1][0][ty * MPT];
-#pragma unroll 2
-    for (int k = 0; k < CDF_K; ++k) {
-      float4 rv[MPT];
-#pragma unroll
-      for (int m = 0; m < MPT; ++m) rv[m] = rs[k * (16 + 1) + m];
-      float h[CX ? 8 : 4], l[CX ? 8 : 4];
-#pragma unroll
-      for (int q = 0; q < (CX ? 2 : 1); ++q) {
-        *reinterpret_cast<float4*>(h + 4 * q) = *reinterpret_cast<const float4*>(wh + k * (TM * EL) + 16 * q);
-        *reinterpret_cast<float4*>(l + 4 * q) = *reinterpret_cast<const float4*>(wl + k * (TM * EL) + 16 * q);
-      }
-#pragma unroll
-      for (int m = 0; m < MPT; ++m)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          float p, q;
-          if constexpr (!CX) {
-            df_mul(h[u], l[u], rv[m].x, rv[m].y, p, q);
-            df_add(rh[m][u], rl[m][u], p, q);
-            df_mul(h[u], l[u], rv[m].z, rv[m].w, p, q);
-            df_add(ih[m][u], il[m][u], p, q);
-          } else {   // conj(w) x
-            df_mul(h[2 * u], l[2 * u], rv[m].x, rv[m].y, p, q);
-            df_add(rh[m][u], rl[m][u], p, q);
-            df_mul(h[2 * u + 1], l[2 * u + 1], rv[m].z, rv[m].w, p, q);
-            df_add(rh[m][u], rl[m][u], p, q);
-            df_mul(h[2 * u], l[2 * u], rv[m].z, rv[m].w, p, q);
-            df_add(ih[m][u], il[m][u], p, q);
-            df_mul(h[2 * u + 1], l[2 * u + 1], rv[m].x, rv[m].y, p, q);
-            df_add(ih[m][u], il[m][u], -p, -q);
-          }
-        }
-    }
-    if (c + 1 < nch) store_val(c + 1);
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int a = a0 + 4 * tx + u;
-    if (a >= n) continue;
-    const bool s = !CX && rep_idx[a] < offU;   // output phase i, exact
-#pragma unroll
-    for (int m = 0; m < MPT; ++m) {
-      const int q = ty * MPT + m;
-      if (q < cnt)
-        out[sm.base[q] + a] = s ? make_float4(-ih[m][u], -il[m][u], rh[m][u], rl[m][u])
-                                : make_float4(rh[m][u], rl[m][u], ih[m][u], il[m][u]);
-    }
-  }
+__device__ __forceinline__ void mma_bf16(float c[4], const uint4& a, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+               "{%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
 
-static __global__ void __launch_bounds__(CLS_THREADS, 4) k_class_cell_df(const int32_t* __restrict__ idx,
-                                                               const int32_t* __restrict__ cls, int n, int64_t stride,
-                                                               const int4* __restrict__ items,
-                                                               const int32_t* __restrict__ mem,
-                                                               const float2* __restrict__ Wh,
-                                                               const float2* __restrict__ Wl,
-                                                               const uint8_t* __restrict__ rflag,
-                                                               const float2* __restrict__ xh,
-                                                               const float2* __restrict__ xl,
-                                                               float4* __restrict__ ybuf, int64_t offU) {
-  __shared__ ClassDfSmem sm;
-  const int4 it = items[blockIdx.x];
-  const int cnt = it.y, a0 = it.z;
-  const int e = mem[it.x], c = cls[e];
-  if ((int)threadIdx.x < cnt) sm.base[threadIdx.x] = (int64_t)mem[it.x + threadIdx.x] * n;
+// the value of h + l in units of 2^(emax - 180): below 2^54 when emax is the
+// largest exponent field of the column (denormal parts count as zero)
+__device__ __forceinline__ long long digit_fixed(float h, int emax) {
+  const uint32_t u = __float_as_uint(h);
+  const int e = (u >> 23) & 255, sh = e - emax + 30;
+  const long long m = (u & 0x7fffff) | 0x800000;
+  if (e == 0 || sh < -25) return 0;
+  const long long f = sh >= 0 ? m << min(sh, 30) : (m + (1ll << (-sh - 1))) >> -sh;
+  return (int)u < 0 ? -f : f;
+}
+
+static __global__ void __launch_bounds__(DG_THREADS, 2) k_class_cell_dg(
+    const int32_t* __restrict__ idx, const int32_t* __restrict__ cls, int n, int64_t stride,
+    const int4* __restrict__ items, const int32_t* __restrict__ mem, const uint4* __restrict__ Dall,
+    const float* __restrict__ rowscale, const uint8_t* __restrict__ rflag, const float2* __restrict__ xh,
+    const float2* __restrict__ xl, float4* __restrict__ ybuf, int64_t offU) {
+  extern __shared__ __align__(16) uint16_t Bs[];   // [DG_S][DG_COLS][DG_LD] digits of column 2 m + (0 re, 1 im)
+  __shared__ float cscale[32];
+  __shared__ int64_t base[32];
+  const int4 it = items[blockIdx.x];   // first member, members, first 16-row tile, tiles
+  const int cnt = it.y, c = cls[mem[it.x]];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (tid < 32) base[tid] = tid < cnt ? (int64_t)mem[it.x + tid] * n : -1;
   __syncthreads();
-  const float2 *H = Wh + c * stride, *L = Wl + c * stride;
-  const int32_t* rep = idx + (int64_t)e * n;
-#define DPG_ITEM(TX, MPT)                                                                                   \
-  if (rflag[c] != 0)                                                                                        \
-    class_item_df<TX, MPT, false>(sm, H, L, patch_ldr(n), n, a0, cnt, idx, xh, xl, ybuf, rep, offU);        \
-  else                                                                                                      \
-    class_item_df<TX, MPT, true>(sm, H, L, patch_ld(n), n, a0, cnt, idx, xh, xl, ybuf, rep, offU)
-  switch (it.w) {   // items of at most 16 members
-    case CLS_64x16: DPG_ITEM(16, 2); break;
-    case CLS_64x8: DPG_ITEM(16, 1); break;
-    default: DPG_ITEM(8, 1); break;   // CLS_32x16
+  const int nq = (cnt + 7) / 8, npair = nq * it.w, KT = (n + 15) / 16, MT = KT;
+  const bool real = rflag[c] != 0;
+  const uint4* Dc = Dall + c * stride;
+  const float* rs = rowscale + (int64_t)c * MT * 16;
+  const int32_t* rep = idx + (int64_t)mem[it.x] * n;
+  for (int k0 = 0; k0 < n; k0 += DG_KC) {
+    const int nkt = min(DG_KC / 16, KT - k0 / 16);
+    if (k0 > 0) __syncthreads();   // the last chunk's readers are done
+    // digits of the columns: a warp takes members w, w + 8, ..., lanes two rows each
+    int g[4][2][2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int m = w + 8 * j, k = k0 + 64 * i + 2 * lane + u;
+          g[j][i][u] = (m < cnt && k < n && 64 * i + 2 * lane < DG_KC) ? __ldg(idx + base[m] + k) : -1;
+        }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int m = w + 8 * j;
+      if (m >= 8 * nq) break;   // uniform over the warp
+      float2 h[2][2], l[2][2];
+      uint32_t emax = 0;
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int gi = g[j][i][u];
+          h[i][u] = l[i][u] = make_float2(0.f, 0.f);
+          if (gi >= 0) {
+            h[i][u] = xh[gi];
+            l[i][u] = xl[gi];
+            if (real) {
+              const int s = gi < offU ? -1 : 0;
+              h[i][u] = mul_i(h[i][u], s);
+              l[i][u] = mul_i(l[i][u], s);
+            }
+          }
+          emax = max(emax, max(__float_as_uint(h[i][u].x) & 0x7fffffffu, __float_as_uint(h[i][u].y) & 0x7fffffffu));
+        }
+      emax = __reduce_max_sync(0xffffffffu, emax) >> 23;
+      // 2^(ex - 1), the column being 2^(ex - 54) times its integers, ex = emax - 126; infinities and NaN give NaN
+      if (lane == 0)
+        cscale[m] = emax == 255 ? __uint_as_float(0x7fffffffu) : (emax == 0 ? 0.f : __uint_as_float(emax << 23));
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int k = 64 * i + 2 * lane;
+        if (k >= 16 * nkt) continue;
+        uint32_t dr[DG_S], di[DG_S];
+        digit_pairs(digit_fixed(h[i][0].x, emax) + digit_fixed(l[i][0].x, emax),
+                    digit_fixed(h[i][1].x, emax) + digit_fixed(l[i][1].x, emax), dr);
+        digit_pairs(digit_fixed(h[i][0].y, emax) + digit_fixed(l[i][0].y, emax),
+                    digit_fixed(h[i][1].y, emax) + digit_fixed(l[i][1].y, emax), di);
+#pragma unroll
+        for (int s = 0; s < DG_S; ++s) {
+          *reinterpret_cast<uint32_t*>(Bs + (s * DG_COLS + 2 * m) * DG_LD + k) = dr[s];
+          *reinterpret_cast<uint32_t*>(Bs + (s * DG_COLS + 2 * m + 1) * DG_LD + k) = di[s];
+        }
+      }
+    }
+    __syncthreads();
+    const int gr = lane >> 2, tq = lane & 3;
+    for (int p = w; p < npair; p += DG_THREADS / 32) {
+      const int mt = it.z + p / nq, q0 = p % nq;   // rows 16 mt .. + 15, members 8 q0 .. + 7
+      float rh[2][4], rl[2][4];
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) rh[t][q] = rl[t][q] = 0.f;
+      // real classes: one pass.  Complex ones: Ar (xr, xi), then Ai (-xi, xr)
+      for (int half = 0; half < (real ? 1 : 2); ++half) {
+        float acc[2][DG_S][4];
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+          for (int s = 0; s < DG_S; ++s)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[t][s][q] = 0.f;
+        // ldmatrix rows: lanes 0-7 column tile 0, k 0-7; 8-15 the same, k 8-15; 16-31 column tile 1
+        const int col = 16 * q0 + ((lane >> 4) << 3) + (lane & 7);
+        uint32_t saddr = (uint32_t)__cvta_generic_to_shared(Bs + (col ^ half) * DG_LD + ((lane >> 3) & 1) * 8);
+        const uint32_t flip = (half && (gr & 1) == 0) ? 0x80008000u : 0u;   // column re of the second pass: -xi
+        const uint4* Da = Dc + ((int64_t)(half * MT + mt) * KT + k0 / 16) * (DG_S * 32) + lane;
+        for (int kt = 0; kt < nkt; ++kt, Da += DG_S * 32, saddr += 32) {
+          uint4 a[DG_S];
+#pragma unroll
+          for (int s = 0; s < DG_S; ++s) a[s] = __ldg(Da + s * 32);
+#pragma unroll
+          for (int t = 0; t < DG_S; ++t) {
+            uint32_t b0, b1, b2, b3;
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                         : "=r"(b0), "=r"(b1), "=r"(b2), "=r"(b3)
+                         : "r"(saddr + t * (DG_COLS * DG_LD * 2)));
+            b0 ^= flip;
+            b1 ^= flip;
+            b2 ^= flip;
+            b3 ^= flip;
+#pragma unroll
+            for (int s = 0; s + t < DG_S; ++s) {
+              mma_bf16(acc[0][s + t], a[s], b0, b1);
+              mma_bf16(acc[1][s + t], a[s], b2, b3);
+            }
+          }
+        }
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            float f = 1.f;
+#pragma unroll
+            for (int o = 0; o < DG_S; ++o, f *= 1.f / 256.f) df_add(rh[t][q], rl[t][q], acc[t][o][q] * f, 0.f);
+          }
+      }
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const int m = 8 * q0 + 4 * t + tq;
+        if (m >= cnt) continue;
+        const float cs = cscale[m];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const int a = 16 * mt + gr + 8 * r;
+          if (a >= n) continue;
+          const float sc = rs[a];
+          auto scale = [&](float v) { return v * sc * cs; };
+          float4 v = make_float4(scale(rh[t][2 * r]), scale(rl[t][2 * r]), scale(rh[t][2 * r + 1]),
+                                 scale(rl[t][2 * r + 1]));
+          if (real && rep[a] < offU) v = make_float4(-v.z, -v.w, v.x, v.y);   // output phase i, exact
+          float4* o = ybuf + base[m] + a;
+          if (k0 > 0) {   // this thread's sum over the earlier chunks
+            const float4 y = *o;
+            df_add(v.x, v.y, y.x, y.y);
+            df_add(v.z, v.w, y.z, y.w);
+          }
+          *o = v;
+        }
+      }
+    }
   }
-#undef DPG_ITEM
 }
 
 // calls f(value) for the slots of DOF g in list order (a fixed-pitch row of
@@ -300,11 +320,11 @@ static __global__ void k_cell_sum_df(const int32_t* __restrict__ tab, const int6
   y[g] = mode ? make_double2(b[g].x - re, b[g].y - im) : make_double2(re, im);
 }
 
-// y = A x (mode 0) or b - A x (mode 1) in double-float, x = xh + xl
+// y = A x (mode 0) or b - A x (mode 1), x = xh + xl
 inline void cell_op_apply_df(const CellOpDev& D, const float2* xh, const float2* xl, const double2* b, double2* y,
                              int mode, cudaStream_t st) {
-  k_class_cell_df<<<(unsigned)D.nitems16, CLS_THREADS, 0, st>>>(D.idx, D.cls, D.n, D.stride(), D.items16, D.mem, D.W,
-                                                               D.Wlo, D.rflag, xh, xl, D.ydf, D.offU);
+  k_class_cell_dg<<<(unsigned)D.ndgitems, DG_THREADS, DG_SMEM, st>>>(D.idx, D.cls, D.n, D.dgstride(), D.dgitems, D.mem,
+                                                                    D.dig, D.dgrow, D.rflag, xh, xl, D.ydf, D.offU);
   DPG_CHECK_LAUNCH();
   k_cell_sum_df<<<(unsigned)((D.ndof + 255) / 256), 256, 0, st>>>(D.tab, D.sptr, D.slots, D.offE, D.offF, D.ydf, b, y,
                                                                  D.ndof, mode);

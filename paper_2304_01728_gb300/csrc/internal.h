@@ -61,6 +61,8 @@ template <class T, class AL> T* upload(Alloc& A, const std::vector<T, AL>& h, cu
 // stored matrix per cell class (classes.cuh): the elements of a p level, the
 // macro elements of an h level.  Kept beside the assembled rows when the cells
 // are many per class.
+constexpr int DG_S = 7;        // 8-bit digits of a fixed-point operand of the CG operator by cells
+constexpr int DG_KC = 112;     // columns per exact accumulation: DG_S DG_KC 2^14 < 2^24
 struct CellOpDev {
   bool on = false;             // applied in place of the assembled rows (complex64 V-cycle operator)
   bool df_on = false;          // the same for the double-float CG operator
@@ -69,12 +71,16 @@ struct CellOpDev {
   int32_t* idx = nullptr;      // [ncell][n] DOF, or -1
   int32_t* cls = nullptr;      // [ncell] class
   float2* W = nullptr;         // [ncls][n x ld] conj(A_K)^T, complex64, or reals (rflag)
-  float2* Wlo = nullptr;       // low parts (A_K ~ W + Wlo), CG operator only
+  // CG operator only: digits of the class matrices (cells.cuh) in fragment order
+  // [class][re, im part][16-row tile][16-column tile][digit][lane] (uint4: one lane's share of a 16 x 16 tile) and
+  // the rows' scales
+  uint4* dig = nullptr;
+  float* dgrow = nullptr;
   uint8_t* rflag = nullptr;    // [ncls] real once the unit phases are taken out, rows of patch_ldr(n) reals
   int4* items = nullptr;       // work items as PatchDev::cls_items, over cells
   int64_t nitems = 0;
-  int4* items16 = nullptr;     // items of at most 16 members (double-float product)
-  int64_t nitems16 = 0;
+  int4* dgitems = nullptr;     // work items (first member, members, first 16-row tile, tiles)
+  int64_t ndgitems = 0;
   int32_t* mem = nullptr;      // cells class by class
   // the (cell, local) slots of every DOF: fixed-pitch rows (8 per vertex, 4 per edge and 2 per face DOF, -1 =
   // none) on a p level, CSR on an h level
@@ -85,6 +91,8 @@ struct CellOpDev {
   float2* ybuf = nullptr;      // [ncell][n] cell products
   float4* ydf = nullptr;       // the same in double-float (CG operator only)
   int64_t stride() const { return n * patch_ld(n); }   // entries per class matrix
+  int64_t tiles() const { return (n + 15) / 16; }
+  int64_t dgstride() const { return 2 * tiles() * tiles() * DG_S * 32; }
 };
 
 // first place of DOF g's row in CellOpDev::tab (also the table's size, for g = ndof)
@@ -267,7 +275,7 @@ struct LevelPlan {
   int64_t uniq_sq = 0;
   std::vector<int32_t> ocls;       // classes of the operator's cells, or empty (no shared cell matrices)
   std::vector<int64_t> orep;       // first cell of each class
-  std::vector<int4> oitems, oitems16;
+  std::vector<int4> oitems, dgitems;
   std::vector<int32_t> omem;
   std::vector<int4> mbitems, mcitems;   // macro transfers: outputs I, outputs S
   std::vector<int32_t> kcls;       // h-transition: classes of the macro elements and each class's
@@ -385,6 +393,7 @@ void spmv64(const ECSRDev& A, const double2* x, double2* y, cudaStream_t st);
 // inverses their high parts in P.inv32 and low parts in plo)
 void estimate_theta(SystemImpl& S, int level, double* rayleigh, const float2* plo, cudaStream_t st);
 // class matrices and work items of an h level's macro transfers (mixed path; needs Y32 and Ai32)
+void cell_op_df_init();   // launch attributes of the CG operator by cells
 void macro_op_setup(SystemImpl& S, Level& F, const LevelPlan& lp, cudaStream_t st);
 // double-float split of an operator's values: v32 (kept if already set) + vlo
 void split_operator(Alloc& M, ECSRDev& A, int64_t offU, bool pack, cudaStream_t st);

@@ -23,6 +23,7 @@
 #include "smoother.cuh"
 #include "block.cuh"
 #include "classes.cuh"
+#include "digits.cuh"
 
 namespace dpgmg {
 
@@ -312,11 +313,11 @@ __global__ void k_macro_copy(MacroArgs<C> a, const int32_t* __restrict__ cls) {
 // (E + (rep[c] - e0) n^2; classes whose first cell is outside e0 .. e0 + ne - 1
 // are skipped; ne = 0: E holds one matrix per class): W[k][a] = conj(A[a][k]) (classes.cuh), as reals when every
 // entry is real once the unit phases are taken out (pack; exact test, as
-// k_pack_ops), with low parts when Wlo is given (TE = double2).
+// k_pack_ops).
 template <class TE>
 __global__ void k_cell_class(const TE* __restrict__ E, int64_t e0, int64_t ne, const int64_t* __restrict__ rep,
                              const int32_t* __restrict__ idx, int n, int64_t stride, int64_t offU, bool pack,
-                             float2* __restrict__ W, float2* __restrict__ Wlo, uint8_t* __restrict__ rflag) {
+                             float2* __restrict__ W, uint8_t* __restrict__ rflag) {
   const int64_t c = blockIdx.x, e = rep[c];
   if (ne > 0 && (e < e0 || e >= e0 + ne)) return;
   const TE* A = E + (ne > 0 ? e - e0 : c) * (size_t)n * n;
@@ -328,7 +329,6 @@ __global__ void k_cell_class(const TE* __restrict__ E, int64_t e0, int64_t ne, c
       if (mul_i(A[q], phat(q % n) - phat(q / n)).y != 0) cplx = true;
   cplx = __syncthreads_or(cplx) != 0;
   float2* Wc = W + c * stride;
-  float2* Lc = Wlo ? Wlo + c * stride : nullptr;
   const int ld = (int)(cplx ? patch_ld(n) : patch_ldr(n));
   for (int q = threadIdx.x; q < n * ld; q += blockDim.x) {
     const int k = q / ld, a = q % ld;
@@ -337,17 +337,55 @@ __global__ void k_cell_class(const TE* __restrict__ E, int64_t e0, int64_t ne, c
       const TE t = A[(size_t)a * n + k];
       v = cplx ? make_double2(t.x, -(double)t.y) : make_double2(mul_i(t, phat(k) - phat(a)).x, 0.0);
     }
-    const float2 h = make_float2((float)v.x, (float)v.y);
-    const float2 l = make_float2((float)(v.x - (double)h.x), (float)(v.y - (double)h.y));
-    if (cplx) {
-      Wc[q] = h;
-      if (Lc) Lc[q] = l;
-    } else {
-      reinterpret_cast<float*>(Wc)[q] = h.x;
-      if (Lc) reinterpret_cast<float*>(Lc)[q] = l.x;
-    }
+    if (cplx) Wc[q] = make_float2((float)v.x, (float)v.y);
+    else reinterpret_cast<float*>(Wc)[q] = (float)v.x;
   }
   if (threadIdx.x == 0) rflag[c] = cplx ? 0 : 1;
+}
+
+// Digits of the class matrices (cells.cuh; after k_cell_class, which sets
+// rflag).  One CTA per class; dynamic shared memory: an int per padded row.
+static __global__ void k_cell_digits(const double2* __restrict__ E, const int64_t* __restrict__ rep,
+                                     const int32_t* __restrict__ idx, int n, int64_t offU,
+                                     const uint8_t* __restrict__ rflag, uint4* __restrict__ dig, int64_t stride,
+                                     float* __restrict__ rowscale) {
+  extern __shared__ int rowexp[];   // row a: |entries| < 2^rowexp[a]
+  const int64_t c = blockIdx.x, e = rep[c];
+  const double2* A = E + e * (size_t)n * n;
+  const int32_t* g = idx + e * n;
+  const bool real = rflag[c] != 0;
+  const int T = (n + 15) / 16, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  auto phat = [&](int q) { return g[q] >= 0 && g[q] < offU ? 1 : 0; };
+  auto entry = [&](int a, int k, int part) {
+    if (a >= n || k >= n) return 0.0;
+    const double2 v = A[(size_t)a * n + k];
+    return real ? mul_i(v, phat(k) - phat(a)).x : (part ? v.y : v.x);
+  };
+  for (int a = w; a < 16 * T; a += blockDim.x / 32) {
+    double mx = 0.0;
+    for (int k = lane; k < n; k += 32) mx = fmax(mx, fmax(fabs(entry(a, k, 0)), real ? 0.0 : fabs(entry(a, k, 1))));
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) {
+      const int ex = mx > 0.0 ? ilogb(mx) + 1 : 0;
+      rowexp[a] = ex;
+      rowscale[c * T * 16 + a] = scalbnf(mx > 0.0 ? 1.f : 0.f, ex - 11);
+    }
+  }
+  __syncthreads();
+  const int64_t total = (int64_t)(real ? 1 : 2) * T * T * 32;
+  for (int64_t q = threadIdx.x; q < total; q += blockDim.x) {
+    const int64_t tile = q / 32;
+    const int ln = (int)(q % 32), kt = (int)(tile % T), mt = (int)(tile / T % T), part = (int)(tile / ((int64_t)T * T));
+    uint32_t d[4][DG_S];
+    for (int u = 0; u < 4; ++u) {   // registers of the fragment: rows + 8 (u & 1), columns + 8 (u >> 1)
+      const int a = 16 * mt + (ln >> 2) + 8 * (u & 1), k = 16 * kt + 2 * (ln & 3) + 8 * (u >> 1);
+      long long f[2];
+      for (int j = 0; j < 2; ++j) f[j] = __double2ll_rn(ldexp(entry(a, k + j, part), 54 - rowexp[a]));
+      digit_pairs(f[0], f[1], d[u]);
+    }
+    uint4* o = dig + c * stride + tile * (DG_S * 32) + ln;
+    for (int s = 0; s < DG_S; ++s) o[s * 32] = make_uint4(d[0][s], d[1][s], d[2][s], d[3][s]);
+  }
 }
 
 // 32-bit DOF list of the cells and, on a p level (tab), the slot table: local
@@ -380,13 +418,15 @@ static void cell_op_begin(SystemImpl& S, Level& F, const LevelPlan& lp, cudaStre
   D.cls = upload(A, lp.ocls, st);
   D.items = upload(A, lp.oitems, st);
   D.nitems = (int64_t)lp.oitems.size();
-  D.items16 = upload(A, lp.oitems16, st);
-  D.nitems16 = (int64_t)lp.oitems16.size();
   D.mem = upload(A, lp.omem, st);
   const bool cg = &F == &S.levels.back() && F.kind == 1 && !(S.op.flags & DPGMG_FLAG_CG_C128);
   D.W = A.arr<float2>((size_t)D.ncls * D.stride());
   if (cg) {
-    D.Wlo = A.arr<float2>((size_t)D.ncls * D.stride());
+    D.dgitems = upload(A, lp.dgitems, st);
+    D.ndgitems = (int64_t)lp.dgitems.size();
+    D.dig = A.arr<uint4>((size_t)(D.ncls * D.dgstride()));
+    D.dgrow = A.arr<float>((size_t)(D.ncls * D.tiles() * 16));
+    cell_op_df_init();
     D.ydf = A.arr<float4>((size_t)D.ncell * D.n);
     D.df_on = true;
   }
@@ -428,8 +468,14 @@ static void cell_op_matrices(SystemImpl& S, Level& F, const int64_t* rep, const 
   CellOpDev& D = F.A.cell;
   if (!D.W) return;
   k_cell_class<TE><<<(unsigned)D.ncls, 256, 0, st>>>(E, e0, ne, rep, D.idx, D.n, D.stride(), D.offU, pack_storage(S),
-                                                    D.W, D.Wlo, D.rflag);
+                                                    D.W, D.rflag);
   DPG_CHECK_LAUNCH();
+  if constexpr (sizeof(TE) == sizeof(double2))
+    if (D.dig) {   // finest level: E holds every cell's matrix
+      k_cell_digits<<<(unsigned)D.ncls, 256, D.tiles() * 16 * sizeof(int), st>>>(E, rep, D.idx, D.n, D.offU, D.rflag,
+                                                                               D.dig, D.dgstride(), D.dgrow);
+      DPG_CHECK_LAUNCH();
+    }
 }
 
 // Macro elements of one class (macro_classes) have the same matrices, bit for
@@ -1042,9 +1088,26 @@ static void plan_cell_classes(LevelPlan& lp, const std::vector<int32_t>& cells, 
   for (const auto& m : members) lp.orep.push_back(m[0]);
   auto size_of = [&](int64_t) { return (int64_t)n; };
   class_items(members, size_of, lp.omem, lp.oitems);
-  lp.omem.clear();
-  class_items(members, size_of, lp.omem, lp.oitems16, 16);
-  if (nI > 0) {
+  if (nI == 0) {   // CG operator by cells (the finest level's, which is a p level)
+    const int T = (n + 15) / 16;
+    // warps' shares (16 rows x 8 cells) per CTA: up to 28 (p = 3: every row of
+    // the cells, 158 us; 16 shares 165 us, which convert the cells' values
+    // twice), 8 where that leaves SMs without work
+    for (int share : {28, 8}) {
+      lp.dgitems.clear();
+      int m0 = 0;
+      for (const auto& m : members) {
+        for (int q = 0; q < (int)m.size(); q += 32) {
+          const int cnt = std::min(32, (int)m.size() - q), nt = share / ((cnt + 7) / 8);
+          for (int t = 0; t < T; t += nt) lp.dgitems.push_back(make_int4(m0 + q, cnt, t, std::min(nt, T - t)));
+        }
+        m0 += (int)m.size();
+      }
+      if (lp.dgitems.size() >= 200) break;
+    }
+    auto cost = [](const int4& t) { return (t.y + 7) / 8 * t.w; };
+    std::stable_sort(lp.dgitems.begin(), lp.dgitems.end(), [&](const int4& u, const int4& v) { return cost(u) > cost(v); });
+  } else {
     lp.omem.clear();
     class_items(members, size_of, lp.omem, lp.mcitems);   // outputs S
     auto in_of = [&](int64_t) { return (int64_t)nI; };

@@ -1461,6 +1461,10 @@ __global__ void k_scatter_add(const int32_t* __restrict__ idx, const C* __restri
   if (i < n) y[idx[i]] = Ops<C>::add(y[idx[i]], x[i]);
 }
 
+void cell_op_df_init() {
+  DPG_CUDA(cudaFuncSetAttribute(k_class_cell_dg, cudaFuncAttributeMaxDynamicSharedMemorySize, DG_SMEM));
+}
+
 void macro_op_setup(SystemImpl& S, Level& F, const LevelPlan& lp, cudaStream_t st) {
   if (lp.mbitems.empty() || !F.Y32) return;
   Alloc& A = S.mem;
@@ -2466,9 +2470,9 @@ void prepare_solve(SystemImpl& S, cudaStream_t st) {
       const TuneKey key{2, F.mesh.p, F.kind, log2i(n)};
       auto run = [&](int G) { spmv_df_g(Acg, W.xh, W.xl, nullptr, W.q, 0, G, st); };
       Acg.gsel[2] = pick_group(key, ev, st, run, Acg.rent != nullptr, true);
-      if (Acg.cell.Wlo) {
+      if (Acg.cell.dig) {
         TuneKey ck = key;
-        ck.kind += 16 * (1 + log2i(Acg.cell.nitems16));
+        ck.kind += 16 * (1 + log2i(Acg.cell.ndgitems));
         Acg.cell.df_on = pick_variant(ck, ev, st, {SPMV_CELLS, Acg.gsel[2]}, run) == SPMV_CELLS;
       }
     }
