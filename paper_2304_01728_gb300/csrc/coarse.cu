@@ -613,7 +613,7 @@ void coarse_setup(SystemImpl& S, Level& C0, int* info, cudaStream_t st, Alloc& A
 }
 
 // ------------------------------------------------------------------ apply
-// One warp per row pair (i, N-1-i): every warp reads N+1 entries.  Four
+// One warp per row pair (i, N-1-i): every warp reads N+1 entries.  Eight
 // streaming loads per lane per step keep enough bytes in flight; the two
 // accumulators take the entries in the same order as a two-load loop (a0:
 // t, t + 64, ...; a1: t + 32, t + 96, ...), so the result is bitwise that
@@ -623,6 +623,16 @@ __device__ __forceinline__ C dot_row(const C* __restrict__ row, const C* __restr
   using O = Ops<C>;
   C a0 = O::zero(), a1 = O::zero();
   int64_t t = lane;
+  for (; t + 224 < len; t += 256) {
+    C m[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) m[k] = __ldcs(row + t + 32 * k);
+#pragma unroll
+    for (int k = 0; k < 8; k += 2) {
+      a0 = O::fma(m[k], v[t + 32 * k], a0);
+      a1 = O::fma(m[k + 1], v[t + 32 * k + 32], a1);
+    }
+  }
   for (; t + 96 < len; t += 128) {
     const C m0 = __ldcs(row + t), m1 = __ldcs(row + t + 32), m2 = __ldcs(row + t + 64), m3 = __ldcs(row + t + 96);
     a0 = O::fma(m0, v[t], a0);
@@ -662,13 +672,16 @@ __global__ void __launch_bounds__(256) k_trmv_upper(const C* __restrict__ Up, in
   const int64_t half = (N + 1) / 2;
   const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); w < half; w += nw) {
+    // the short row first: warps that begin with long rows of nearly the same
+    // length run through memory in step (9,777 unknowns, complex64, 382 MB: 72
+    // us; long rows first and four loads a lane, 84 us)
     const int64_t j1 = w, j2 = N - 1 - w;
-    C s1 = dot_row<C>(Up + j1 * N - j1 * (j1 - 1) / 2, y + j1, N - j1, lane);
-    if (lane == 0) e[j1] = s1;
     if (j2 != j1) {
       C s2 = dot_row<C>(Up + j2 * N - j2 * (j2 - 1) / 2, y + j2, N - j2, lane);
       if (lane == 0) e[j2] = s2;
     }
+    C s1 = dot_row<C>(Up + j1 * N - j1 * (j1 - 1) / 2, y + j1, N - j1, lane);
+    if (lane == 0) e[j1] = s1;
   }
 }
 
