@@ -316,7 +316,7 @@ static __global__ void k_cell_sum_df(const int32_t* __restrict__ tab, const int6
     df_add(rh, rl, v.x, v.y);
     df_add(ih, il, v.z, v.w);
   });
-  const double re = (double)rh + (double)rl, im = (double)ih + (double)il;
+  const double re = wide(rh) + wide(rl), im = wide(ih) + wide(il);
   y[g] = mode ? make_double2(b[g].x - re, b[g].y - im) : make_double2(re, im);
 }
 

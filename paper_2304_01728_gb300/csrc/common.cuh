@@ -204,6 +204,36 @@ __device__ __forceinline__ int fx_col(int t, int c) { return t * TL + (BT ? c ^ 
 template <bool AT>
 __device__ __forceinline__ int fx_row(int r, int t) { return r * NB + (AT ? t ^ (r & ~1) : t); }
 
+// Conversions between float and double by bits: the conversion instructions run
+// on the FP64 pipe (1.7 lanes a clock and SM), these on the integer pipe.
+
+// f as a double, exact
+__device__ __forceinline__ double wide(float f) {
+  const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+  if (a - 0x00800000u < 0x7f000000u)   // normal: the exponent's bias grows by 896
+    return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(u << 29));
+  return a == 0 ? __hiloint2double((int)u, 0) : (double)f;
+}
+__device__ __forceinline__ double wide(double f) { return f; }
+
+// v as (high, low): high is v rounded to 24 bits, low the rest rounded to 24
+__device__ __forceinline__ float2 split_float(double v) {
+  const int hi = __double2hiint(v), e = (hi >> 20) & 0x7ff;
+  if ((unsigned)(e - (1023 - 70)) > 170u) {   // zero, small, large, not finite
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
+  }
+  const unsigned lo = (unsigned)__double2loint(v);
+  const long long m = ((long long)((hi & 0xfffff) | 0x100000) << 32) | lo;
+  int t = (int)((m + (1ll << 28)) >> 29);   // 2^23 .. 2^24
+  int r = (int)(m - ((long long)t << 29));  // -2^28 .. 2^28
+  if (hi < 0) {
+    t = -t;
+    r = -r;
+  }
+  return make_float2((float)t * __int_as_float((e - 1046 + 127) << 23), (float)r * __int_as_float((e - 1075 + 127) << 23));
+}
+
 template <class T> struct IsFp64 { static constexpr bool v = false; };
 template <> struct IsFp64<double> { static constexpr bool v = true; };
 template <> struct IsFp64<double2> { static constexpr bool v = true; };

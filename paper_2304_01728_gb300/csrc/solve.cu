@@ -896,9 +896,9 @@ __global__ void k_split_vec(const double2* __restrict__ x, float2* __restrict__ 
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double2 v = x[i];
-  const float hx = (float)v.x, hy = (float)v.y;
-  xh[i] = make_float2(hx, hy);
-  xl[i] = make_float2((float)(v.x - (double)hx), (float)(v.y - (double)hy));
+  const float2 sx = split_float(v.x), sy = split_float(v.y);
+  xh[i] = make_float2(sx.x, sy.x);
+  xl[i] = make_float2(sx.y, sy.y);
 }
 
 __global__ void k_split_vals(const double2* __restrict__ v, float2* __restrict__ vh, float2* __restrict__ vl,
@@ -1517,20 +1517,29 @@ static unsigned red_blocks(int64_t n) { return (unsigned)std::max<int64_t>(1, st
 // scalar slots of the CG state
 enum { SC_RHO = 0, SC_PQ, SC_ALPHA, SC_BETA, SC_RR, SC_RHONEW, SC_COUNT };
 
+// Sum of acc over a block of 256 threads (the result in warp 0).  Eight values
+// per lane of one warp, then its lanes: 24 warp additions on the FP64 pipe (1.7
+// lanes a clock and SM), where a shuffle tree in every warp took 94.
+__device__ __forceinline__ double2 block_sum(double2 acc) {
+  __shared__ double2 sh[256];
+  sh[threadIdx.x] = acc;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int k = 1; k < 8; ++k) acc = Ops<double2>::add(acc, sh[threadIdx.x + 32 * k]);
+    acc = warp_sum(acc);
+  }
+  return acc;
+}
+
 // which: 0 -> PQ then ALPHA = RHO / PQ ; 1 -> RR ; 2 -> RHONEW, BETA, RHO ; 3 -> RHO
 // (one block of 256 threads; the partials are read from L2: other SMs wrote them)
 __device__ void block_finish(const double2* part, int nparts, double2* sc, int which) {
-  __shared__ double2 sh[256];
   double2 acc = make_double2(0, 0);
   for (int k = threadIdx.x; k < nparts; k += blockDim.x) acc = Ops<double2>::add(acc, __ldcg(part + k));
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) sh[threadIdx.x] = Ops<double2>::add(sh[threadIdx.x], sh[threadIdx.x + s]);
-    __syncthreads();
-  }
+  __syncthreads();   // block_sum's buffer may still be read (the block's own partial)
+  const double2 d = block_sum(acc);
   if (threadIdx.x != 0) return;
-  double2 d = sh[0];
   if (which == 0) {
     sc[SC_PQ] = d;
     double2 rho = sc[SC_RHO];
@@ -1569,25 +1578,18 @@ __device__ __forceinline__ bool last_block(unsigned* ticket) {
 }
 
 __device__ __forceinline__ double2 to_c128(double2 a) { return a; }
-__device__ __forceinline__ double2 to_c128(float2 a) { return make_double2(a.x, a.y); }   // exact
+__device__ __forceinline__ double2 to_c128(float2 a) { return make_double2(wide(a.x), wide(a.y)); }   // exact
 
 // sum conj(u_i) v_i in FP64 (u complex128, or complex64 widened exactly): block
 // partials, finished by the last block
 template <class TU>
 __global__ void k_dot_fused(const TU* __restrict__ u, const double2* __restrict__ v, int64_t n,
                             double2* __restrict__ part, double2* sc, int which, unsigned* ticket) {
-  __shared__ double2 sh[8];
   double2 acc = make_double2(0, 0);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     acc = Ops<double2>::fmac(v[i], to_c128(u[i]), acc);
-  acc = warp_sum(acc);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double2 s = make_double2(0, 0);
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s = Ops<double2>::add(s, sh[k]);
-    part[blockIdx.x] = s;
-  }
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) part[blockIdx.x] = acc;
   if (!last_block(ticket)) return;
   block_finish(part, gridDim.x, sc, which);
   if (threadIdx.x == 0) *ticket = 0u;
@@ -1598,7 +1600,6 @@ __global__ void k_dot_fused(const TU* __restrict__ u, const double2* __restrict_
 __global__ void k_cg_update_fused(double2* __restrict__ x, double2* __restrict__ r, const double2* __restrict__ p,
                                   const double2* __restrict__ q, double2* sc, int64_t n, double2* __restrict__ part,
                                   unsigned* ticket, float2* __restrict__ r32) {
-  __shared__ double2 sh[8];
   const double2 al = sc[SC_ALPHA];
   double acc = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -1612,14 +1613,8 @@ __global__ void k_cg_update_fused(double2* __restrict__ x, double2* __restrict__
     if (r32) r32[i] = make_float2((float)ri.x, (float)ri.y);
     acc += ri.x * ri.x + ri.y * ri.y;
   }
-  double2 a2 = warp_sum(make_double2(acc, 0.0));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a2;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double2 s = make_double2(0, 0);
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s = Ops<double2>::add(s, sh[k]);
-    part[blockIdx.x] = s;
-  }
+  const double2 a2 = block_sum(make_double2(acc, 0.0));
+  if (threadIdx.x == 0) part[blockIdx.x] = a2;
   if (!last_block(ticket)) return;
   block_finish(part, gridDim.x, sc, 1);
   if (threadIdx.x == 0) *ticket = 0u;
@@ -1635,9 +1630,9 @@ __global__ void k_cg_dir(double2* __restrict__ p, const TZ* __restrict__ z, cons
     double2 pi = p[i], zi = to_c128(z[i]);
     const double2 v = make_double2(zi.x + be.x * pi.x - be.y * pi.y, zi.y + be.x * pi.y + be.y * pi.x);
     p[i] = v;
-    const float hx = (float)v.x, hy = (float)v.y;
-    ph[i] = make_float2(hx, hy);
-    pl[i] = make_float2((float)(v.x - (double)hx), (float)(v.y - (double)hy));
+    const float2 sx = split_float(v.x), sy = split_float(v.y);
+    ph[i] = make_float2(sx.x, sy.x);
+    pl[i] = make_float2(sx.y, sy.y);
   }
 }
 
@@ -1655,18 +1650,11 @@ __global__ void k_dot_fused_blk(const TU* __restrict__ u, const double2* __restr
   v += (int64_t)k * n;
   part += (int64_t)k * RED_BLOCKS;
   sc += (int64_t)k * SC_COUNT;
-  __shared__ double2 sh[8];
   double2 acc = make_double2(0, 0);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     acc = Ops<double2>::fmac(v[i], to_c128(u[i]), acc);
-  acc = warp_sum(acc);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double2 s = make_double2(0, 0);
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) s = Ops<double2>::add(s, sh[q]);
-    part[blockIdx.x] = s;
-  }
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) part[blockIdx.x] = acc;
   if (!last_block(ticket + k)) return;
   block_finish(part, gridDim.x, sc, which);
   if (threadIdx.x == 0) ticket[k] = 0u;
@@ -1684,7 +1672,6 @@ __global__ void k_cg_update_fused_blk(double2* __restrict__ x, double2* __restri
   q += o;
   sc += (int64_t)k * SC_COUNT;
   part += (int64_t)k * RED_BLOCKS;
-  __shared__ double2 sh[8];
   const double2 al = sc[SC_ALPHA];
   double acc = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -1697,14 +1684,8 @@ __global__ void k_cg_update_fused_blk(double2* __restrict__ x, double2* __restri
     r[i] = ri;
     acc += ri.x * ri.x + ri.y * ri.y;
   }
-  double2 a2 = warp_sum(make_double2(acc, 0.0));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a2;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double2 s = make_double2(0, 0);
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s = Ops<double2>::add(s, sh[w]);
-    part[blockIdx.x] = s;
-  }
+  const double2 a2 = block_sum(make_double2(acc, 0.0));
+  if (threadIdx.x == 0) part[blockIdx.x] = a2;
   if (!last_block(ticket + k)) return;
   block_finish(part, gridDim.x, sc, 1);
   if (threadIdx.x == 0) ticket[k] = 0u;
@@ -2833,21 +2814,14 @@ __global__ void k_start_vector(C* x, int64_t n, const int64_t* slot_ptr) {
 // partial[b] = sum conj(u_i) v_i (accumulated in FP64 whatever the vector precision)
 template <class C>
 __global__ void k_dot_partial_t(const C* __restrict__ u, const C* __restrict__ v, int64_t n, double2* __restrict__ part) {
-  __shared__ double2 sh[8];
   double2 acc = make_double2(0, 0);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double ux = u[i].x, uy = u[i].y, vx = v[i].x, vy = v[i].y;
+    const double ux = wide(u[i].x), uy = wide(u[i].y), vx = wide(v[i].x), vy = wide(v[i].y);
     acc.x += ux * vx + uy * vy;
     acc.y += ux * vy - uy * vx;
   }
-  acc = warp_sum(acc);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double2 s2 = make_double2(0, 0);
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s2 = Ops<double2>::add(s2, sh[k]);
-    part[blockIdx.x] = s2;
-  }
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
 template <class C>
