@@ -400,10 +400,22 @@ __global__ void k_cell_index(const int64_t* __restrict__ dofs, const uint8_t* __
   if (tab && g >= 0) tab[cell_row(g, offE, offF) + code[q % n]] = (int32_t)q;
 }
 
+// Bytes a level's class operators may take: the admission bound counts a block
+// for every patch, and the shared ones leave room; 16 MB (of the bound's
+// constant part) also where patches share little.
+static int64_t class_room(const LevelPlan& lp) {
+  return std::max((lp.sum_sq - lp.uniq_sq) * (int64_t)sizeof(float2), (int64_t)16 << 20);
+}
+
 // Index data and storage of a level's operator by cells; the matrices follow
 // (k_cell_class).
 static void cell_op_begin(SystemImpl& S, Level& F, const LevelPlan& lp, cudaStream_t st) {
   if (lp.ocls.empty()) return;   // mixed path only (plan_host)
+  {
+    const int64_t n = F.kind == 2 ? F.nS : F.nloc, nI = F.kind == 2 ? F.nI : 0, nc = (int64_t)lp.orep.size();
+    const int64_t cells = (int64_t)lp.ocls.size() * (n * 20 + nI * 4);   // lists, slots, cell products
+    if (cells + nc * (n * n + nI * (nI + 2 * n)) * 9 > class_room(lp)) return;
+  }
   Alloc& A = S.mem;
   CellOpDev& D = F.A.cell;
   const bool macro = F.kind == 2;
@@ -421,7 +433,8 @@ static void cell_op_begin(SystemImpl& S, Level& F, const LevelPlan& lp, cudaStre
   D.mem = upload(A, lp.omem, st);
   const bool cg = &F == &S.levels.back() && F.kind == 1 && !(S.op.flags & DPGMG_FLAG_CG_C128);
   D.W = A.arr<float2>((size_t)D.ncls * D.stride());
-  if (cg) {
+  const int64_t dg = D.ncls * D.dgstride() * (int64_t)sizeof(uint4) + D.ncell * D.n * (int64_t)sizeof(float4);
+  if (cg && dg + D.ncls * D.stride() * 8 + D.ncell * D.n * 20 <= class_room(lp)) {
     D.dgitems = upload(A, lp.dgitems, st);
     D.ndgitems = (int64_t)lp.dgitems.size();
     D.dig = A.arr<uint4>((size_t)(D.ncls * D.dgstride()));
@@ -998,9 +1011,11 @@ static bool smooth_coarsest(const SystemImpl& S) {
 // windows hold every patch's own block).
 static bool share_patches(const SystemImpl& S) { return !(S.op.flags & DPGMG_FLAG_RECOMPUTE_PATCHES); }
 
-// The class product pays when the blocks are shared by at least
-// CLS_MIN_SHARE patches on average (by entries); below that the streaming
-// product, which keeps more of a block's bytes in flight, reads them.
+// The class product is planned when the blocks are shared by at least
+// CLS_MIN_SHARE patches on average (by entries); below that it reads as many
+// bytes as the streaming product, which keeps more of them in flight.  Above,
+// setup times both: many patches gain (18,513 patches, 451 -> 92 us), a level
+// with few items loses (405 macro patches of up to 488 DOFs: 24 us streamed).
 constexpr double CLS_MIN_SHARE = 2.0;
 
 // Work items of a class product: mem lists the members class by class, items

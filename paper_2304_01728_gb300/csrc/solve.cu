@@ -1466,7 +1466,7 @@ void cell_op_df_init() {
 }
 
 void macro_op_setup(SystemImpl& S, Level& F, const LevelPlan& lp, cudaStream_t st) {
-  if (lp.mbitems.empty() || !F.Y32) return;
+  if (lp.mbitems.empty() || !F.Y32 || !F.A.cell.cls) return;
   Alloc& A = S.mem;
   MacroOpDev& D = F.mop;
   D.nI = F.nI;
