@@ -547,15 +547,16 @@ def run_gb300(args, rank, world, local_rank):
         "config": {"workload": w["name"], "n": list(w["problem"]["n"]), "p": w["problem"]["p"],
                    "omega": w["problem"]["omega"], "levels": w["opts"]["n_levels"], "precision": args.precision,
                    "n_dof": n_dof, "parallelism": "replicas" if world > 1 else "single GPU",
-                   "l2": "operators (GBs) exceed L2; no flush needed"},
+                   "l2": "the solve's matrices and vectors exceed L2; no flush needed"},
         "iters": it_last[0], "pcg_ms": pcg_ms / args.steps, "setup_ms": sum(s[2] for s in stats) / args.steps,
         "true_relres": it_last[3], "relres": it_last[4], "bytes_per_iter": it_last[5],
         "pcg_GBps": it_last[5] * it_last[0] / (stats[-1][1] / 1e3) / 1e9,
         "gpu_launches": int(launches),
-        "roofline": {"kernel": "k_patch_apply (finest smoother)", "bound": "hbm", "achieved": achieved,
+        "roofline": {"kernel": "finest smoother product (k_class_apply where patches share blocks, then bound by "
+                               "the FP32 pipe and not by these bytes; else k_patch_apply)", "bound": "hbm", "achieved": achieved,
                      "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_source": peak_kind,
                      "bytes_per_launch": prof_b, "launches": prof_n, "avg_launch_ms": per_launch_ms,
-                     "bytes_rule": "stored patch-inverse entries read once: 8 B per complex64 entry, 4 B per "
+                     "bytes_rule": "distinct stored patch-inverse entries read once: 8 B per complex64 entry, 4 B per "
                                    "entry of a real packed block",
                      "real_packed_fraction_of_entries": (patch_store["real_sq"] / patch_store["sum_patch_sq"]
                                                          if patch_store.get("sum_patch_sq") else None),

@@ -215,7 +215,7 @@ typedef struct dpgmg_stats {
   double true_relres;      /* ||b - A x|| / ||b|| recomputed at exit (FP64) */
   double t_setup_ms;       /* device time of dpgmg_setup */
   double t_pcg_ms;         /* device time from the first CG step to convergence */
-  long long bytes_per_iter;/* algorithmic bytes of one CG iteration (matrix entries read once) */
+  long long bytes_per_iter;/* algorithmic bytes of one CG iteration (distinct matrix entries read once) */
   long long n_dof;         /* finest trace DOFs */
   long long dev_bytes_peak;/* peak device bytes held by the system */
 } dpgmg_stats;
@@ -230,8 +230,9 @@ typedef struct dpgmg_level_desc {
   long long sum_patch_sq;  /* sum of squared patch sizes */
   long long op_nnz;        /* stored entries of the level's smoothing operator */
   double theta;
-  long long patch_stored;  /* stored patch-inverse entries (sum n_j^2, or sum n_j(n_j+1)/2 in
-                              Hermitian half storage) */
+  long long patch_stored;  /* stored patch-inverse entries: sum of n_j^2 over the distinct blocks
+                              (patches with the same surroundings share one), rows padded to even
+                              length, or sum n_j(n_j+1)/2 in Hermitian half storage */
   long long patch_real_sq; /* sum of n_j^2 over the patches whose inverses are stored as real
                               blocks (mixed path, see DPGMG_FLAG_COMPLEX_STORAGE): half the bytes */
   long long op_real_nnz;   /* entries of the level's complex64 operator stored as reals (the same) */
@@ -401,7 +402,10 @@ long long dpgmg_launch_count(void);
  * feed, or (G = 32) by one warp per row with the warp's stream of values and
  * column indices copied 8 steps ahead into shared memory by asynchronous
  * copies (cp.async), or (G = 64, V-cycle operators only) by one half-warp
- * per row, two rows of a warp at a time.  dpgmg_setup times every variant on each operator and
+ * per row, two rows of a warp at a time.  Where the cells of a level share
+ * matrices (mixed path, uniform parts of the medium), setup also times the
+ * product cell by cell, which has no code here; an override selects the
+ * assembled rows instead.  dpgmg_setup times every variant on each operator and
  * keeps the fastest; choices are cached per (product type, p, level kind,
  * log2 of the row count) for the life of the process.  level >= 1 addresses
  * that level's V-cycle operator, level == -1 the CG operator.  set = 1, 2, 4,
