@@ -1,8 +1,8 @@
 // Operators by cells: y = sum_K R_K^T A_K R_K x with one stored matrix per cell
 // class (classes.cuh), for the V-cycle residual (complex64) and the CG operator
-// (double-float).  The assembled rows stream every stored entry from HBM once
-// per product; here a class's matrix stays in L2 and shared memory for all its
-// cells, so the FP32 pipe and the gathers set the time.
+// (fixed point on the tensor cores).  The assembled rows stream every stored
+// entry from HBM once per product; here a class's matrix stays in L2 and shared
+// memory for all its cells, so the arithmetic and the gathers set the time.
 #pragma once
 #include "classes.cuh"
 #include "digits.cuh"

@@ -56,16 +56,17 @@ template <class T, class AL> T* upload(Alloc& A, const std::vector<T, AL>& h, cu
   return d;
 }
 
+constexpr int DG_S = 7;        // 8-bit digits of a fixed-point operand of the CG operator by cells
+constexpr int DG_KC = 112;     // columns per exact accumulation: DG_S DG_KC 2^14 < 2^24
+
 // ----------------------------------------------------------- device structs
 // An operator as a sum over its cells, y = sum_K R_K^T A_K R_K x, with one
 // stored matrix per cell class (classes.cuh): the elements of a p level, the
 // macro elements of an h level.  Kept beside the assembled rows when the cells
 // are many per class.
-constexpr int DG_S = 7;        // 8-bit digits of a fixed-point operand of the CG operator by cells
-constexpr int DG_KC = 112;     // columns per exact accumulation: DG_S DG_KC 2^14 < 2^24
 struct CellOpDev {
   bool on = false;             // applied in place of the assembled rows (complex64 V-cycle operator)
-  bool df_on = false;          // the same for the double-float CG operator
+  bool df_on = false;          // the same for the CG operator (digits)
   int n = 0;                   // local DOFs of a cell
   int64_t ncell = 0, ndof = 0, ncls = 0;
   int32_t* idx = nullptr;      // [ncell][n] DOF, or -1
@@ -89,7 +90,7 @@ struct CellOpDev {
   int32_t* slots = nullptr;
   int64_t offE = 0, offF = 0, offU = 0;
   float2* ybuf = nullptr;      // [ncell][n] cell products
-  float4* ydf = nullptr;       // the same in double-float (CG operator only)
+  float4* ydf = nullptr;       // the same as FP32 high and low parts (CG operator only)
   int64_t stride() const { return n * patch_ld(n); }   // entries per class matrix
   int64_t tiles() const { return (n + 15) / 16; }
   int64_t dgstride() const { return 2 * tiles() * tiles() * DG_S * 32; }
