@@ -139,61 +139,118 @@ struct Team {
 // ------------------------------------------------- 32 x 32 x 32 tile products
 // acc[q] += sum_t A[r][t] B[t][c] for the thread's outputs r = w + 8 q, c = lane
 // (warp w of 8, q < 4), the inner step of every blocked routine below.  The
-// operands come in registers: a[i] = A[4 w + i][lane], and b[i] = B[4 w + i][lane];
-// with BT, b[i] = B[lane][4 w + i] (rows of the transpose).  At, Bt: TL x NB
-// elements of shared memory each.  All 256 threads call it; it synchronises
-// before it writes shared memory and before it reads it.
+// operands come in registers: a[i] = A[4 w + i][lane], with AT a[i] = A[lane][4 w + i];
+// b[i] = B[4 w + i][lane], with BT b[i] = B[lane][4 w + i] (rows of the transpose).
+// At, Bt: TL x NB elements of shared memory each, Z: NB x NB (FP64 types only),
+// all on 16-byte boundaries.  All 256 threads call it; it synchronises before it
+// writes shared memory and before it reads it.
 //
 // FP32 types: FMA chains in increasing t, continued from acc.
 //
 // FP64 types: this GPU's FP64 pipe runs 1.7 FMAs per clock and SM, its integer
 // pipe 59 32 x 32 -> 64-bit multiply-adds.  A row of A and a column of B are
-// taken as fixed-point numbers with the exponent of their largest entry, 57
-// bits each in two 28-bit limbs, and multiplied exactly on the integer pipe:
-// hi hi, and hi lo + lo hi in a second 64-bit sum (lo lo is below 2^-58 of the
-// largest product and dropped), three multiply-adds per product.  |hi| <= 2^28
-// and |lo| <= 2^27, so 64 products (32 complex ones) stay below 2^62.  The sum
-// is rounded once per chunk.  Element matrices of random (p, h, omega, c), p = 1
-// to 4, carry the same error against 128-bit arithmetic as with FP64 FMA chains
-// (geometric means of the two within 7%, either way; unchanged with 60-bit
-// operands, so what is left comes from the FP64 panels).  Tiles with an
-// infinity, a NaN or an exponent at the top of the range take the FP64 chain.
-// Measured (GB300): element stage of 800 elements of order 3 with distinct
-// wavespeeds 88 -> 45 ms, 64 of order 5 1,107 -> 174 ms; complex128 setup on
-// 8^3 p = 3 78 -> 50 ms.
+// taken as fixed-point numbers with the exponent of their largest entry, 82
+// bits each in limbs of 26, 28 and 28 bits, and the products of limbs down to
+// 2^-56 of the largest (six of nine) are summed exactly in three 64-bit sums:
+// |hi| <= 2^26, |mid|, |lo| <= 2^27, so the 64 products of a complex chunk stay
+// below 2^62.  The sum is rounded once per chunk.
+//
+// Error: absolute, below 2^-74 max_t |A[r][t]| max_t |B[t][c]|, beside the
+// final rounding.  An FMA chain's error is 2^-53 times the sum of |A[r][t] B[t][c]|,
+// so the result is the more exact one wherever that sum exceeds 2^-21 of the
+// product of the maxima.  Scaling the rows of A or the columns of B changes
+// neither.  Scaling the inner index (the columns of A against the rows of B)
+// does: triangular solves with L^H and products with a solution meet it, where
+// the operands carry inverse scales of the unknowns.  With BAL column t of A and
+// row t of B are first shifted by powers of two (on the exponents, exact) to
+// equal maxima, which takes the product of the maxima to its smallest value.
+//
+// With two limbs (57 bits) the element matrices were as exact as with FMA
+// chains, but not the recovery blocks on boxes far from a cube: 9 times the
+// error on a 1/8 x 1/100 x 1/1000 element of order 2; with three 1.0 times.
+// Over p = 1 to 5, elements from 1e-4 to 125 wide and 1:125 flat ones, rows
+// scaled to unit diagonal, the errors against 128-bit arithmetic are 0.3 to 1.2
+// times those of FMA chains in element matrices, in the mean and at the worst
+// entry.  Tiles with an infinity, a NaN or an exponent at the top of the range
+// take the FP64 chain.
+//
+// Bound: the integer pipe.  Measured (GB300; FP64 chains, two limbs, three): element
+// stage of 800 elements of order 3 with distinct wavespeeds 88, 46, 60 ms, of 64
+// of order 5 1,104, 163, 211 ms; patch inversion of 8^3, p = 3, complex128 57, 27,
+// 31 ms.  The inner loops are unrolled by two steps: by four the kernels spill.
 __device__ __forceinline__ int fx_exponent(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 __device__ __forceinline__ int fx_exponent(double2 v) { return max(fx_exponent(v.x), fx_exponent(v.y)); }
 
-// round(v 2^(1078 - E)) for a biased exponent E >= v's: |v| < 2^(E - 1022) maps below 2^56 (zero and
-// denormals to 0); hi, lo: limbs with v = hi 2^28 + lo
-__device__ __forceinline__ void fx_limbs(double v, int E, int& hi, int& lo) {
+constexpr int FX_NONE = -100000;   // exponent of an all-zero row, column or entry
+
+// round(v 2^(1104 - E)) for an exponent E >= v's biased one + sft (v is taken as v 2^sft): |f| < 2^82, as
+// f = l.x 2^56 + l.y 2^28 + l.z (zero and denormals give 0)
+__device__ __forceinline__ int3 fx_limbs(double v, int sft, int E) {
   const int e = fx_exponent(v);
-  const int sh = E - e - 3;   // shift right (left when negative) of the 53-bit mantissa
+  const int sh = E - e - sft - 29;   // shift right (left when negative) of the 53-bit mantissa
   const long long m = ((long long)((__double2hiint(v) & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
-  long long f = 0;
-  if (e != 0 && sh < 60) f = sh <= 0 ? m << -sh : (m + (1ll << (sh - 1))) >> sh;
-  if (__double2hiint(v) < 0) f = -f;
-  hi = (int)((f + (1ll << 27)) >> 28);
-  lo = (int)(f - ((long long)hi << 28));
+  if (e == 0 || sh > 60) return make_int3(0, 0, 0);
+  long long g;   // f's bits from 28 on
+  int lo;        // and the 28 below
+  if (sh <= 0) {
+    g = sh <= -28 ? m << (-28 - sh) : m >> (28 + sh);
+    lo = (int)((unsigned)m << -sh) & 0xfffffff;
+  } else {
+    const long long f = (m + (1ll << (sh - 1))) >> sh;
+    g = f >> 28;
+    lo = (int)f & 0xfffffff;
+  }
+  if (lo >= 1 << 27) {
+    lo -= 1 << 28;
+    ++g;
+  }
+  const int hi = (int)((g + (1ll << 27)) >> 28);
+  const int mid = (int)(g - ((long long)hi << 28));
+  return __double2hiint(v) < 0 ? make_int3(-hi, -mid, -lo) : make_int3(hi, mid, lo);
 }
 
-// 2^k t, rounded once
-__device__ __forceinline__ double fx_value(long long hh, long long x, int k) {
-  const double t = (double)(hh + ((x + (1ll << 27)) >> 28));
-  if (k >= -1000 && k <= 960) return t * __hiloint2double((k + 1023) << 20, 0);
-  return ldexp(t, k);
+// 2^(k - 56) (h 2^56 + x 2^28 + y), rounded once (on the integer pipe)
+__device__ __forceinline__ double fx_value(long long h, long long x, long long y, int k) {
+  constexpr long long M56 = (1ll << 56) - 1;
+  long long a = y + ((x & 0xfffffff) << 28);
+  h += x >> 28;
+  h += a >> 56;
+  a &= M56;
+  const bool neg = h < 0;
+  if (neg) {
+    h = -h - (a != 0);
+    a = (1ll << 56) - a & M56;
+  }
+  unsigned long long t;   // leading bit at 63
+  int q;                  // value = t 2^(q + k - 56)
+  if (h != 0) {
+    const int z = __clzll(h);
+    q = 56 - z;
+    t = z <= 56 ? ((unsigned long long)h << z) | ((unsigned long long)a >> q)
+                : (((unsigned long long)h << 56) | (unsigned long long)a) << (z - 56);
+  } else {
+    if (a == 0) return 0.0;
+    const int z = __clzll(a);
+    q = -z;
+    t = (unsigned long long)a << z;
+  }
+  const long long mant = (long long)(t >> 11) + ((t >> 10) & 1);   // 2^52 .. 2^53
+  const int e = q + k - 56 + 63 + 1023;
+  const long long sign = neg ? (long long)0x8000000000000000ull : 0;
+  if (e >= 1 && e < 2046) return __longlong_as_double(sign | (((long long)(e - 1) << 52) + mant));
+  return ldexp(__longlong_as_double(sign | ((1022ll << 52) + mant)), e - 1023);
 }
 
-__device__ __forceinline__ void fx_store(double* p, double v, int E) {
-  int2 f;
-  fx_limbs(v, E, f.x, f.y);
-  *reinterpret_cast<int2*>(p) = f;
+// limbs of an entry: high and middle ones in a tile, low ones in Z
+__device__ __forceinline__ void fx_store(double* p, int* z, double v, int sft, int E) {
+  const int3 f = fx_limbs(v, sft, E);
+  *reinterpret_cast<int2*>(p) = make_int2(f.x, f.y);
+  *z = f.z;
 }
-__device__ __forceinline__ void fx_store(double2* p, double2 v, int E) {
-  int4 f;
-  fx_limbs(v.x, E, f.x, f.y);
-  fx_limbs(v.y, E, f.z, f.w);
-  *reinterpret_cast<int4*>(p) = f;
+__device__ __forceinline__ void fx_store(double2* p, int2* z, double2 v, int sft, int E) {
+  const int3 f = fx_limbs(v.x, sft, E), g = fx_limbs(v.y, sft, E);
+  *reinterpret_cast<int4*>(p) = make_int4(f.x, f.y, g.x, g.y);
+  *z = make_int2(f.z, g.z);
 }
 
 // column c of row t of Bt: swizzled with BT, so that stores along t do not conflict
@@ -237,9 +294,11 @@ __device__ __forceinline__ float2 split_float(double v) {
 template <class T> struct IsFp64 { static constexpr bool v = false; };
 template <> struct IsFp64<double> { static constexpr bool v = true; };
 template <> struct IsFp64<double2> { static constexpr bool v = true; };
+template <class T> struct FxLow { typedef int V; };
+template <> struct FxLow<double2> { typedef int2 V; };
 
-template <class T, bool BT, bool AT = false>
-__device__ void tile_product(const T a[4], const T b[4], T* At, T* Bt, int kb, T acc[4]) {
+template <class T, bool BT, bool AT = false, bool BAL = false>
+__device__ void tile_product(const T a[4], const T b[4], T* At, T* Bt, T* Z, int kb, T acc[4]) {
   using O = Ops<T>;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   // place of a[i] and b[i]
@@ -264,20 +323,63 @@ __device__ void tile_product(const T a[4], const T b[4], T* At, T* Bt, int kb, T
     __syncthreads();   // the last product's readers are done
     plain();
   } else {
-    __shared__ int s_ea[TL], s_eb[TL], s_pa[8][TL], s_pb[8][TL];
-    int ea[4], eb[4], ma = 0, mb = 0;
+    static_assert(!(BT && BAL), "balancing reads rows of B along the lanes");
+    using Low = typename FxLow<T>::V;
+    Low* Za = reinterpret_cast<Low*>(Z);   // low limbs, places as At and Bt
+    Low* Zb = Za + TL * NB;
+    __shared__ int s_ea[TL], s_eb[TL], s_pa[8][TL], s_pb[8][TL], s_pt[8][TL], s_tb[NB];
+    int ea[4], eb[4], sa[4] = {0, 0, 0, 0}, sb[4] = {0, 0, 0, 0}, top = 0;   // exponents and shifts of a[i], b[i]
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       ea[i] = fx_exponent(a[i]);
       eb[i] = fx_exponent(b[i]);
+      top = max(top, max(ea[i], eb[i]));
+      if (ea[i] == 0) ea[i] = FX_NONE;
+      if (eb[i] == 0) eb[i] = FX_NONE;
+    }
+    if (__syncthreads_or(top >= 0x7fe)) {   // uniform over the CTA; also: the last product's readers are done
+      plain();
+      return;
+    }
+    if constexpr (BAL) {
+      auto shift = [](int u, int v) { return u == FX_NONE || v == FX_NONE ? 0 : (v - u) >> 1; };
+      int tb[4];   // largest exponent of row t = 4 w + i of B
+#pragma unroll
+      for (int i = 0; i < 4; ++i) tb[i] = __reduce_max_sync(0xffffffffu, eb[i]);
+      if constexpr (AT) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sa[i] = shift(__reduce_max_sync(0xffffffffu, ea[i]), tb[i]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sb[i] = -sa[i];
+      } else {   // column t = lane of A runs across the warps
+        s_pt[w][lane] = max(max(ea[0], ea[1]), max(ea[2], ea[3]));
+        if (lane == 0)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) s_tb[4 * w + i] = tb[i];
+        __syncthreads();
+        int ta = s_pt[0][lane];
+#pragma unroll
+        for (int u = 1; u < 8; ++u) ta = max(ta, s_pt[u][lane]);
+        const int s = shift(ta, s_tb[lane]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          sa[i] = s;
+          sb[i] = -__shfl_sync(0xffffffffu, s, 4 * w + i);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (ea[i] != FX_NONE) ea[i] += sa[i];
+        if (eb[i] != FX_NONE) eb[i] += sb[i];
+      }
+    }
+    int ma = FX_NONE, mb = FX_NONE;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
       if (!AT) ea[i] = __reduce_max_sync(0xffffffffu, ea[i]);   // over the row's t
       if (BT) eb[i] = __reduce_max_sync(0xffffffffu, eb[i]);
       ma = max(ma, ea[i]);
       mb = max(mb, eb[i]);
-    }
-    if (__syncthreads_or(max(ma, mb) >= 0x7fe)) {   // uniform over the CTA; also: the last product's readers are done
-      plain();
-      return;
     }
     if (AT || !BT) {   // exponents of the rows or columns that run across the warps
       if (AT) s_pa[w][lane] = ma;
@@ -293,8 +395,8 @@ __device__ void tile_product(const T a[4], const T b[4], T* At, T* Bt, int kb, T
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      fx_store(&At[pa(i)], a[i], AT ? ma : ea[i]);
-      fx_store(&Bt[pb(i)], b[i], BT ? eb[i] : mb);
+      fx_store(&At[pa(i)], &Za[pa(i)], a[i], sa[i], AT ? ma : ea[i]);
+      fx_store(&Bt[pb(i)], &Zb[pb(i)], b[i], sb[i], BT ? eb[i] : mb);
       if (lane == 0) {
         if (!AT) s_ea[4 * w + i] = ea[i];
         if (BT) s_eb[4 * w + i] = eb[i];
@@ -305,52 +407,75 @@ __device__ void tile_product(const T a[4], const T b[4], T* At, T* Bt, int kb, T
     if constexpr (sizeof(T) == sizeof(double)) {
       const int2* Af = reinterpret_cast<const int2*>(At);
       const int2* Bf = reinterpret_cast<const int2*>(Bt);
-      long long hh[4] = {0, 0, 0, 0}, x[4] = {0, 0, 0, 0};
-#pragma unroll 4
+      long long h[4] = {0, 0, 0, 0}, x[4] = {0, 0, 0, 0}, y[4] = {0, 0, 0, 0};
+#pragma unroll 2
       for (int t = 0; t < NB; t += 2) {
         const int2 b0 = Bf[fx_col<BT>(t, lane)], b1 = Bf[fx_col<BT>(t + 1, lane)];
+        const int c0 = Zb[fx_col<BT>(t, lane)], c1 = Zb[fx_col<BT>(t + 1, lane)];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int4 u = *reinterpret_cast<const int4*>(&Af[fx_row<AT>(w + 8 * q, t)]);
-          hh[q] += (long long)u.x * b0.x;
+          const int2 v = *reinterpret_cast<const int2*>(&Za[fx_row<AT>(w + 8 * q, t)]);
+          h[q] += (long long)u.x * b0.x;
           x[q] += (long long)u.x * b0.y;
           x[q] += (long long)u.y * b0.x;
-          hh[q] += (long long)u.z * b1.x;
+          y[q] += (long long)u.x * c0;
+          y[q] += (long long)u.y * b0.y;
+          y[q] += (long long)v.x * b0.x;
+          h[q] += (long long)u.z * b1.x;
           x[q] += (long long)u.z * b1.y;
           x[q] += (long long)u.w * b1.x;
+          y[q] += (long long)u.z * c1;
+          y[q] += (long long)u.w * b1.y;
+          y[q] += (long long)v.y * b1.x;
         }
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] += fx_value(hh[q], x[q], s_ea[w + 8 * q] + ec - 2100);
+      for (int q = 0; q < 4; ++q) acc[q] += fx_value(h[q], x[q], y[q], s_ea[w + 8 * q] + ec - 2096);
     } else {
       const int4* Af = reinterpret_cast<const int4*>(At);
       const int4* Bf = reinterpret_cast<const int4*>(Bt);
-      long long rh[4] = {0, 0, 0, 0}, rx[4] = {0, 0, 0, 0}, ih[4] = {0, 0, 0, 0}, ix[4] = {0, 0, 0, 0};
+      long long rh[4] = {0, 0, 0, 0}, rx[4] = {0, 0, 0, 0}, ry[4] = {0, 0, 0, 0};
+      long long ih[4] = {0, 0, 0, 0}, ix[4] = {0, 0, 0, 0}, iy[4] = {0, 0, 0, 0};
 #pragma unroll 2
       for (int t = 0; t < NB; ++t) {
-        const int4 v = Bf[fx_col<BT>(t, lane)];   // (re hi, re lo, im hi, im lo)
+        const int4 v = Bf[fx_col<BT>(t, lane)];   // (re hi, re mid, im hi, im mid)
+        const int2 vl = Zb[fx_col<BT>(t, lane)];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int4 u = Af[fx_row<AT>(w + 8 * q, t)];
+          const int2 ul = Za[fx_row<AT>(w + 8 * q, t)];
           rh[q] += (long long)u.x * v.x;
           rh[q] -= (long long)u.z * v.z;
           rx[q] += (long long)u.x * v.y;
           rx[q] += (long long)u.y * v.x;
           rx[q] -= (long long)u.z * v.w;
           rx[q] -= (long long)u.w * v.z;
+          ry[q] += (long long)u.x * vl.x;
+          ry[q] += (long long)u.y * v.y;
+          ry[q] += (long long)ul.x * v.x;
+          ry[q] -= (long long)u.z * vl.y;
+          ry[q] -= (long long)u.w * v.w;
+          ry[q] -= (long long)ul.y * v.z;
           ih[q] += (long long)u.x * v.z;
           ih[q] += (long long)u.z * v.x;
           ix[q] += (long long)u.x * v.w;
           ix[q] += (long long)u.y * v.z;
           ix[q] += (long long)u.z * v.y;
           ix[q] += (long long)u.w * v.x;
+          iy[q] += (long long)u.x * vl.y;
+          iy[q] += (long long)u.y * v.w;
+          iy[q] += (long long)ul.x * v.z;
+          iy[q] += (long long)u.z * vl.x;
+          iy[q] += (long long)u.w * v.y;
+          iy[q] += (long long)ul.y * v.x;
         }
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int k = s_ea[w + 8 * q] + ec - 2100;
-        acc[q].x += fx_value(rh[q], rx[q], k);
-        acc[q].y += fx_value(ih[q], ix[q], k);
+        const int k = s_ea[w + 8 * q] + ec - 2096;
+        acc[q].x += fx_value(rh[q], rx[q], ry[q], k);
+        acc[q].y += fx_value(ih[q], ix[q], iy[q], k);
       }
     }
   }
@@ -364,7 +489,7 @@ template <class T, bool CL = false>
 __device__ int cta_potrf(T* A, int n, int lda, T* smem, Team<CL> tm = Team<CL>()) {
   using O = Ops<T>;
   using R = typename O::R;
-  T* D = smem;
+  T* D = smem;   // the diagonal block; the products' Z once the panel is solved
   T* Pi = smem + NB * NB;
   T* Pj = Pi + TL * NB;
   __shared__ int info;
@@ -437,7 +562,7 @@ __device__ int cta_potrf(T* A, int n, int lda, T* smem, Team<CL> tm = Team<CL>()
           b[u] = (j0 + r < n && lane < kb) ? O::conj(tm.ld(&A[(size_t)(j0 + r) * lda + k0 + lane])) : O::zero();
           acc[u] = O::zero();
         }
-        tile_product<T, true>(a, b, Pi, Pj, kb, acc);
+        tile_product<T, true>(a, b, Pi, Pj, D, kb, acc);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int i = i0 + w + 8 * q, j = j0 + lane;
@@ -470,14 +595,15 @@ __device__ __forceinline__ float lmul(float l, float b) { return l * b; }
 
 // Solve L X = B in place (L lower triangular n x n of type TLt, B n x nrhs
 // of type TB; TLt may be the real type of TB).  smem (bytes): room for
-// NB*NB elements of TLt followed by 2*NB*TL elements of TB.
+// NB*NB + 2*NB*TL elements of TB.
 template <class TLt, class TB>
 __device__ void cta_trsm_lower(const TLt* L, int n, int ldl, TB* B, int nrhs, int ldb, char* smem) {
   using OL = Ops<TLt>;
   using OB = Ops<TB>;
   using RB = typename OB::R;
-  TLt* D = reinterpret_cast<TLt*>(smem);
-  TB* Lt = reinterpret_cast<TB*>(D + NB * NB);
+  TB* Z = reinterpret_cast<TB*>(smem);
+  TLt* D = reinterpret_cast<TLt*>(smem);   // the diagonal block; the products' Z once it is solved
+  TB* Lt = Z + NB * NB;
   TB* Xt = Lt + TL * NB;
   __shared__ RB rdiag[NB];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -517,7 +643,7 @@ __device__ void cta_trsm_lower(const TLt* L, int n, int ldl, TB* B, int nrhs, in
           b[u] = (t < kb && c0 + lane < nrhs) ? B[(size_t)(k0 + t) * ldb + c0 + lane] : OB::zero();
           acc[u] = OB::zero();
         }
-        tile_product<TB, false>(a, b, Lt, Xt, kb, acc);
+        tile_product<TB, false>(a, b, Lt, Xt, Z, kb, acc);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int i = i0 + w + 8 * q, cc = c0 + lane;
@@ -581,7 +707,7 @@ __device__ void cta_trsm_lower_h(const T* L, int n, int ldl, T* B, int nrhs, int
           b[u] = (t < kb && c0 + lane < nrhs) ? B[(size_t)(k0 + t) * ldb + c0 + lane] : O::zero();
           acc[u] = O::zero();
         }
-        tile_product<T, false, true>(a, b, Lt, Xt, kb, acc);
+        tile_product<T, false, true, true>(a, b, Lt, Xt, D, kb, acc);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int i = i0 + w + 8 * q, cc = c0 + lane;
@@ -599,7 +725,7 @@ __device__ void cta_trsm_lower_h(const T* L, int n, int ldl, T* B, int nrhs, int
 
 // C (m x n) = beta*C + alpha * op(A) * B where op(A) = A^H (A is k x m,
 // transA = true) or A (m x k).  B is k x n.  All of type T (alpha real).
-// smem: 2*TL*NB elements of T.
+// smem: NB*NB + 2*TL*NB elements of T.
 template <class T>
 __device__ void cta_gemm(bool transA, int m, int n, int k, typename Ops<T>::R alpha,
                          const T* A, int lda, const T* B, int ldb,
@@ -607,6 +733,7 @@ __device__ void cta_gemm(bool transA, int m, int n, int k, typename Ops<T>::R al
   using O = Ops<T>;
   T* At = smem;
   T* Bt = smem + TL * NB;
+  T* Z = Bt + TL * NB;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   constexpr int PER = TL * TL / CTA_THREADS;   // outputs per thread
   for (int i0 = 0; i0 < m; i0 += TL) {
@@ -622,8 +749,8 @@ __device__ void cta_gemm(bool transA, int m, int n, int k, typename Ops<T>::R al
           else a[u] = (i0 + v < m && k0 + lane < k) ? A[(size_t)(i0 + v) * lda + k0 + lane] : O::zero();
           b[u] = (k0 + v < k && j0 + lane < n) ? B[(size_t)(k0 + v) * ldb + j0 + lane] : O::zero();
         }
-        if (transA) tile_product<T, false, true>(a, b, At, Bt, NB, acc);
-        else tile_product<T, false>(a, b, At, Bt, NB, acc);
+        if (transA) tile_product<T, false, true, true>(a, b, At, Bt, Z, NB, acc);
+        else tile_product<T, false, false, true>(a, b, At, Bt, Z, NB, acc);
       }
       for (int q = 0; q < PER; ++q) {
         int e = tid + q * CTA_THREADS;
@@ -688,7 +815,7 @@ __device__ void cta_trinv_lower(const T* L, int n, int ldl, T* X, int ldx, char*
           b[u] = (t < kb && c0 + lane < k1) ? tm.ld(&X[(size_t)(k0 + t) * ldx + c0 + lane]) : O::zero();
           acc[u] = O::zero();
         }
-        tile_product<T, false>(a, b, Lt, Xt, kb, acc);
+        tile_product<T, false>(a, b, Lt, Xt, D, kb, acc);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int i = i0 + w + 8 * q, cc = c0 + lane;
@@ -708,13 +835,14 @@ __device__ void cta_trinv_lower(const T* L, int n, int ldl, T* X, int ldx, char*
 // strictly upper tiles are written as their conjugate mirror (half the flops
 // of a full product).  With `tri` X is lower triangular (kdim = n) and each
 // tile sums only over rows k >= its first row (X[k][i] = 0 for k < i):
-// n^3/6 multiply-adds.  smem: 2*TL*NB elements of T.
+// n^3/6 multiply-adds.  smem: NB*NB + 2*TL*NB elements of T.
 template <class T, bool CL = false>
 __device__ void cta_herk_lower(const T* X, int kdim, int n, int ldx, T* M, int ldm, T* smem, bool tri,
                                Team<CL> tm = Team<CL>()) {
   using O = Ops<T>;
   T* At = smem;
   T* Bt = smem + TL * NB;
+  T* Z = Bt + TL * NB;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   constexpr int PER = TL * TL / CTA_THREADS;
   for (int i0 = 0; i0 < n; i0 += TL) {
@@ -730,7 +858,7 @@ __device__ void cta_herk_lower(const T* X, int kdim, int n, int ldx, T* M, int l
           a[u] = (i0 + lane < n && k0 + t < kdim) ? O::conj(tm.ld(&X[(size_t)(k0 + t) * ldx + i0 + lane])) : O::zero();
           b[u] = (k0 + t < kdim && j0 + lane < n) ? tm.ld(&X[(size_t)(k0 + t) * ldx + j0 + lane]) : O::zero();
         }
-        tile_product<T, false, true>(a, b, At, Bt, NB, acc);
+        tile_product<T, false, true>(a, b, At, Bt, Z, NB, acc);
       }
       for (int q = 0; q < PER; ++q) {
         int e = tid + q * CTA_THREADS;
