@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(256) k_patch_apply_blk(const int64_t* __restri
                                                          const TIN* __restrict__ r, int64_t ldr,
                                                          C* __restrict__ pbuf, int64_t ldp,
                                                          const uint8_t* __restrict__ rflag, int64_t offU) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   __shared__ C part[8][32 * PER + 1];
   __shared__ float4 ring[PER == 2 ? BLK_DEPTH : 1][PER == 2 ? 256 : 1];
   C* rj = reinterpret_cast<C*>(shraw);   // [KB][n]
@@ -280,7 +280,7 @@ __global__ void k_slot_sum_blk(const int64_t* __restrict__ sptr, const int32_t* 
 template <class C, int KB>
 __global__ void k_condense_apply_blk(int nS, int nI, const int64_t* __restrict__ Ig, const C* __restrict__ Y,
                                      const C* __restrict__ r, int64_t ld, C* __restrict__ cbuf, int64_t ldc) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   C* rI = reinterpret_cast<C*>(shraw);   // [KB][nI]
   const int64_t K = blockIdx.x;
   for (int i = threadIdx.x; i < nI; i += blockDim.x) {
@@ -308,7 +308,7 @@ template <class C, int KB>
 __global__ void k_backsub_blk(int nS, int nI, const int64_t* __restrict__ Sg, const int64_t* __restrict__ Ig,
                               const C* __restrict__ Ai, const C* __restrict__ Y, const C* __restrict__ r,
                               C* __restrict__ x, int64_t ld) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   C* rI = reinterpret_cast<C*>(shraw);   // [KB][nI]
   C* xS = rI + KB * nI;                  // [KB][nS]
   using O = Ops<C>;

@@ -90,7 +90,7 @@ __device__ __forceinline__ void block_mul(const C* P, const C* Q, C* X, typename
 template <class C>
 __global__ void __launch_bounds__(CTA_THREADS) k_dense_diag(C* A, int64_t N, int64_t ld, int k0, C* Dinv,
                                                             int* info) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   using O = Ops<C>;
   using R = typename O::R;
   constexpr int LD = CNB + 1, B = 16;
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(CTA_THREADS) k_dense_diag(C* A, int64_t N, int
 template <class C, int Q>
 __global__ void __launch_bounds__(CTA_THREADS) k_dense_panel(C* A, int64_t N, int64_t ld, int k0,
                                                              const C* __restrict__ Dinv) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   using O = Ops<C>;
   constexpr int LD = CNB + 1;
   C* Pa = reinterpret_cast<C*>(shraw);   // [CNB][LD] Pa[r][t] = A[i0 + r][k0 + t]
@@ -322,7 +322,7 @@ static void dense_cholesky(C* A, int64_t n, int64_t ld, C* Dinv, int* info, cuda
 // X[kb rows, tile cols] <- Dinv_kb * X[kb rows, tile cols], one CTA per W-column tile
 template <class C, int W>
 __global__ void __launch_bounds__(CTA_THREADS) k_trinv_scale(C* X, const C* Dinv, int64_t N, int64_t ld, int kb) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   C* D = reinterpret_cast<C*>(shraw);
   C* T = D + CNB * CNB;
   using O = Ops<C>;

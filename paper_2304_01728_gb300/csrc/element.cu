@@ -370,7 +370,7 @@ __device__ __forceinline__ Team<true> tile_share() {
 
 template <bool CL>
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_potrf(ElemArgs a) {
-  extern __shared__ double sh[];
+  extern __shared__ __align__(16) double sh[];
   Team<CL> tm;
   if constexpr (CL) {
     tm.rank = (int)elem_cluster_rank();
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(CTA_THREADS) k_elem_potrf(ElemArgs a) {
 
 template <class T>
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_trsm(ElemArgs a) {
-  extern __shared__ char shc[];
+  extern __shared__ __align__(16) char shc[];
   const int64_t le = blockIdx.x;
   int c0, cnt;
   strip(a.m + 1, &c0, &cnt);
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(CTA_THREADS) k_elem_trsm(ElemArgs a) {
 
 template <class T>
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_herk(ElemArgs a) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   const int64_t le = blockIdx.x;
   const int ld = a.m + 1;
   const T* W = reinterpret_cast<const T*>(a.W) + le * (size_t)a.nt * ld;
@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(CTA_THREADS) k_elem_herk(ElemArgs a) {
 //   Re K'[a][b] = R[a][b] + R[a~][b~],   Im K'[a][b] = R[a][b~] - R[a~][b]
 // (a~ = the imaginary column of a, terms absent where a has none).
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_trsm_split(ElemArgs a) {
-  extern __shared__ char shc[];
+  extern __shared__ __align__(16) char shc[];
   const int64_t le = blockIdx.x;
   const int ld2 = a.m + 1 + a.nph;
   const double* G = a.G + le * (size_t)a.nt * a.nt;
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(CTA_THREADS) k_elem_trsm_split(ElemArgs a) {
 }
 
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_herk_split(ElemArgs a) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   const int64_t le = blockIdx.x;
   const int ld = a.m + 1, ld2 = ld + a.nph;
   const double* W = reinterpret_cast<const double*>(reinterpret_cast<const double2*>(a.W) + le * (size_t)a.nt * ld);
@@ -477,7 +477,7 @@ __device__ __forceinline__ int phase_of(bool a_i, bool b_i) { return (a_i && !b_
 // strips' outputs (and a share of the recovery data Y).
 template <class T>
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_field_potrf(ElemArgs a) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   const int64_t le = blockIdx.x;
   const int ld = a.m + 1;
   T* K = reinterpret_cast<T*>(a.K) + le * (size_t)ld * ld;
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(CTA_THREADS) k_elem_field_potrf(ElemArgs a) {
 
 template <class T>
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_field_solve(ElemArgs a) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   const int64_t le = blockIdx.x;
   const int ld = a.m + 1, nf = a.nf;
   int c0, cnt;
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(CTA_THREADS) k_elem_field_solve(ElemArgs a) {
 
 template <class T, bool PH = false>
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_condense(ElemArgs a) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   T* sh = reinterpret_cast<T*>(shraw);
   const int64_t le = blockIdx.x;
   const int64_t e = a.elist[a.e0 + le];
@@ -599,7 +599,7 @@ template <class T, bool PH>
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_member_condense(ElemArgs a, const int64_t* __restrict__ mem_e,
                                                                       const int4* __restrict__ chunks, double* Ub,
                                                                       double* Cb, double* scr, int64_t stride) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   const int4 ch = chunks[blockIdx.x];
   const int slot = ch.x, cnt = ch.z;
   const int64_t rep = a.elist[a.e0 + slot];
@@ -1130,7 +1130,7 @@ static void element_core(SystemImpl& S, Level& L, const std::vector<double>& cva
 __global__ void __launch_bounds__(CTA_THREADS) k_elem_eta(ElemArgs a, const double2* __restrict__ fields,
                                                           const int64_t* __restrict__ dofs,
                                                           const double2* __restrict__ x, double* __restrict__ eta2) {
-  extern __shared__ unsigned char she[];
+  extern __shared__ __align__(16) unsigned char she[];
   const int64_t le = blockIdx.x;
   const int64_t e = a.elist[a.e0 + le];
   const int nt = a.nt, m = a.m, ldw = m + 1;

@@ -232,7 +232,7 @@ struct MacroArgs {
 
 template <class C>
 __global__ void __launch_bounds__(CTA_THREADS) k_macro(MacroArgs<C> a) {
-  extern __shared__ unsigned char shm[];
+  extern __shared__ __align__(16) unsigned char shm[];
   C* sh2 = reinterpret_cast<C*>(shm);
   using O = Ops<C>;
   using R = typename O::R;
@@ -349,7 +349,7 @@ static __global__ void k_cell_digits(const double2* __restrict__ E, const int64_
                                      const int32_t* __restrict__ idx, int n, int64_t offU,
                                      const uint8_t* __restrict__ rflag, uint4* __restrict__ dig, int64_t stride,
                                      float* __restrict__ rowscale) {
-  extern __shared__ int rowexp[];   // row a: |entries| < 2^rowexp[a]
+  extern __shared__ __align__(16) int rowexp[];   // row a: |entries| < 2^rowexp[a]
   const int64_t c = blockIdx.x, e = rep[c];
   const double2* A = E + e * (size_t)n * n;
   const int32_t* g = idx + e * n;
@@ -609,7 +609,7 @@ __global__ void __launch_bounds__(CTA_THREADS) k_patch_invert(const int64_t* ptr
                                                             const int64_t* vptr, C* vals, C* scratch,
                                                             const int64_t* soff, const int64_t* order, int64_t j0,
                                                             int64_t offU, int* info, uint8_t* rpack) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   C* sh = reinterpret_cast<C*>(shraw);
   Team<CL> tm;
   if constexpr (CL) {

@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(256, MINB) k_patch_apply(const int64_t* __rest
                                                      const C* __restrict__ inv, const TIN* __restrict__ r,
                                                      C* __restrict__ pbuf, const uint8_t* __restrict__ rflag,
                                                      int64_t offU) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   __shared__ C part[8][32 * PER + 1];
   C* rj = reinterpret_cast<C*>(shraw);
   using O = Ops<C>;
@@ -339,7 +339,7 @@ template <class C, class TIN>
 __global__ void __launch_bounds__(256) k_patch_apply_h(const int64_t* __restrict__ ptr, const int32_t* __restrict__ dofs,
                                                        const int64_t* __restrict__ hptr, const C* __restrict__ H,
                                                        const TIN* __restrict__ r, C* __restrict__ pbuf) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   using O = Ops<C>;
   const int64_t j = blockIdx.x;
   const int64_t b = ptr[j];

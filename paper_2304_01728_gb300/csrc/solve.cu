@@ -1182,7 +1182,7 @@ __global__ void __launch_bounds__(256) k_patch_apply_df(const int64_t* __restric
                                                         const float2* __restrict__ Mh, const float2* __restrict__ Ml,
                                                         const double2* __restrict__ r, double2* __restrict__ pbuf,
                                                         const uint8_t* __restrict__ rflag, int64_t offU) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   float4* rj = reinterpret_cast<float4*>(shraw);   // (re_hi, re_lo, im_hi, im_lo) per patch DOF
   __shared__ float4 part[8][33];
   const int2 ch = chunks[blockIdx.x];
@@ -1368,7 +1368,7 @@ void smooth_apply64(const Level& L, const double2* r, double2* y, double theta, 
 template <class C>
 __global__ void k_condense_apply(int nS, int nI, const int64_t* __restrict__ Ig, const C* __restrict__ Y,
                                  const C* __restrict__ r, C* __restrict__ cbuf) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   C* rI = reinterpret_cast<C*>(shraw);
   const int64_t K = blockIdx.x;
   for (int i = threadIdx.x; i < nI; i += blockDim.x) rI[i] = r[Ig[K * nI + i]];
@@ -1401,7 +1401,7 @@ template <class C>
 __global__ void k_backsub(int nS, int nI, const int64_t* __restrict__ Sg, const int64_t* __restrict__ Ig,
                           const C* __restrict__ Ai, const C* __restrict__ Y, const C* __restrict__ r,
                           C* __restrict__ x) {
-  extern __shared__ unsigned char shraw[];
+  extern __shared__ __align__(16) unsigned char shraw[];
   C* rI = reinterpret_cast<C*>(shraw);
   C* xS = rI + nI;
   using O = Ops<C>;

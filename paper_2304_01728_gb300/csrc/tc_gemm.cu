@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(TG_THREADS) k_tc_gemm(const unsigned char* __r
                                                         const unsigned char* __restrict__ Bimg, int64_t M, int64_t N,
                                                         int nst, float2* __restrict__ C, int64_t ldc, float alpha,
                                                         float beta, int lower, int* __restrict__ err, int fault) {
-  extern __shared__ unsigned char tg_raw[];
+  extern __shared__ __align__(16) unsigned char tg_raw[];
   __shared__ __align__(8) uint64_t bar_full[TG_NS];
   __shared__ __align__(8) uint64_t bar_empty[TG_NS];
   __shared__ __align__(8) uint64_t bar_acc[2];      // MMAs of a stage done: its TMEM buffer is ready
