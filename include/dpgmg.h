@@ -403,18 +403,30 @@ long long dpgmg_launch_count(void);
  * column indices copied 8 steps ahead into shared memory by asynchronous
  * copies (cp.async), or (G = 64, V-cycle operators only) by one half-warp
  * per row, two rows of a warp at a time.  Where the cells of a level share
- * matrices (mixed path, uniform parts of the medium), setup also times the
- * product cell by cell, which has no code here; an override selects the
- * assembled rows instead.  dpgmg_setup times every variant on each operator and
+ * matrices (mixed path, uniform parts of the medium) the product also runs
+ * cell by cell with one stored matrix per class (G = 128).
+ * dpgmg_setup times every variant on each operator and
  * keeps the fastest; choices are cached per (product type, p, level kind,
  * log2 of the row count) for the life of the process.  level >= 1 addresses
  * that level's V-cycle operator, level == -1 the CG operator.  set = 1, 2, 4,
- * 8, 16, 32 or 64 overrides the choice (0 leaves it; 64 is refused for the CG
- * operator); *group (may be NULL)
- * receives the value in force.  Returns DPGMG_ERR_ARG for an invalid level or
- * size.  Results do not depend on the variant beyond rounding order (G = 1,
- * 16 and 32: bitwise). */
+ * 8, 16, 32, 64 or 128 overrides the choice (0 leaves it; 64 is refused for the
+ * CG operator, 128 for an operator that keeps no class matrices); *group (may
+ * be NULL) receives the value in force, so that setting a value read before
+ * restores it.  Returns DPGMG_ERR_ARG for an invalid level or size.  Results do
+ * not depend on the variant beyond rounding order (G = 1, 16 and 32: bitwise). */
 int dpgmg_spmv_group(dpgmg_handle h, dpgmg_system sys, int level, int set, int* group);
+
+/* The same for the other products that may run with matrices shared by a class
+ * (mixed path): the smoother's patch inverses and an h level's macro transfers.
+ * which: DPGMG_FORM_SMOOTH, DPGMG_FORM_CONDENSE or DPGMG_FORM_BACKSUB; set = 0
+ * selects the general form (every block read where it is used), 1 the class
+ * form, -1 leaves the choice of dpgmg_setup; *form (may be NULL) receives the
+ * one in force.  Returns DPGMG_ERR_ARG for an invalid level or argument, and
+ * for set = 1 where the level has no class form.  Results differ by rounding. */
+#define DPGMG_FORM_SMOOTH   0
+#define DPGMG_FORM_CONDENSE 1
+#define DPGMG_FORM_BACKSUB  2
+int dpgmg_class_form(dpgmg_handle h, dpgmg_system sys, int level, int which, int set, int* form);
 
 /* DPG error indicator (Sec. 1.2: the residual that DPG minimises, in the
  * dual test norm, is the method's built-in error indicator; Sec. 3 refines

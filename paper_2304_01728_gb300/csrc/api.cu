@@ -687,29 +687,65 @@ int dpgmg_setup_phases(dpgmg_handle h, dpgmg_system sys, double* ms, int n) {
 
 int dpgmg_spmv_group(dpgmg_handle h, dpgmg_system sys, int level, int set, int* group) {
   if (!h || !sys) return DPGMG_ERR_ARG;
-  if (set != 0 && set != 1 && set != 2 && set != 4 && set != 8 && set != 16 && set != 32 && set != 64)
+  if (set != 0 && set != 1 && set != 2 && set != 4 && set != 8 && set != 16 && set != 32 && set != 64 && set != 128)
     return DPGMG_ERR_ARG;
   if (level == -1 && set == 64) return DPGMG_ERR_ARG;   // no half-warp form of the CG operator
   std::lock_guard<std::mutex> lk(h->mu);
   SystemImpl& S = sys->s;
   const int slot = S.op.precision == DPGMG_PREC_MIXED ? 0 : 1;
   int* g = nullptr;
-  bool* cells = nullptr;   // an override also selects the assembled rows
+  bool *cells = nullptr, kept = false;   // the product by cells: in force, available
   if (level == -1) {
     ECSRDev* A = cg_operator_of(S);
     if (!A) return DPGMG_ERR_ARG;
     g = &A->gsel[2];
     cells = &A->cell.df_on;
+    kept = A->cell.dig != nullptr;
   } else {
     if (level < 1 || level >= (int)S.levels.size()) return DPGMG_ERR_ARG;
-    g = &S.levels[level].A.gsel[slot];
-    cells = &S.levels[level].A.cell.on;
+    ECSRDev& A = S.levels[level].A;
+    g = &A.gsel[slot];
+    cells = &A.cell.on;
+    kept = A.cell.W != nullptr;
   }
-  if (set) {
+  if (set == 128) {
+    if (!kept) return DPGMG_ERR_ARG;
+    *cells = true;
+  } else if (set) {
     *g = set;
     *cells = false;
   }
-  if (group) *group = *g;
+  if (group) *group = *cells ? 128 : *g;
+  return DPGMG_OK;
+}
+
+int dpgmg_class_form(dpgmg_handle h, dpgmg_system sys, int level, int which, int set, int* form) {
+  if (!h || !sys || set < -1 || set > 1) return DPGMG_ERR_ARG;
+  std::lock_guard<std::mutex> lk(h->mu);
+  SystemImpl& S = sys->s;
+  if (level < 1 || level >= (int)S.levels.size()) return DPGMG_ERR_ARG;
+  Level& L = S.levels[level];
+  int now = 0;
+  if (which == DPGMG_FORM_SMOOTH) {
+    PatchDev& P = L.P;
+    if (set == 1 && !P.cls_items) return DPGMG_ERR_ARG;
+    if (set == 1 && P.variant != SMOOTH_CLASS) {
+      P.streamed = P.variant;
+      P.variant = SMOOTH_CLASS;
+    } else if (set == 0 && P.variant == SMOOTH_CLASS) {
+      P.variant = P.streamed ? P.streamed : (P.rflag ? SMOOTH_PER2_WIDE : 2);
+    }
+    P.cols = P.variant == 1 ? 1 : 2;
+    now = P.variant == SMOOTH_CLASS;
+  } else if (which == DPGMG_FORM_CONDENSE || which == DPGMG_FORM_BACKSUB) {
+    bool& on = which == DPGMG_FORM_CONDENSE ? L.mop.cond : L.mop.back;
+    if (set == 1 && !L.mop.Wb) return DPGMG_ERR_ARG;
+    if (set >= 0) on = set == 1;
+    now = on;
+  } else {
+    return DPGMG_ERR_ARG;
+  }
+  if (form) *form = now;
   return DPGMG_OK;
 }
 

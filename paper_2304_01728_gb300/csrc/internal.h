@@ -155,6 +155,10 @@ struct ECSRDev {
 // outputs x members of a class-product work item
 enum { CLS_64x32 = 0, CLS_64x16, CLS_64x8, CLS_32x32, CLS_32x16 };
 
+// variants of the complex64 smoother product beside 1 and 2 columns per lane (smoother.cuh)
+constexpr int SMOOTH_PER2_WIDE = 3;
+constexpr int SMOOTH_CLASS = 4;   // shared blocks, one product per patch class (classes.cuh)
+
 struct PatchDev {
   int64_t np = 0, nslots = 0, nvals = 0, max_n = 0, sum_sq = 0;
   int64_t* ptr = nullptr;
@@ -170,6 +174,7 @@ struct PatchDev {
   int64_t nchunks64 = 0;
   int cols = 2;                // complex64 product: columns per lane (1 or 2), tuned at setup
   int variant = 2;             // complex64 single-vector product variant (smoother.cuh), tuned at setup
+  int streamed = 0;            // the variant that the class product was chosen over by dpgmg_class_form (0: none)
   // complex64 inverses of the mixed path: rflag[j] = 1 when patch j's block
   // holds the real matrix w (A^-1[r][c] = w[r][c] i^(s_r - s_c), s = 1 on
   // p-hat DOFs, global index < offU) as n rows of ld reals in its first half

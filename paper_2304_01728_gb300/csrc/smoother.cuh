@@ -268,8 +268,7 @@ inline const int2* patch_chunks(const PatchDev& P, int per, int64_t* n) {
 // (64-column work items, 8 CTAs per SM, 32 registers), 3 = two columns per
 // lane at 6 CTAs per SM (40 registers: the real packed path then keeps its
 // loads in registers).
-constexpr int SMOOTH_PER2_WIDE = 3;
-constexpr int SMOOTH_CLASS = 4;   // shared blocks, one product per patch class (classes.cuh)
+// (SMOOTH_PER2_WIDE, SMOOTH_CLASS: internal.h)
 
 template <class TIN>
 inline void launch_patch_apply_c64(const PatchDev& P, int variant, const float2* inv, const TIN* r, float2* pbuf,

@@ -71,7 +71,9 @@ EXPORTS = ["dpgmg_create", "dpgmg_destroy", "dpgmg_query_sizes", "dpgmg_default_
            "dpgmg_element_matrix", "dpgmg_rhs", "dpgmg_apply", "dpgmg_launch_count", "dpgmg_profile",
            "dpgmg_profile_read", "dpgmg_smooth_noalloc", "dpgmg_serve_start", "dpgmg_submit", "dpgmg_poll",
            "dpgmg_spmv_group", "dpgmg_setup_profile", "dpgmg_error_indicator", "dpgmg_setup_phases",
-           "dpgmg_dof_map", "dpgmg_boundary_points", "dpgmg_solve_block"]
+           "dpgmg_dof_map", "dpgmg_boundary_points", "dpgmg_solve_block", "dpgmg_class_form"]
+SPMV_CELLS = 128   # dpgmg_spmv_group: the product by cells with class matrices
+FORM_SMOOTH, FORM_CONDENSE, FORM_BACKSUB = 0, 1, 2
 PROF_OFF, PROF_SMOOTH_FINE, PROF_SPMV_FINE, PROF_SPMV_CG = 0, 1, 2, 3
 
 
@@ -117,6 +119,8 @@ def lib():
     L.dpgmg_profile.argtypes = [vp, vp, i]
     L.dpgmg_spmv_group.argtypes = [vp, vp, i, i, ctypes.POINTER(i)]
     L.dpgmg_spmv_group.restype = i
+    L.dpgmg_class_form.argtypes = [vp, vp, i, i, i, ctypes.POINTER(i)]
+    L.dpgmg_class_form.restype = i
     L.dpgmg_setup_profile.argtypes = [vp, vp, ctypes.POINTER(d), ctypes.POINTER(d), ctypes.POINTER(d)]
     L.dpgmg_setup_profile.restype = i
     L.dpgmg_setup_phases.argtypes = [vp, vp, ctypes.POINTER(d), i]
@@ -351,6 +355,12 @@ def dpgmg_spmv_group(h, s, level, set_to=0):
     g = ctypes.c_int()
     _check(lib().dpgmg_spmv_group(h, s, int(level), int(set_to), ctypes.byref(g)), "dpgmg_spmv_group")
     return g.value
+
+
+def dpgmg_class_form(h, s, level, which, set_to=-1):
+    f = ctypes.c_int()
+    _check(lib().dpgmg_class_form(h, s, int(level), int(which), int(set_to), ctypes.byref(f)), "dpgmg_class_form")
+    return f.value
 
 
 def dpgmg_profile(h, s, which):
