@@ -21,14 +21,19 @@
 // shared-memory wavefronts at MPT = 4, so that the FP32 pipe and not shared
 // memory sets the rate.
 //
-// FP32 throughout, each output summed over k in increasing order.
+// FP32 throughout.  An output's products are summed in chains of eight, two of
+// them joined per chunk of 16 rows and the chunks added: a rounding error of 0.97
+// to 1.03 times that of 16 interleaved chains (the streaming smoother's order) for
+// n = 54 to 770, where one chain over all rows had 1.8 to 3.5 times as much.
 //
 // Finest smoother of a layered 32 x 32 x 16 mesh, p = 3 (473 M entries, 66% of
-// them real): 92 us, streamed 451 us; V-cycle operator by cells 47 us + 11 us of
+// them real): 99 us, streamed 451 us; V-cycle operator by cells 49 us + 11 us of
 // sums, assembled rows 295 us.  72 FMA a clock and SM inside the items, of 101
 // that an outer product fed from shared memory reaches; the rest is the start
-// of each item (dependent gathers) and the last wave.  Tried: 64 x 64 tiles 111
-// to 125 us, 128 x 16 tiles and 4 stages equal, 8-byte cp.async gathers 118 us.
+// of each item (dependent gathers) and the last wave.  The three sums take 168
+// registers: three CTAs per SM; one chain at four CTAs took 98 us, the three
+// sums at four (with spills) 106.  Tried: 64 x 64 tiles 111 to 125 us, 128 x 16
+// tiles and 4 stages equal, 8-byte cp.async gathers 118 us.
 #pragma once
 #include "common.cuh"
 #include "host_mesh.h"
@@ -41,7 +46,7 @@ constexpr int CLS_K = 16;       // rows of W per stage
 constexpr int CLS_STAGES = 3;   // stages of W in flight
 constexpr int CLS_THREADS = 128;
 constexpr int CLS_MEM = 32;     // members per item at most
-constexpr int CLS_CTAS = 4;     // resident per SM at least (registers)
+constexpr int CLS_CTAS = 3;     // resident per SM at least (registers)
 
 typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 pack2(float a, float b) {
@@ -57,6 +62,12 @@ __device__ __forceinline__ float2 unpack2(f32x2 v) {
 __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   f32x2 r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
 
@@ -138,11 +149,11 @@ __device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict
     for (int q = 0; q < NG; ++q) sm.r[c & 1][gk][gm + 8 * q] = gv[q];
   };
 
-  f32x2 acc[MPT][4];
+  f32x2 sum[MPT][4];   // the chunks' sums
 #pragma unroll
   for (int m = 0; m < MPT; ++m)
 #pragma unroll
-    for (int u = 0; u < 4; ++u) acc[m][u] = 0ull;
+    for (int u = 0; u < 4; ++u) sum[m][u] = 0ull;
 
 #pragma unroll
   for (int c = 0; c < CLS_STAGES - 1; ++c) load_w(c);
@@ -158,8 +169,22 @@ __device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict
     load_idx(c + 2);
     const unsigned char* ws = sm.w[c % CLS_STAGES] + tx * 16;
     const float2* rs = &sm.r[c & 1][0][ty * MPT];
+    f32x2 acc[MPT][4], half[MPT][4];
+#pragma unroll
+    for (int m = 0; m < MPT; ++m)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc[m][u] = 0ull;
 #pragma unroll
     for (int k = 0; k < CLS_K; ++k) {
+      if (k == CLS_K / 2) {
+#pragma unroll
+        for (int m = 0; m < MPT; ++m)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            half[m][u] = acc[m][u];
+            acc[m][u] = 0ull;
+          }
+      }
       f32x2 rv[MPT];
       if constexpr (MPT == 1) {
         const float2 t = rs[k * (CLS_MEM + 2)];
@@ -193,6 +218,11 @@ __device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict
         }
       }
     }
+#pragma unroll
+    for (int m = 0; m < MPT; ++m)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        sum[m][u] = add2(sum[m][u], add2(half[m][u], acc[m][u]));
     if (c + 1 < nch) store_val(c + 1);   // its last readers finished chunk c - 1
   }
 #pragma unroll
@@ -203,7 +233,7 @@ __device__ __forceinline__ void class_item(ClassSmem& sm, const void* __restrict
 #pragma unroll
     for (int m = 0; m < MPT; ++m) {
       const int q = ty * MPT + m;
-      if (q < cnt) out[oidx ? (int64_t)oidx[sm.obase[q] + a] : sm.obase[q] + a] = mul_i(unpack2(acc[m][u]), s);
+      if (q < cnt) out[oidx ? (int64_t)oidx[sm.obase[q] + a] : sm.obase[q] + a] = mul_i(unpack2(sum[m][u]), s);
     }
   }
 }
