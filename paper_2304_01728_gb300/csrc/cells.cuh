@@ -59,7 +59,7 @@ __device__ __forceinline__ void df_mul(float ah, float al, float xh, float xl, f
 }
 
 // The same product for the CG operator: 56-bit fixed point on the tensor cores.
-// A row a of a class matrix is 2^ea times integers of 55 bits, the DOFs of a
+// A row a of a class matrix is 2^ea times integers below 2^55, the DOFs of a
 // cell are 2^ex times such integers, and both are written as DG_S = 7 signed
 // digits of 8 bits (-128 .. 127), which bf16 holds exactly.  Digit products of
 // equal weight s + t = o share one FP32 accumulator per output: at most
@@ -72,10 +72,24 @@ __device__ __forceinline__ void df_mul(float ah, float al, float xh, float xl, f
 // Bound: 28 bf16 products per entry and real column on mma.sync (m16n8k16,
 // 0.5 a clock and SM: 50 us on a layered 32 x 32 x 16 mesh, p = 3), where the
 // double-float form took 12 FP32 instructions per real product.  Operator there
-// 281 -> 158 us, on 16^3, p = 3, 88 -> 66 us, and half the error against
-// complex128 (2.6e-15 to 5e-15 in norm, before 5.5e-15 to 8.8e-15).  Tried:
+// 281 -> 154 us, on 16^3, p = 3, 88 -> 65 us, and 0.2 to 0.9 of the error against
+// complex128 in norm (2.2e-15 to 3e-15 on residuals, before 3e-15 to 6e-15).  Tried:
 // the next tile's digits prefetched into L1, no change; the conversions are
-// half of the instructions, but twice as many only cost 4%.  A CTA turns the DOFs of up to 32 cells (64 real columns,
+// half of the instructions, but twice as many only cost 4%.
+//
+// Error of an output: about 2^-55 of the row's largest entry times the column's
+// largest per product, where the double-float form has 2^-48 of each product.  The
+// matrices are dense, Hermitian and positive definite, and how far an output's own
+// products stay below that product of the maxima goes with the spread of the
+// diagonal, max A_kk / min A_kk.  Relative to sum_k |A_ak x_k|, entry by entry, the
+// error is at most the assembled double-float rows' in the mean square (0.2 to 1.0
+// times on random vectors, residuals, V-cycle outputs and solutions; 0.3 to 1.3
+// times at the worst entry) up to a spread of 2^12 for p <= 4 and 2^11 for p = 5:
+// cubes of 1/4 to 1/24 at omega h > 0.5 or so.  At 2^12, p = 5, it has twice the error on
+// smooth solutions, at 2^25 (elements of 1/3000, or 1:100 flat ones) 30 to 70 times.
+// So digits are kept up to digit_spread(n), beyond it the assembled rows.
+//
+// A CTA turns the DOFs of up to 32 cells (64 real columns,
 // DG_KC rows) into digits once, in shared memory; a warp owns 16 outputs x 8
 // cells, with the matrix's digits read from L2 in fragment order (512 bytes a
 // warp and tile).
@@ -91,14 +105,14 @@ __device__ __forceinline__ void mma_bf16(float c[4], const uint4& a, uint32_t b0
                : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
 
-// the value of h + l in units of 2^(emax - 180): below 2^54 when emax is the
-// largest exponent field of the column (denormal parts count as zero)
+// the value of h in units of 2^(emax - 181): below 2^55 when emax is the column's
+// exponent (denormal parts count as zero)
 __device__ __forceinline__ long long digit_fixed(float h, int emax) {
   const uint32_t u = __float_as_uint(h);
-  const int e = (u >> 23) & 255, sh = e - emax + 30;
+  const int e = (u >> 23) & 255, sh = e - emax + 31;
   const long long m = (u & 0x7fffff) | 0x800000;
   if (e == 0 || sh < -25) return 0;
-  const long long f = sh >= 0 ? m << min(sh, 30) : (m + (1ll << (-sh - 1))) >> -sh;
+  const long long f = sh >= 0 ? m << min(sh, 31) : (m + (1ll << (-sh - 1))) >> -sh;
   return (int)u < 0 ? -f : f;
 }
 
@@ -139,7 +153,7 @@ static __global__ void __launch_bounds__(DG_THREADS, 2) k_class_cell_dg(
       const int m = w + 8 * j;
       if (m >= 8 * nq) break;   // uniform over the warp
       float2 h[2][2], l[2][2];
-      uint32_t emax = 0;
+      uint32_t top = 0;   // bits of the largest magnitude
 #pragma unroll
       for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -155,12 +169,17 @@ static __global__ void __launch_bounds__(DG_THREADS, 2) k_class_cell_dg(
               l[i][u] = mul_i(l[i][u], s);
             }
           }
-          emax = max(emax, max(__float_as_uint(h[i][u].x) & 0x7fffffffu, __float_as_uint(h[i][u].y) & 0x7fffffffu));
+          top = max(top, max(__float_as_uint(h[i][u].x) & 0x7fffffffu, __float_as_uint(h[i][u].y) & 0x7fffffffu));
         }
-      emax = __reduce_max_sync(0xffffffffu, emax) >> 23;
-      // 2^(ex - 1), the column being 2^(ex - 54) times its integers, ex = emax - 126; infinities and NaN give NaN
+      top = __reduce_max_sync(0xffffffffu, top);
+      // the column is 2^(emax - 181) times its integers; a largest value above 1 - 2^-7 of the power of two takes
+      // the next one, so that the leading digit with its carry stays below 128
+      const int emax = (int)((top + 0x20000u) >> 23);
+      // 2^(emax - 128); infinities and NaN give NaN
       if (lane == 0)
-        cscale[m] = emax == 255 ? __uint_as_float(0x7fffffffu) : (emax == 0 ? 0.f : __uint_as_float(emax << 23));
+        cscale[m] = top >= 0x7f800000u ? __uint_as_float(0x7fffffffu)
+                                       : (emax > 1 ? __uint_as_float((uint32_t)(emax - 1) << 23)
+                                                   : (emax == 1 ? __uint_as_float(0x00400000u) : 0.f));
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const int k = 64 * i + 2 * lane;

@@ -4,7 +4,7 @@
 
 namespace dpgmg {
 
-// the signed 8-bit digits of two fixed-point values (below 2^55), the leading one
+// the signed 8-bit digits of two fixed-point values (below 127.4 2^48), the leading one
 // first, as pairs of bf16: f's in the low halves, g's in the high ones
 __device__ __forceinline__ void digit_pairs(long long f, long long g, uint32_t d[DG_S]) {
   const long long bias = 0x0080808080808080ll;

@@ -58,6 +58,8 @@ template <class T, class AL> T* upload(Alloc& A, const std::vector<T, AL>& h, cu
 
 constexpr int DG_S = 7;        // 8-bit digits of a fixed-point operand of the CG operator by cells
 constexpr int DG_KC = 112;     // columns per exact accumulation: DG_S DG_KC 2^14 < 2^24
+// largest ratio of a class matrix's diagonal entries, in bits, for which digits are kept (cells.cuh)
+inline int digit_spread(int n) { return n <= 2 * DG_KC ? 12 : 11; }
 
 // ----------------------------------------------------------- device structs
 // An operator as a sum over its cells, y = sum_K R_K^T A_K R_K x, with one
@@ -77,6 +79,7 @@ struct CellOpDev {
   // the rows' scales
   uint4* dig = nullptr;
   float* dgrow = nullptr;
+  int* dgspread = nullptr;     // largest ratio of diagonal entries of a class, in bits; above digit_spread(n) no digits are kept
   uint8_t* rflag = nullptr;    // [ncls] real once the unit phases are taken out, rows of patch_ldr(n) reals
   int4* items = nullptr;       // work items as PatchDev::cls_items, over cells
   int64_t nitems = 0;

@@ -10,6 +10,7 @@
 //     ("V-cycle and smoother"),
 //   * the coarsest level (coarse.cu).
 #include <algorithm>
+#include <climits>
 #include <mutex>
 #include <cstdlib>
 #include <map>
@@ -348,8 +349,14 @@ __global__ void k_cell_class(const TE* __restrict__ E, int64_t e0, int64_t ne, c
 static __global__ void k_cell_digits(const double2* __restrict__ E, const int64_t* __restrict__ rep,
                                      const int32_t* __restrict__ idx, int n, int64_t offU,
                                      const uint8_t* __restrict__ rflag, uint4* __restrict__ dig, int64_t stride,
-                                     float* __restrict__ rowscale) {
-  extern __shared__ __align__(16) int rowexp[];   // row a: |entries| < 2^rowexp[a]
+                                     float* __restrict__ rowscale, int* __restrict__ spread) {
+  extern __shared__ __align__(16) int rowexp[];   // row a: |entries| <= (1 - 2^-7) 2^rowexp[a]
+  __shared__ int dmin, dmax;                      // exponents of the diagonal entries
+  if (threadIdx.x == 0) {
+    dmin = INT_MAX;
+    dmax = INT_MIN;
+  }
+  __syncthreads();
   const int64_t c = blockIdx.x, e = rep[c];
   const double2* A = E + e * (size_t)n * n;
   const int32_t* g = idx + e * n;
@@ -366,12 +373,18 @@ static __global__ void k_cell_digits(const double2* __restrict__ E, const int64_
     for (int k = lane; k < n; k += 32) mx = fmax(mx, fmax(fabs(entry(a, k, 0)), real ? 0.0 : fabs(entry(a, k, 1))));
     for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (lane == 0) {
-      const int ex = mx > 0.0 ? ilogb(mx) + 1 : 0;
+      int ex = mx > 0.0 ? ilogb(mx) + 1 : 0;
+      if (ldexp(mx, -ex) > 1.0 - 0x1p-7) ++ex;   // the leading digit with its carry stays below 128
       rowexp[a] = ex;
-      rowscale[c * T * 16 + a] = scalbnf(mx > 0.0 ? 1.f : 0.f, ex - 11);
+      rowscale[c * T * 16 + a] = scalbnf(mx > 0.0 ? 1.f : 0.f, ex - 12);
+      if (a < n && g[a] >= 0 && A[(size_t)a * n + a].x > 0.0) {
+        atomicMin(&dmin, ilogb(A[(size_t)a * n + a].x));
+        atomicMax(&dmax, ilogb(A[(size_t)a * n + a].x));
+      }
     }
   }
   __syncthreads();
+  if (threadIdx.x == 0 && dmax > dmin) atomicMax(spread, dmax - dmin);
   const int64_t total = (int64_t)(real ? 1 : 2) * T * T * 32;
   for (int64_t q = threadIdx.x; q < total; q += blockDim.x) {
     const int64_t tile = q / 32;
@@ -380,7 +393,7 @@ static __global__ void k_cell_digits(const double2* __restrict__ E, const int64_
     for (int u = 0; u < 4; ++u) {   // registers of the fragment: rows + 8 (u & 1), columns + 8 (u >> 1)
       const int a = 16 * mt + (ln >> 2) + 8 * (u & 1), k = 16 * kt + 2 * (ln & 3) + 8 * (u >> 1);
       long long f[2];
-      for (int j = 0; j < 2; ++j) f[j] = __double2ll_rn(ldexp(entry(a, k + j, part), 54 - rowexp[a]));
+      for (int j = 0; j < 2; ++j) f[j] = __double2ll_rn(ldexp(entry(a, k + j, part), 55 - rowexp[a]));
       digit_pairs(f[0], f[1], d[u]);
     }
     uint4* o = dig + c * stride + tile * (DG_S * 32) + ln;
@@ -441,7 +454,8 @@ static void cell_op_begin(SystemImpl& S, Level& F, const LevelPlan& lp, cudaStre
     D.dgrow = A.arr<float>((size_t)(D.ncls * D.tiles() * 16));
     cell_op_df_init();
     D.ydf = A.arr<float4>((size_t)D.ncell * D.n);
-    D.df_on = true;
+    D.dgspread = A.arr<int>(1);
+    DPG_CUDA(cudaMemsetAsync(D.dgspread, 0, sizeof(int), st));
   }
   D.rflag = A.arr<uint8_t>((size_t)D.ncls);
   D.ybuf = A.arr<float2>((size_t)D.ncell * D.n);
@@ -486,7 +500,8 @@ static void cell_op_matrices(SystemImpl& S, Level& F, const int64_t* rep, const 
   if constexpr (sizeof(TE) == sizeof(double2))
     if (D.dig) {   // finest level: E holds every cell's matrix
       k_cell_digits<<<(unsigned)D.ncls, 256, D.tiles() * 16 * sizeof(int), st>>>(E, rep, D.idx, D.n, D.offU, D.rflag,
-                                                                               D.dig, D.dgstride(), D.dgrow);
+                                                                               D.dig, D.dgstride(), D.dgrow,
+                                                                               D.dgspread);
       DPG_CHECK_LAUNCH();
     }
 }
@@ -1448,7 +1463,20 @@ void build_hierarchy(SystemImpl& S, cudaStream_t st) {
   std::vector<double> th((size_t)2 * (L + 1));
   DPG_CUDA(cudaMemcpyAsync(&info_main, dinfo, sizeof(int), cudaMemcpyDeviceToHost, st));
   DPG_CUDA(cudaMemcpyAsync(th.data(), dtheta, th.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
+  CellOpDev& cg = S.levels[L].A.cell;
+  int spread = 0;
+  if (cg.dig) DPG_CUDA(cudaMemcpyAsync(&spread, cg.dgspread, sizeof(int), cudaMemcpyDeviceToHost, st));
   DPG_CUDA(cudaStreamSynchronize(st));
+  if (spread > digit_spread(cg.n)) {   // rows of very different size: the CG operator keeps the assembled double-float rows
+    A.release(cg.dig);
+    A.release(cg.dgrow);
+    A.release(cg.ydf);
+    A.release(cg.dgitems);
+    cg.dig = nullptr;
+    cg.dgrow = nullptr;
+    cg.ydf = nullptr;
+    cg.dgitems = nullptr;
+  }
   A.release(dtheta);
   for (int l = lmin; l <= L; ++l)
     if (!(S.op.theta > 0.0)) S.levels[l].theta = theta_from_rayleigh(th[2 * l], th[2 * l + 1]);

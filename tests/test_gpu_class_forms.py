@@ -8,6 +8,8 @@ CG operator sums products good to 2^-46, 1e-12.
 import numpy as np
 import pytest
 
+from oracle.assembly import FineSystem
+from oracle.mesh import Mesh
 from paper_2304_01728_gb300 import dpgmg as D
 from tests.oracle_adapter import MIXED_VCYCLE_TOL, rand_vec, rel
 
@@ -33,7 +35,9 @@ CASES = [   # n, p, wavespeed layers, levels, p_min, flags
 
 def solver(case):
     n, p, lay, nl, p_min, fl = case
-    pk = dict(n=n, p=p, omega=4.0, src_center=(0.4, 0.55, 0.5), src_width=0.2)
+    # a frequency and a box at which the CG operator's digits are kept
+    pk = dict(n=n, p=p, omega=20.0 if p == 5 else 24.0, x1=(1, 0.8, 1.2) if p == 5 else (1, 1, 1),
+              src_center=(0.4, 0.55, 0.5), src_width=0.2)
     if lay:
         pk["wavespeed"] = layers(n, sum(n))
     return D.Solver(pk, n_levels=nl, p_min=p_min, precision="mixed", tol=1e-8, flags=fl)
@@ -160,3 +164,43 @@ def test_forms_that_a_system_does_not_have_are_refused():
             for level, which, v in ((0, 0, 0), (3, 0, 0), (1, 3, 0), (1, -1, 0), (1, 0, 2)):
                 with pytest.raises(D.DpgmgError):
                     D.dpgmg_class_form(s.h, s.s, level, which, v)
+
+
+@pytest.mark.parametrize("n,p,omega,box,digits", [
+    ((4, 4, 4), 2, 6.0, (1, 1, 1), True), ((6, 3, 1), 3, 12.0, (1.6, 1, 0.3), True),
+    ((6, 3, 1), 4, 8.0, (1, 0.5, 1 / 6), True), ((5, 4, 6), 5, 20.0, (1, 0.8, 1.2), True),
+    ((6, 3, 1), 3, 0.02, (2e3, 1e3, 300), True), ((6, 3, 1), 3, 12.0, (2e-3, 1e-3, 3e-4), False),
+    ((6, 3, 1), 3, 8.0, (2, 1, 0.003), False), ((6, 3, 1), 2, 8.0, (2, 0.1, 0.003), False)])
+def test_cg_operator_entry_by_entry(n, p, omega, box, digits):
+    """Error of every entry against complex128, relative to sum |A_ak| |x_k|.
+
+    The double-float form's operands and products are good to 2^-48; sums of up
+    to 8 x 302 products stay below 2^-43 of that sum.  The digits of a matrix row
+    and of a cell's values are relative to the largest of each, so they are kept
+    only where the class matrices' diagonals do not spread (cells.cuh), and are
+    there as good as the assembled rows (1.25: scatter of the two samples)."""
+    pk = dict(n=n, p=p, omega=omega, x1=box, src_center=tuple(0.4 * b for b in box), src_width=0.2 * max(box))
+    kw = dict(n_levels=2, p_min=p - 1, precision="mixed", tol=1e-8, max_iter=300)
+    g = np.asarray(FineSystem(Mesh(n, p, (0, 0, 0), box), omega, elements=[]).dofs)
+    nloc = g.shape[1]
+    with D.Solver(pk, **kw) as s, D.Solver(pk, flags=D.FLAG_CG_C128, **kw) as s1:
+        m = s.n_trace
+        if digits:
+            assert D.dpgmg_spmv_group(s.h, s.s, -1, D.SPMV_CELLS) == D.SPMV_CELLS
+        else:
+            assert D.dpgmg_spmv_group(s.h, s.s, -1) != D.SPMV_CELLS
+            with pytest.raises(D.DpgmgError):
+                D.dpgmg_spmv_group(s.h, s.s, -1, D.SPMV_CELLS)
+        sol = s1.solve(fields=False)[0]
+        K = np.array([np.abs(D.dpgmg_element_matrix(s.h, s.s, 1, e, nloc)) for e in range(len(g))])
+        for x in (sol, rand_vec(m, 3), D.dpgmg_rhs(s.h, s.s, m)):
+            xl = np.where(g >= 0, np.abs(x)[np.maximum(g, 0)], 0)
+            bound = np.zeros(m)
+            np.add.at(bound, g[g >= 0], np.einsum("eij,ej->ei", K, xl)[g >= 0])
+            want, q = D.dpgmg_apply(s1.h, s1.s, D.OP_AFULL, 1, x, m), []
+            for form in (D.SPMV_CELLS, 1) if digits else (1,):
+                assert D.dpgmg_spmv_group(s.h, s.s, -1, form) == form
+                err = np.abs(D.dpgmg_apply(s.h, s.s, D.OP_AFULL, 1, x, m) - want) / np.maximum(bound, 1e-300)
+                assert np.max(err) <= 2.0 ** -43
+                q.append(np.sqrt(np.mean(err ** 2)))
+            assert q[0] <= 1.25 * q[-1], q
