@@ -25,6 +25,16 @@ void count_launch() {
 void count_launches(long long n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 long long thread_launch_count() { return t_launches; }
 
+static std::atomic<int> g_running{0};
+static std::atomic<long long> g_started{0};
+GpuWork::GpuWork() {
+  ++g_running;
+  ++g_started;
+}
+GpuWork::~GpuWork() { --g_running; }
+int gpu_work_running() { return g_running.load(); }
+long long gpu_work_started() { return g_started.load(); }
+
 void* Alloc::get(size_t bytes) {
   bytes = (bytes + 255) & ~(size_t)255;
   if (used + bytes > budget) throw Err{DPGMG_ERR_NOMEM, "device-memory budget exceeded"};
@@ -220,6 +230,7 @@ static void fill_bytes_per_iter(SystemImpl& S) {
 }
 
 void setup_system(SystemImpl& S, const dpgmg_problem* pb, const dpgmg_opts* op, size_t budget, cudaStream_t st) {
+  GpuWork work;
   S.pb = *pb;
   S.op = *op;
   const int64_t ne = (int64_t)pb->n[0] * pb->n[1] * pb->n[2];

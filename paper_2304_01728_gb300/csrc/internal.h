@@ -26,6 +26,18 @@ void set_last_error(const std::string& m);
     if (e_ != cudaSuccess)                                                             \
       throw ::dpgmg::Err{DPGMG_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)}; \
   } while (0)
+// Setups and solves of this process in flight, and how many have ever begun: a
+// timing on the GPU is undisturbed when its setup is the only one and none begins
+// meanwhile.
+struct GpuWork {
+  GpuWork();
+  ~GpuWork();
+  GpuWork(const GpuWork&) = delete;
+  GpuWork& operator=(const GpuWork&) = delete;
+};
+int gpu_work_running();
+long long gpu_work_started();
+
 void count_launch();
 void count_launches(long long n);
 long long thread_launch_count();

@@ -26,6 +26,7 @@
 #include "smoother.cuh"
 #include "classes.cuh"
 #include "cells.cuh"
+#include "tune.h"
 
 namespace dpgmg {
 
@@ -2221,11 +2222,10 @@ static void cg_apply(SystemImpl& S, WS& W, const ECSRDev& A, const double2* x, c
 // ------------------------------------------------------------ tuning
 // The SpMV group size G (rows of one entity per warp, 1 = one warp per row)
 // and the smoother's columns per lane are chosen per operator by timing the
-// variants on the operator itself (one warm-up and three timed launches each,
-// each timed launch after an L2 eviction, CUDA events on the setup stream).
-// The first variant is kept unless another is at least 5% faster.  Choices
-// are cached per (product kind, order p, level kind, log2 of the size), so
-// later systems of the same shape skip the timing.
+// variants on the operator itself (one warm-up launch each, then TUNE_REPS in turn,
+// each after an L2 eviction, CUDA events on the setup stream; tune.h says what
+// decides).  Choices are cached per (product kind, order p, level kind, log2 of
+// the size), so later systems of the same shape skip the timing.
 struct TuneKey {
   int kind, p, lkind, lg;
   bool operator<(const TuneKey& o) const {
@@ -2233,7 +2233,7 @@ struct TuneKey {
   }
 };
 static std::mutex g_tune_mu;
-static std::map<TuneKey, int> g_tune;
+static std::map<TuneKey, TuneRecord> g_tune;
 
 // Reads `n` 16-byte words so that the timed launch after it finds the L2
 // holding other data, as inside a V-cycle (the sum is stored only if it hits
@@ -2276,47 +2276,42 @@ static int pick_group(const TuneKey& key, const Evict& ev, cudaStream_t st, F&& 
 template <class F>
 static int pick_variant(const TuneKey& key, const Evict& ev, cudaStream_t st, std::initializer_list<int> variants,
                         F&& run) {
+  const std::vector<int> forms(variants);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(key);
-    if (it != g_tune.end()) return it->second;
+    if (it != g_tune.end() && it->second.settled && it->second.ms.size() == forms.size())
+      return forms[it->second.best()];
   }
-  constexpr int REPS = 3;
-  cudaEvent_t a[REPS], b[REPS];
-  for (int r = 0; r < REPS; ++r) {
-    DPG_CUDA(cudaEventCreate(&a[r]));
-    DPG_CUDA(cudaEventCreate(&b[r]));
-  }
-  int best = *variants.begin();
-  float best_ms = 0.f;
-  for (int G : variants) {
-    run(G);
-    for (int r = 0; r < REPS; ++r) {
+  struct Events {   // destroyed on every exit path
+    std::vector<cudaEvent_t> e;
+    explicit Events(size_t n) : e(n, nullptr) {
+      for (cudaEvent_t& x : e) DPG_CUDA(cudaEventCreate(&x));
+    }
+    ~Events() {
+      for (cudaEvent_t x : e)
+        if (x) cudaEventDestroy(x);
+    }
+  } ev2(2 * TUNE_REPS * forms.size());
+  auto at = [&](size_t v, int r, int end) { return ev2.e[2 * (v * TUNE_REPS + r) + end]; };
+  const long long work = gpu_work_started();
+  const bool crowded = gpu_work_running() > 1;
+  for (int G : forms) run(G);
+  for (int r = 0; r < TUNE_REPS; ++r)
+    for (size_t v = 0; v < forms.size(); ++v) {
       ev.run(st);
-      DPG_CUDA(cudaEventRecord(a[r], st));
-      run(G);
-      DPG_CUDA(cudaEventRecord(b[r], st));
+      DPG_CUDA(cudaEventRecord(at(v, r, 0), st));
+      run(forms[v]);
+      DPG_CUDA(cudaEventRecord(at(v, r, 1), st));
     }
-    DPG_CUDA(cudaEventSynchronize(b[REPS - 1]));
-    float ms = 0.f;
-    for (int r = 0; r < REPS; ++r) {
-      float t = 0.f;
-      DPG_CUDA(cudaEventElapsedTime(&t, a[r], b[r]));
-      ms += t;
-    }
-    // the first variant is the default: another must be at least 5% faster
-    if (G == *variants.begin() || ms < (best == *variants.begin() ? 0.95f : 1.0f) * best_ms) {
-      best = G;
-      best_ms = ms;
-    }
-  }
-  for (int r = 0; r < REPS; ++r) {
-    cudaEventDestroy(a[r]);
-    cudaEventDestroy(b[r]);
-  }
+  DPG_CUDA(cudaEventSynchronize(at(forms.size() - 1, TUNE_REPS - 1, 1)));
+  std::vector<std::vector<float>> ms(forms.size(), std::vector<float>(TUNE_REPS));
+  for (size_t v = 0; v < forms.size(); ++v)
+    for (int r = 0; r < TUNE_REPS; ++r) DPG_CUDA(cudaEventElapsedTime(&ms[v][r], at(v, r, 0), at(v, r, 1)));
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  g_tune[key] = best;
-  return best;
+  TuneRecord& rec = g_tune[key];
+  rec.add(ms, !crowded && gpu_work_started() == work);
+  return forms[rec.best()];
 }
 
 static int log2i(int64_t n) {
@@ -2453,6 +2448,16 @@ void prepare_solve(SystemImpl& S, cudaStream_t st) {
       F.A.gsel[1] = pick_group(key, ev, st, [&](int G) { spmv_g<double2>(F.A, F.A.v64, x, nullptr, y, 0, G, st); });
     }
   }
+  if (L >= 1 && mixed && S.levels[0].P.cls_items) {   // level 0 smoothed (DPGMG_COARSEST_SMOOTH)
+    PatchDev& P = S.levels[0].P;
+    float2* x = W.w32[0].x;
+    DPG_CUDA(cudaMemsetAsync(x, 0, (size_t)S.levels[0].mesh.ndof * sizeof(float2), st));
+    const TuneKey key{(P.rflag ? 4 : 3) + 16 * (1 + log2i(P.ncls_items)), S.levels[0].mesh.p, 0, log2i(P.np)};
+    P.variant = pick_variant(key, ev, st, {SMOOTH_CLASS, 2}, [&](int c) {
+      if (c == SMOOTH_CLASS) launch_class_apply<float2>(P, x, 0, W.w32[0].pbuf, 0, 1, st);
+      else launch_patch_apply_c64<float2>(P, c, P.inv32, x, W.w32[0].pbuf, st);
+    });
+  }
   {
     const Level& F = S.levels[L];
     const int64_t n = F.mesh.ndof;
@@ -2476,6 +2481,7 @@ void prepare_solve(SystemImpl& S, cudaStream_t st) {
 }
 
 int pcg_solve(SystemImpl& S, cudaStream_t st, double2* xout, dpgmg_stats* stats, const double2* x0) {
+  GpuWork work;
   ensure_workspace(S, st);
   WS& W = *reinterpret_cast<WS*>(S.ws);
   const ECSRDev& A = cg_operator(S, W, st);
@@ -2618,6 +2624,7 @@ int pcg_solve(SystemImpl& S, cudaStream_t st, double2* xout, dpgmg_stats* stats,
 // graph captured for the current set of active columns (captured again when
 // a column converges).
 int pcg_solve_block(SystemImpl& S, cudaStream_t st, int K, const double2* B, double2* X, dpgmg_stats* stats) {
+  GpuWork work;
   ensure_workspace(S, st);
   WS& W = *reinterpret_cast<WS*>(S.ws);
   const ECSRDev& A = cg_operator(S, W, st);
