@@ -302,7 +302,9 @@ int dpgmg_solve(dpgmg_handle h, dpgmg_system sys, void* trace_out, void* field_o
  * cost of the smoothing patches): k independent MG-PCG solves from x0 = 0, one
  * per right-hand side, each with its own scalars and stopping test (the
  * recurrence of dpgmg_solve), sharing every V-cycle.  The V-cycle's smoother
- * and SpMV read their stored matrices once for up to 4 right-hand sides.
+ * and SpMV read their stored matrices once for up to 4 right-hand sides; where
+ * blocks are shared by a class, the first call times the class products (one
+ * right-hand side after the other) against that, per product and for this k.
  * rhs: c128 [k][n_trace] condensed right-hand sides (e.g. dpgmg_rhs of
  * systems with other sources); trace_out: c128 [k][n_trace]; both device
  * pointers when on_device != 0, else host.  stats: k entries or NULL; each
@@ -412,7 +414,7 @@ long long dpgmg_launch_count(void);
  * 8, 16, 32, 64 or 128 overrides the choice (0 leaves it; 64 is refused for the
  * CG operator, 128 for an operator that keeps no class matrices); *group (may
  * be NULL) receives the value in force, so that setting a value read before
- * restores it.  Returns DPGMG_ERR_ARG for an invalid level or size.  Results do
+ * restores it (a value set here also holds for dpgmg_solve_block).  Returns DPGMG_ERR_ARG for an invalid level or size.  Results do
  * not depend on the variant beyond rounding order (G = 1, 16 and 32: bitwise). */
 int dpgmg_spmv_group(dpgmg_handle h, dpgmg_system sys, int level, int set, int* group);
 

@@ -706,17 +706,20 @@ int dpgmg_spmv_group(dpgmg_handle h, dpgmg_system sys, int level, int set, int* 
   const int slot = S.op.precision == DPGMG_PREC_MIXED ? 0 : 1;
   int* g = nullptr;
   bool *cells = nullptr, kept = false;   // the product by cells: in force, available
+  BlockForm* blk = nullptr;              // an override holds for several vectors too
   if (level == -1) {
     ECSRDev* A = cg_operator_of(S);
     if (!A) return DPGMG_ERR_ARG;
     g = &A->gsel[2];
     cells = &A->cell.df_on;
+    blk = &A->cell.df_blk;
     kept = A->cell.dig != nullptr;
   } else {
     if (level < 1 || level >= (int)S.levels.size()) return DPGMG_ERR_ARG;
     ECSRDev& A = S.levels[level].A;
     g = &A.gsel[slot];
     cells = &A.cell.on;
+    blk = &A.cell.blk;
     kept = A.cell.W != nullptr;
   }
   if (set == 128) {
@@ -726,6 +729,7 @@ int dpgmg_spmv_group(dpgmg_handle h, dpgmg_system sys, int level, int set, int* 
     *g = set;
     *cells = false;
   }
+  if (set) blk->set(*cells);
   if (group) *group = *cells ? 128 : *g;
   return DPGMG_OK;
 }
@@ -748,10 +752,14 @@ int dpgmg_class_form(dpgmg_handle h, dpgmg_system sys, int level, int which, int
     }
     P.cols = P.variant == 1 ? 1 : 2;
     now = P.variant == SMOOTH_CLASS;
+    if (set >= 0) P.blk.set(now);
   } else if (which == DPGMG_FORM_CONDENSE || which == DPGMG_FORM_BACKSUB) {
     bool& on = which == DPGMG_FORM_CONDENSE ? L.mop.cond : L.mop.back;
     if (set == 1 && !L.mop.Wb) return DPGMG_ERR_ARG;
-    if (set >= 0) on = set == 1;
+    if (set >= 0) {
+      on = set == 1;
+      (which == DPGMG_FORM_CONDENSE ? L.mop.cond_blk : L.mop.back_blk).set(set);
+    }
     now = on;
   } else {
     return DPGMG_ERR_ARG;

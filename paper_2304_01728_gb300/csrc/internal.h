@@ -74,6 +74,19 @@ constexpr int DG_KC = 112;     // columns per exact accumulation: DG_S DG_KC 2^1
 inline int digit_spread(int n) { return n <= 2 * DG_KC ? 12 : 11; }
 
 // ----------------------------------------------------------- device structs
+// Form of a product with class matrices for k right-hand sides at once.  The
+// block kernels of the general forms read a stored matrix once for up to four
+// vectors, the class forms run vector after vector (the smoother: with the
+// vectors as a grid dimension), so the choice for one vector does not carry over:
+// each k up to four (more: in groups) has its own, timed in the first block solve.
+struct BlockForm {
+  signed char f[5] = {-1, -1, -1, -1, -1};   // by min(k, 4): 1 class, 0 general, -1 not timed (class)
+  bool by_class(int k) const { return f[k < 4 ? k : 4] != 0; }
+  void set(int v) {
+    for (signed char& x : f) x = (signed char)v;
+  }
+};
+
 // An operator as a sum over its cells, y = sum_K R_K^T A_K R_K x, with one
 // stored matrix per cell class (classes.cuh): the elements of a p level, the
 // macro elements of an h level.  Kept beside the assembled rows when the cells
@@ -81,6 +94,7 @@ inline int digit_spread(int n) { return n <= 2 * DG_KC ? 12 : 11; }
 struct CellOpDev {
   bool on = false;             // applied in place of the assembled rows (complex64 V-cycle operator)
   bool df_on = false;          // the same for the CG operator (digits)
+  BlockForm blk, df_blk;       // both for several vectors, where they are on for one
   int n = 0;                   // local DOFs of a cell
   int64_t ncell = 0, ndof = 0, ncls = 0;
   int32_t* idx = nullptr;      // [ncell][n] DOF, or -1
@@ -122,6 +136,7 @@ inline int64_t cell_row(int64_t g, int64_t offE, int64_t offF) {
 // Macro-grid transfers with one stored matrix per macro class (cells.cuh)
 struct MacroOpDev {
   bool back = false, cond = false;   // back-substitution, condensation by classes (tuned)
+  BlockForm back_blk, cond_blk;
   int nI = 0, nS = 0;
   int64_t offU = 0;
   int32_t* idx = nullptr;      // [nK][nI + nS] DOFs, I then S
@@ -189,6 +204,7 @@ struct PatchDev {
   int64_t nchunks64 = 0;
   int cols = 2;                // complex64 product: columns per lane (1 or 2), tuned at setup
   int variant = 2;             // complex64 single-vector product variant (smoother.cuh), tuned at setup
+  BlockForm blk;               // class product for several vectors, where variant is SMOOTH_CLASS
   int streamed = 0;            // the variant that the class product was chosen over by dpgmg_class_form (0: none)
   // complex64 inverses of the mixed path: rflag[j] = 1 when patch j's block
   // holds the real matrix w (A^-1[r][c] = w[r][c] i^(s_r - s_c), s = 1 on

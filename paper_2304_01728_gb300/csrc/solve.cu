@@ -1991,7 +1991,7 @@ static void smooth_blk(const Level& L, const C* r, C* y, double theta, int accum
       DPG_CHECK_LAUNCH();
       return;
     }
-    if (P.variant == SMOOTH_CLASS) {   // shared blocks: the K vectors as a second grid dimension, each block read from L2
+    if (P.variant == SMOOTH_CLASS && P.blk.by_class(K)) {   // the K vectors as a second grid dimension
       launch_class_apply<float2>(P, r, n, pbuf, ldp, K, st);
       k_slot_sum_blk<C><<<dim3(nblk(n), (unsigned)K), 256, 0, st>>>(P.slot_ptr, P.slots, pbuf, ldp, y, n, n, theta,
                                                                      accumulate);
@@ -2026,7 +2026,7 @@ static void spmv_blk(const ECSRDev& A, const C* vals, const C* x, const C* b, C*
                      cudaStream_t st) {
   const int64_t n = A.nrows;
   if constexpr (std::is_same<C, float2>::value) {
-    if (A.cell.on) {   // shared cell matrices, read from L2 for every vector
+    if (A.cell.on && A.cell.blk.by_class(K)) {   // shared cell matrices, read from L2 for every vector
       for (int k = 0; k < K; ++k) cell_op_apply(A.cell, x + k * n, b ? b + k * n : nullptr, y + k * n, mode, st);
       return;
     }
@@ -2059,7 +2059,8 @@ template <class C> static int blk_group(int64_t per_vec) {
 template <class C>
 static void condense_blk(const Level& F, const C* r, C* rs, C* cbuf, int K, cudaStream_t st) {
   const int64_t n = F.mesh.ndof, ldc = (int64_t)F.nK * F.nS;
-  const int cap = F.mop.cond ? 0 : blk_group<C>(F.nI);
+  const bool by_class = std::is_same<C, float2>::value && F.mop.cond && F.mop.cond_blk.by_class(K);
+  const int cap = by_class ? 0 : blk_group<C>(F.nI);
   if (cap < 1) {   // shared classes, or too large a block: one vector at a time
     for (int k = 0; k < K; ++k) condense<C>(F, r + k * n, rs + k * n, cbuf, st);
     return;
@@ -2088,7 +2089,8 @@ static void condense_blk(const Level& F, const C* r, C* rs, C* cbuf, int K, cuda
 template <class C>
 static void backsub_blk(const Level& F, const C* r, C* x, int K, cudaStream_t st) {
   const int64_t n = F.mesh.ndof;
-  const int cap = F.mop.back ? 0 : blk_group<C>((int64_t)F.nI + F.nS);
+  const bool by_class = std::is_same<C, float2>::value && F.mop.back && F.mop.back_blk.by_class(K);
+  const int cap = by_class ? 0 : blk_group<C>((int64_t)F.nI + F.nS);
   if (cap < 1) {
     for (int k = 0; k < K; ++k) backsub<C>(F, r + k * n, x + k * n, st);
     return;
@@ -2377,25 +2379,29 @@ ECSRDev* cg_operator_of(SystemImpl& S) {
   return W.acg_owned ? &W.Acg : nullptr;
 }
 
+// between timed launches, read up to 256 MiB of the finest patch inverses
+static Evict evict_of(const SystemImpl& S, const WS& W) {
+  Evict ev;
+  const bool mixed = S.op.precision == DPGMG_PREC_MIXED;
+  const PatchDev& P = S.levels.back().P;
+  const void* buf = mixed && P.inv32 ? (const void*)P.inv32 : (P.inv64 ? (const void*)P.inv64 : (const void*)P.wbuf);
+  const int64_t bytes = std::min<int64_t>(P.inv32 || P.inv64 ? P.nvals * (mixed && P.inv32 ? 8 : 16) : P.wcap * 8,
+                                          (int64_t)256 << 20);
+  if (S.levels.size() > 1 && buf && bytes >= 16) {
+    ev.buf = reinterpret_cast<const float4*>(buf);
+    ev.n = bytes / 16;
+    ev.sink = reinterpret_cast<float*>(W.part);
+  }
+  return ev;
+}
+
 void prepare_solve(SystemImpl& S, cudaStream_t st) {
   ensure_workspace(S, st);
   WS& W = *reinterpret_cast<WS*>(S.ws);
   ECSRDev& Acg = const_cast<ECSRDev&>(cg_operator(S, W, st));
   const bool mixed = S.op.precision == DPGMG_PREC_MIXED;
   const int L = (int)S.levels.size() - 1;
-  // between timed launches, read up to 256 MiB of the finest patch inverses
-  Evict ev;
-  {
-    const PatchDev& P = S.levels[L].P;
-    const void* buf = mixed && P.inv32 ? (const void*)P.inv32 : (P.inv64 ? (const void*)P.inv64 : (const void*)P.wbuf);
-    const int64_t bytes = std::min<int64_t>(P.inv32 || P.inv64 ? P.nvals * (mixed && P.inv32 ? 8 : 16) : P.wcap * 8,
-                                            (int64_t)256 << 20);
-    if (L >= 1 && buf && bytes >= 16) {
-      ev.buf = reinterpret_cast<const float4*>(buf);
-      ev.n = bytes / 16;
-      ev.sink = reinterpret_cast<float*>(W.part);
-    }
-  }
+  const Evict ev = evict_of(S, W);
   for (int l = 1; l <= L; ++l) {
     Level& F = S.levels[l];
     const int64_t n = F.mesh.ndof;
@@ -2660,7 +2666,7 @@ int pcg_solve_block(SystemImpl& S, cudaStream_t st, int K, const double2* B, dou
     }
     k_split_vec<<<nblk(n * K), 256, 0, st>>>(Xs, XH, XL, n * K);
     DPG_CHECK_LAUNCH();
-    if (A.cell.df_on) {
+    if (A.cell.df_on && A.cell.df_blk.by_class(K)) {
       for (int k = 0; k < K; ++k)
         cell_op_apply_df(A.cell, XH + (size_t)k * n, XL + (size_t)k * n, Bs ? Bs + (size_t)k * n : nullptr,
                          Ys + (size_t)k * n, mode, st);
@@ -2688,6 +2694,37 @@ int pcg_solve_block(SystemImpl& S, cudaStream_t st, int K, const double2* B, dou
   std::vector<BlockLevel<double2>> V64;
   if (mixed) V32 = alloc_block_levels<float2>(M, S, K);
   else V64 = alloc_block_levels<double2>(M, S, K);
+  if (mixed && K > 1) {   // forms for several vectors, where the class form is on for one
+    const Evict ev = evict_of(S, W);
+    const int kb = std::min(K, BLK_MAX);
+    auto choose = [&](BlockForm& form, int product, int64_t items, const Level& F, auto&& run) {
+      if (form.f[kb] >= 0) return;
+      const TuneKey key{-(product * 512 + 8 * log2i(items) + kb), F.mesh.p, F.kind, log2i(F.mesh.ndof)};
+      form.f[kb] = (signed char)pick_variant(key, ev, st, {1, 0}, [&](int v) {
+        form.f[kb] = (signed char)v;
+        run();
+      });
+    };
+    for (int l = 0; l <= L; ++l) {
+      Level& F = S.levels[l];
+      BlockLevel<float2>& V = V32[l];
+      const size_t bytes = (size_t)F.mesh.ndof * kb * sizeof(float2);
+      DPG_CUDA(cudaMemsetAsync(V.x, 0, bytes, st));
+      if (F.P.np > 0 && F.P.variant == SMOOTH_CLASS)
+        choose(F.P.blk, 1, F.P.ncls_items, F, [&]() { smooth_blk<float2>(F, V.x, V.t, 1.0, 0, V.pbuf, kb, st); });
+      if (F.A.cell.on)
+        choose(F.A.cell.blk, 2, F.A.cell.nitems, F,
+               [&]() { spmv_blk<float2>(F.A, F.A.v32, V.x, nullptr, V.t, 0, kb, st); });
+      if (F.mop.cond)
+        choose(F.mop.cond_blk, 3, F.mop.ncitems, F, [&]() { condense_blk<float2>(F, V.x, V.t, V.cbuf, kb, st); });
+      if (F.mop.back)
+        choose(F.mop.back_blk, 4, F.mop.nbitems, F, [&]() { backsub_blk<float2>(F, V.x, V.t, kb, st); });
+    }
+    if (!cg_c128(S) && A.cell.df_on) {
+      DPG_CUDA(cudaMemsetAsync(P, 0, (size_t)n * K * sizeof(double2), st));
+      choose(const_cast<ECSRDev&>(A).cell.df_blk, 5, A.cell.ndgitems, S.levels[L], [&]() { cg_apply_blk(P, nullptr, Q, 0); });
+    }
+  }
   // z = B r for every column (complex128 result in Z)
   auto precondition_blk = [&]() {
     if (mixed) {
