@@ -335,7 +335,23 @@ def traffic_for(kernel, bytes_per_launch):
     return ratio * bytes_per_launch if ratio else None
 
 
+FP32_PEAK_TFLOPS = 74.5   # measured FP32 FMA rate of one GB300 (8 independent FMA chains per thread)
 FP64_PEAK_TFLOPS = 1.20   # measured FP64 FMA rate of one GB300 (8 independent FMA chains per thread)
+
+
+def bf16_peak():
+    """Measured cuBLAS bf16 TFLOP/s (MEASURED_PEAKS.json; else an earlier measurement)."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["bf16_tflops"])
+    except (OSError, KeyError, ValueError):
+        return 1900.0
+
+
+def cell_entries(n, p):
+    """(entries of the element matrices, of those with real class matrices: no boundary face)."""
+    loc = (p + 1) ** 3 - (p - 1) ** 3 + 6 * p * p
+    return math.prod(n) * loc * loc, math.prod(max(k - 2, 0) for k in n) * loc * loc
 
 
 def element_line(acc, full_gflop):
@@ -394,6 +410,7 @@ def run_gb300(args, rank, world, local_rank):
     tuned = {}
     elem_acc = [0.0, 0.0, 0]   # element-stage ms, GFLOP, setups
     phases = []                # device ms of each setup phase, per step
+    forms = {}                 # products of the finest level that run with class matrices
     patch_store = {}           # finest level: sum n_j^2, and over the real packed patches
 
     def step(prof=D.PROF_OFF):
@@ -408,6 +425,9 @@ def run_gb300(args, rank, world, local_rank):
             li = D.dpgmg_level_info(h, s, w["opts"]["n_levels"] - 1)
             patch_store.update(sum_patch_sq=int(li.sum_patch_sq), real_sq=int(li.patch_real_sq),
                                op_nnz=int(li.op_nnz), op_real_nnz=int(li.op_real_nnz))
+            lf = w["opts"]["n_levels"] - 1
+            forms.update(smooth=D.dpgmg_class_form(h, s, lf, D.FORM_SMOOTH) == 1,
+                         spmv=tuned.get("level%d" % lf) == D.SPMV_CELLS, cg=tuned["cg"] == D.SPMV_CELLS)
             em, eg, _ = D.dpgmg_setup_profile(h, s)
             phases.append(D.dpgmg_setup_phases(h, s))
             elem_acc[0] += em
@@ -462,19 +482,33 @@ def run_gb300(args, rank, world, local_rank):
         dof_iters, pcg_ms, total_ms = reduce_ranks(dist, dof_iters, pcg_ms, total_ms, "cuda")
     value = dof_iters / (pcg_ms / 1e3)
 
-    # ---- the other HBM-bound kernels of the iteration, one profiled step each
+    # ---- the operator products of the iteration, one profiled step each
     kernels = []
-    for prof, name in ((D.PROF_SPMV_FINE, "k_spmv (finest V-cycle SpMV, c64 values)"),
-                       (D.PROF_SPMV_CG, "k_spmv_df (CG operator, c64 hi + lo values)")):
+    peak, peak_kind = peaks()
+    ent, ent_real = cell_entries(w["problem"]["n"], w["problem"]["p"])
+    for prof, key in ((D.PROF_SPMV_FINE, "spmv"), (D.PROF_SPMV_CG, "cg")):
         _, pr = step(prof)
         ms = pr[0] / max(pr[1], 1)
-        gbs = pr[2] / (ms / 1e3) / 1e9
-        kernels.append({"kernel": name, "bytes_per_launch": pr[2], "launches": pr[1], "avg_launch_ms": ms,
-                        "achieved": gbs, "unit": "GB/s",
-                        "bytes_rule": "stored values read once: complex64 8 B per entry (CG operator: high + "
-                                      "low parts, 16 B), real packed rows half of that",
-                        "real_packed_fraction_of_entries": (patch_store["op_real_nnz"] / patch_store["op_nnz"]
-                                                            if patch_store.get("op_nnz") else None)})
+        k = {"bytes_per_launch": pr[2], "launches": pr[1], "avg_launch_ms": ms}
+        if forms.get(key):   # by cells: class matrices out of L2, so the arithmetic is the yardstick
+            # per entry and complex vector: 2 real multiply-adds (4 for complex matrices); CG: 28 digit products each
+            flops = 4.0 * (2 * ent - ent_real) * (28 if key == "cg" else 1)
+            k.update({"kernel": "k_class_cell_dg + k_cell_sum_df (CG operator by cells, bf16 digits)" if key == "cg" else
+                                "k_class_cell + k_cell_sum (finest V-cycle operator by cells)",
+                      "bound": "bf16 tensor" if key == "cg" else "fp32", "flops_per_launch": flops,
+                      "achieved": flops / (ms / 1e3) / 1e12, "unit": "TFLOP/s",
+                      "peak": bf16_peak() if key == "cg" else FP32_PEAK_TFLOPS,
+                      "bytes_rule": "class matrices once; per cell DOF its index, gathered value, product written and "
+                                    "read, and slot"})
+        else:
+            k.update({"kernel": "k_spmv_df (CG operator, c64 hi + lo values)" if key == "cg" else
+                                "k_spmv (finest V-cycle SpMV, c64 values)",
+                      "bound": "hbm", "achieved": pr[2] / (ms / 1e3) / 1e9, "unit": "GB/s", "peak": peak,
+                      "bytes_rule": "stored values read once: complex64 8 B per entry (CG operator: high + "
+                                    "low parts, 16 B), real packed rows half of that",
+                      "real_packed_fraction_of_entries": (patch_store["op_real_nnz"] / patch_store["op_nnz"]
+                                                          if patch_store.get("op_nnz") else None)})
+        kernels.append(dict(k, frac=k["achieved"] / k["peak"]))
 
     # ---- end to end through the public API with host buffers
     e2e = None
@@ -535,9 +569,29 @@ def run_gb300(args, rank, world, local_rank):
 
     if rank != 0:
         return None
-    peak, peak_kind = peaks()
     per_launch_ms = prof_ms / max(prof_n, 1)
     achieved = prof_b / (per_launch_ms / 1e3) / 1e9
+    real_frac = patch_store["real_sq"] / patch_store["sum_patch_sq"] if patch_store.get("sum_patch_sq") else None
+    hbm = {"achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_source": peak_kind,
+           "bytes_per_launch": prof_b,
+           "bytes_rule": "distinct stored patch-inverse entries read once: 8 B per complex64 entry, 4 B per "
+                         "entry of a real packed block"}
+    if forms.get("smooth"):   # the block of a class stays in L2 for its patches: the FP32 pipe is the bound
+        flops = 4.0 * (2 * patch_store["sum_patch_sq"] - patch_store["real_sq"])
+        tf = flops / (per_launch_ms / 1e3) / 1e12
+        roofline = {"kernel": "k_class_apply (finest smoother product, one product per patch class)", "bound": "fp32",
+                    "achieved": tf, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": tf / FP32_PEAK_TFLOPS,
+                    "peak_source": "measured FP32 FMA rate", "flops_per_launch": flops,
+                    "flops_rule": "per patch entry and complex vector 2 real multiply-adds (4 for complex blocks)",
+                    "hbm": hbm}
+    else:
+        roofline = dict(hbm, kernel="k_patch_apply (finest smoother product)", bound="hbm",
+                        traffic=traffic_for("k_patch_apply", prof_b),
+                        traffic_source="not measured in this run: ncu dram__bytes_read.sum + dram__bytes_write.sum "
+                                       "per algorithmic byte of the finest launches of one step of the "
+                                       "32x32x16 layered workload (profiles/traffic.json) times this "
+                                       "launch's algorithmic bytes; null once the kernel source has changed")
+    roofline.update(launches=prof_n, avg_launch_ms=per_launch_ms, real_packed_fraction_of_entries=real_frac)
     it_last = stats[-1]
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -552,19 +606,7 @@ def run_gb300(args, rank, world, local_rank):
         "true_relres": it_last[3], "relres": it_last[4], "bytes_per_iter": it_last[5],
         "pcg_GBps": it_last[5] * it_last[0] / (stats[-1][1] / 1e3) / 1e9,
         "gpu_launches": int(launches),
-        "roofline": {"kernel": "finest smoother product (k_class_apply where patches share blocks, then bound by "
-                               "the FP32 pipe and not by these bytes; else k_patch_apply)", "bound": "hbm", "achieved": achieved,
-                     "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_source": peak_kind,
-                     "bytes_per_launch": prof_b, "launches": prof_n, "avg_launch_ms": per_launch_ms,
-                     "bytes_rule": "distinct stored patch-inverse entries read once: 8 B per complex64 entry, 4 B per "
-                                   "entry of a real packed block",
-                     "real_packed_fraction_of_entries": (patch_store["real_sq"] / patch_store["sum_patch_sq"]
-                                                         if patch_store.get("sum_patch_sq") else None),
-                     "traffic": traffic_for("k_patch_apply", prof_b),
-                     "traffic_source": "not measured in this run: ncu dram__bytes_read.sum + dram__bytes_write.sum "
-                                       "per algorithmic byte of the finest launches of one step of the "
-                                       "32x32x16 layered workload (profiles/traffic.json) times this "
-                                       "launch's algorithmic bytes; null once the kernel source has changed"},
+        "roofline": roofline,
         "clocks": clk, "e2e": e2e, "fp64_path": fp64,
         "rel_l2_error_vs_oracle": err_main,
         "rel_l2_distance_to_converged": conv_main,
@@ -575,7 +617,7 @@ def run_gb300(args, rank, world, local_rank):
                                         "128-row seeded sign sketch)" % {2: "c2_oracle.json", 3: "c3_oracle.json"}[
                                             args.config]} if gold else None),
         "precision_options": options,
-        "kernels": [dict(k, frac=k["achieved"] / peak) for k in kernels],
+        "kernels": kernels,
         "spmv_group_tuned": tuned,
         "setup_phases_ms": ({k: sum(p[i] for p in phases) / len(phases) for i, k in enumerate(D.SETUP_PHASES)}
                             if phases else None),
@@ -724,6 +766,8 @@ def c2_summary(args, D):
         s = D.dpgmg_setup(h, pb, op)
         if k >= 3:
             D.dpgmg_profile(h, s, D.PROF_SMOOTH_FINE)
+            lf = w["opts"]["n_levels"] - 1
+            li, by_class = D.dpgmg_level_info(h, s, lf), D.dpgmg_class_form(h, s, lf, D.FORM_SMOOTH)
         code, st = D.dpgmg_solve(h, s, tr.data_ptr(), fl.data_ptr(), out_is_device=False)
         pr = D.dpgmg_profile_read(h, s) if k >= 3 else None
         D.dpgmg_release(h, s)
@@ -739,7 +783,10 @@ def c2_summary(args, D):
             "pcg_ms": sum(r[1] for r in res) / len(res), "setup_ms": sum(r[2] for r in res) / len(res),
             "e2e": {"value": n_dof * sum(r[0] for r in res) / sum(r[3] for r in res), "unit": UNIT,
                     "ms_per_step": 1e3 * sum(r[3] for r in res) / len(res)},
-            "smoother_frac_of_hbm": res[-1][4][2] / (ms / 1e3) / 1e9 / peak,
+            "smoother_avg_launch_ms": ms,
+            ("smoother_frac_of_fp32" if by_class else "smoother_frac_of_hbm"):
+                (4.0 * (2 * li.sum_patch_sq - li.patch_real_sq) / (ms / 1e3) / 1e12 / FP32_PEAK_TFLOPS if by_class else
+                 res[-1][4][2] / (ms / 1e3) / 1e9 / peak),
             "rel_l2_error_vs_oracle": sketch_error(tr.numpy().view(np.complex128), gold) if gold else None}
 
 

@@ -215,7 +215,8 @@ typedef struct dpgmg_stats {
   double true_relres;      /* ||b - A x|| / ||b|| recomputed at exit (FP64) */
   double t_setup_ms;       /* device time of dpgmg_setup */
   double t_pcg_ms;         /* device time from the first CG step to convergence */
-  long long bytes_per_iter;/* algorithmic bytes of one CG iteration (distinct matrix entries read once) */
+  long long bytes_per_iter;/* algorithmic bytes of one CG iteration (distinct matrix entries read once:
+                              matrices shared by a class count once, whichever form of a product runs) */
   long long n_dof;         /* finest trace DOFs */
   long long dev_bytes_peak;/* peak device bytes held by the system */
 } dpgmg_stats;
@@ -478,8 +479,10 @@ int dpgmg_setup_phases(dpgmg_handle h, dpgmg_system sys, double* ms, int n);
 /* Bracket every launch of one kernel with CUDA events on the launching
  * stream during subsequent dpgmg_solve calls (which = DPGMG_PROF_*; OFF
  * clears).  dpgmg_profile_read() synchronises, returns the summed device
- * time, the launch count and the algorithmic bytes per launch (stored
- * matrix entries read once), and resets the accumulators. */
+ * time, the launch count and the algorithmic bytes per launch of the form in
+ * force (stored matrix entries read once; a product by cells its class
+ * matrices, and per cell DOF its index, gathered value, product written and
+ * read, and slot), and resets the accumulators. */
 int dpgmg_profile(dpgmg_handle h, dpgmg_system sys, int which);
 int dpgmg_profile_read(dpgmg_handle h, dpgmg_system sys, double* total_ms, long long* launches,
                        long long* bytes_per_launch);

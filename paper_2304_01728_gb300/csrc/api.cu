@@ -200,6 +200,8 @@ size_t estimate_bytes(const dpgmg_problem* pb, const dpgmg_opts* op) {
   return (size_t)((resident + transient + coarse_transient) * 1.05) + ((size_t)64 << 20);
 }
 
+// Distinct matrix entries of one CG iteration: matrices that a class shares count
+// once, whichever form of a product runs.
 static void fill_bytes_per_iter(SystemImpl& S) {
   const bool mixed = S.op.precision == DPGMG_PREC_MIXED;
   const double esz = mixed ? 8.0 : 16.0;
@@ -215,14 +217,17 @@ static void fill_bytes_per_iter(SystemImpl& S) {
   } else {
     cg_nnz = (int64_t)(F.mesh.nelem * (double)F.nloc * F.nloc * 0.8);
   }
-  b += (cg_nnz - cg_real) * 16.0 + cg_real * 8.0;
+  const CellOpDev& cgc = F.A.cell;
+  b += cgc.dig ? (double)cgc.dig_bytes() : (cg_nnz - cg_real) * 16.0 + cg_real * 8.0;
   const int nu = S.op.nu_pre + S.op.nu_post;
   for (size_t l = 1; l < S.levels.size(); ++l) {
     const Level& L = S.levels[l];
     b += nu * ((double)(L.P.uniq_sq - L.P.uniq_real_sq) + 0.5 * (double)L.P.uniq_real_sq) * esz;  // smoother (n_j^2 per
                                                                                       // stored block, real ones half)
-    b += std::max(1, nu) * ((double)(L.A.nnz_alg - L.A.nnz_real) + 0.5 * (double)L.A.nnz_real) * esz;  // SpMVs
-    if (L.kind == 2) b += (double)L.nK * (2.0 * L.nI * L.nS + L.nI * L.nI) * esz; // condense + backsub
+    b += std::max(1, nu) * (L.A.cell.W ? (double)L.A.cell.mat_bytes()   // operator products
+                                       : ((double)(L.A.nnz_alg - L.A.nnz_real) + 0.5 * (double)L.A.nnz_real) * esz);
+    if (L.kind == 2)   // condense + backsub
+      b += L.mop.Wb ? (double)L.mop.mat_bytes() : (double)L.nK * (2.0 * L.nI * L.nS + L.nI * L.nI) * esz;
   }
   const Level& C0 = S.levels[0];
   if (C0.has_coarse) b += (double)C0.N0 * (C0.N0 + 1) * esz;                     // L^-1 and L^-H (packed)
@@ -317,6 +322,17 @@ void setup_system(SystemImpl& S, const dpgmg_problem* pb, const dpgmg_opts* op, 
         P.real_sq += sq;
         if (own[j] == j) P.uniq_real_sq += sq;
       }
+  }
+  auto real_flags = [](const uint8_t* flags, int64_t n) {
+    std::vector<uint8_t> fl((size_t)std::max<int64_t>(n, 1));
+    DPG_CUDA(cudaMemcpy(fl.data(), flags, (size_t)n, cudaMemcpyDeviceToHost));
+    return (int64_t)std::count_if(fl.begin(), fl.begin() + n, [](uint8_t f) { return f != 0; });
+  };
+  for (size_t l = 1; l < S.levels.size(); ++l) {
+    CellOpDev& D = S.levels[l].A.cell;
+    MacroOpDev& M = S.levels[l].mop;
+    if (D.W) D.real_cls = real_flags(D.rflag, D.ncls);
+    if (M.Wb) M.real_cls = real_flags(M.rflag, M.ncls);
   }
   fill_bytes_per_iter(S);
 }

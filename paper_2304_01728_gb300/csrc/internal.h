@@ -123,6 +123,13 @@ struct CellOpDev {
   int64_t stride() const { return n * patch_ld(n); }   // entries per class matrix
   int64_t tiles() const { return (n + 15) / 16; }
   int64_t dgstride() const { return 2 * tiles() * tiles() * DG_S * 32; }
+  // bytes of the class matrices (complex64 or reals; digits), each once
+  int64_t real_cls = 0;        // classes stored as reals (host copy, after setup)
+  int64_t mat_bytes() const { return (ncls - real_cls) * stride() * 8 + real_cls * n * patch_ldr(n) * 4; }
+  int64_t dig_bytes() const { return (2 * ncls - real_cls) * (dgstride() / 2) * 16 + ncls * tiles() * 16 * 4; }
+  // bytes of one application: the class matrices, and per cell DOF its index, gathered value, product (written and
+  // read) and slot; `val`: bytes of a value
+  int64_t op_bytes(int64_t mat, int64_t val) const { return mat + ncell * n * (8 + 3 * val) + ndof * val; }
 };
 
 // first place of DOF g's row in CellOpDev::tab (also the table's size, for g = ndof)
@@ -149,6 +156,11 @@ struct MacroOpDev {
   int32_t* mem = nullptr;
   int64_t bstride() const { return (nI + nS) * patch_ld(nI); }
   int64_t cstride() const { return nI * patch_ld(nS); }
+  int64_t ncls = 0, real_cls = 0;
+  int64_t mat_bytes() const {   // both transfers' class matrices, each once
+    return (ncls - real_cls) * (bstride() + cstride()) * 8 +
+           real_cls * ((nI + nS) * patch_ldr(nI) + nI * patch_ldr(nS)) * 4;
+  }
 };
 
 struct ECSRDev {

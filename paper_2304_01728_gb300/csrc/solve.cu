@@ -1487,7 +1487,7 @@ void macro_op_setup(SystemImpl& S, Level& F, const LevelPlan& lp, cudaStream_t s
   D.nI = F.nI;
   D.nS = F.nS;
   D.offU = F.mesh.offU;
-  const int64_t ncls = (int64_t)lp.orep.size(), total = F.nK * (F.nI + F.nS);
+  const int64_t ncls = D.ncls = (int64_t)lp.orep.size(), total = F.nK * (F.nI + F.nS);
   D.idx = A.arr<int32_t>((size_t)total);
   D.cls = F.A.cell.cls;
   D.mem = F.A.cell.mem;
@@ -2496,10 +2496,12 @@ int pcg_solve(SystemImpl& S, cudaStream_t st, double2* xout, dpgmg_stats* stats,
     const int64_t esz = S.op.precision == DPGMG_PREC_MIXED ? 8 : 16;
     if (S.prof_which == DPGMG_PROF_SMOOTH_FINE)   // stored blocks read once: real packed ones at half size
       S.prof_bytes = (Ff.P.uniq_sq - Ff.P.uniq_real_sq) * esz + Ff.P.uniq_real_sq * (esz / 2);
-    else if (S.prof_which == DPGMG_PROF_SPMV_FINE)   // packed real entities at half size
-      S.prof_bytes = (Ff.A.nnz_alg - Ff.A.nnz_real) * esz + Ff.A.nnz_real * (esz / 2);
-    else if (S.prof_which == DPGMG_PROF_SPMV_CG)     // hi + lo complex64, or hi + lo reals
-      S.prof_bytes = (A.nnz_alg - A.nnz_real) * 16 + A.nnz_real * 8;
+    else if (S.prof_which == DPGMG_PROF_SPMV_FINE)   // the form in force: by cells, or packed real entities at half size
+      S.prof_bytes = Ff.A.cell.on ? Ff.A.cell.op_bytes(Ff.A.cell.mat_bytes(), 8)
+                                  : (Ff.A.nnz_alg - Ff.A.nnz_real) * esz + Ff.A.nnz_real * (esz / 2);
+    else if (S.prof_which == DPGMG_PROF_SPMV_CG)     // digits by cells, or hi + lo complex64, hi + lo reals
+      S.prof_bytes = A.cell.df_on ? A.cell.op_bytes(A.cell.dig_bytes(), 16)
+                                  : (A.nnz_alg - A.nnz_real) * 16 + A.nnz_real * 8;
   }
   const int64_t n = S.levels.back().mesh.ndof;
   cudaEvent_t e0, e1;

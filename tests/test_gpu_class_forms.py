@@ -204,3 +204,31 @@ def test_cg_operator_entry_by_entry(n, p, omega, box, digits):
                 assert np.max(err) <= 2.0 ** -43
                 q.append(np.sqrt(np.mean(err ** 2)))
             assert q[0] <= 1.25 * q[-1], q
+
+
+def test_bytes_of_the_form_that_ran():
+    """Bytes per launch follow the form in force; bytes per iteration count what
+    is distinct, whichever form runs."""
+    case = CASES[2]
+    n, p, nel = case[0], case[1], 16 * 16 * 8
+    loc = (p + 1) ** 3 - (p - 1) ** 3 + 6 * p * p
+    tiles = (loc + 15) // 16
+    ldr, ld = (loc + 3) // 4 * 4, (loc + 1) // 2 * 2
+    with solver(case) as s:
+        L, g = case[3] - 1, s.level(case[3] - 1)
+        # 27 classes by boundary faces, the interior one real; digits: 7 of 2 bytes per entry and part
+        mat = 26 * loc * ld * 8 + loc * ldr * 4
+        dig = (2 * 27 - 1) * (16 * tiles) ** 2 * 14 + 27 * tiles * 16 * 4
+        want = {(D.PROF_SPMV_FINE, 1): mat + nel * loc * (8 + 3 * 8) + g.n_dof * 8,
+                (D.PROF_SPMV_CG, 1): dig + nel * loc * (8 + 3 * 16) + g.n_dof * 16,
+                (D.PROF_SPMV_FINE, 0): (g.op_nnz - g.op_real_nnz) * 8 + g.op_real_nnz * 4,
+                (D.PROF_SPMV_CG, 0): (g.op_nnz - g.op_real_nnz) * 16 + g.op_real_nnz * 8}
+        per_iter = set()
+        for on in (1, 0):
+            select(s, L, on)
+            for which in (D.PROF_SPMV_FINE, D.PROF_SPMV_CG):
+                D.dpgmg_profile(s.h, s.s, which)
+                per_iter.add(s.solve(fields=False)[2].bytes_per_iter)
+                ms, launches, b = D.dpgmg_profile_read(s.h, s.s)
+                assert launches > 0 and ms > 0 and b == want[which, on], (which, on, b, want[which, on])
+        assert len(per_iter) == 1 and per_iter.pop() > 2 * mat + dig
