@@ -105,13 +105,12 @@ __device__ __forceinline__ void mma_bf16(float c[4], const uint4& a, uint32_t b0
                : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
 
-// the value of h in units of 2^(emax - 181): below 2^55 when emax is the column's
-// exponent (denormal parts count as zero)
+// the value of h in units of 2^(emax - 181): below 2^55 when emax is the column's exponent
 __device__ __forceinline__ long long digit_fixed(float h, int emax) {
   const uint32_t u = __float_as_uint(h);
-  const int e = (u >> 23) & 255, sh = e - emax + 31;
-  const long long m = (u & 0x7fffff) | 0x800000;
-  if (e == 0 || sh < -25) return 0;
+  const int e = max((int)(u >> 23) & 255, 1), sh = e - emax + 31;   // denormal parts: exponent 1, no leading bit
+  const long long m = (u & 0x7fffff) | ((u & 0x7f800000u) ? 0x800000 : 0);
+  if (sh < -25) return 0;
   const long long f = sh >= 0 ? m << min(sh, 31) : (m + (1ll << (-sh - 1))) >> -sh;
   return (int)u < 0 ? -f : f;
 }
@@ -174,12 +173,12 @@ static __global__ void __launch_bounds__(DG_THREADS, 2) k_class_cell_dg(
       top = __reduce_max_sync(0xffffffffu, top);
       // the column is 2^(emax - 181) times its integers; a largest value above 1 - 2^-7 of the power of two takes
       // the next one, so that the leading digit with its carry stays below 128
-      const int emax = (int)((top + 0x20000u) >> 23);
+      const int emax = max((int)((top + 0x20000u) >> 23), 1);
       // 2^(emax - 128); infinities and NaN give NaN
       if (lane == 0)
         cscale[m] = top >= 0x7f800000u ? __uint_as_float(0x7fffffffu)
                                        : (emax > 1 ? __uint_as_float((uint32_t)(emax - 1) << 23)
-                                                   : (emax == 1 ? __uint_as_float(0x00400000u) : 0.f));
+                                                   : __uint_as_float(0x00400000u));
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const int k = 64 * i + 2 * lane;

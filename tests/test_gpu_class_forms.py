@@ -232,3 +232,18 @@ def test_bytes_of_the_form_that_ran():
                 ms, launches, b = D.dpgmg_profile_read(s.h, s.s)
                 assert launches > 0 and ms > 0 and b == want[which, on], (which, on, b, want[which, on])
         assert len(per_iter) == 1 and per_iter.pop() > 2 * mat + dig
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e-32, 1e-34, 1e-36])
+def test_digits_of_small_values(scale):
+    """Values whose low FP32 parts are denormal keep what those parts hold: 2^-149
+    of resolution in the operands and in the parts of the cells' products, up to 8
+    cells of 54 terms, beside the double-float form's 1e-12."""
+    with solver(CASES[1]) as s:
+        L = CASES[1][3] - 1
+        n = s.level(L).n_dof
+        x = rand_vec(n, 3)
+        assert D.dpgmg_spmv_group(s.h, s.s, -1, D.SPMV_CELLS) == D.SPMV_CELLS
+        want = scale * D.dpgmg_apply(s.h, s.s, D.OP_AFULL, L, x, n)
+        err = rel(D.dpgmg_apply(s.h, s.s, D.OP_AFULL, L, scale * x, n), want)
+        assert err < 1e-12 + 8 * 54 * 2.0 ** -149 / scale, err
