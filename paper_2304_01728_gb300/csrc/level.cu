@@ -1011,7 +1011,10 @@ static void setup_patches(SystemImpl& S, Level& F, const LevelPlan& lp, int* din
   k_patch_gather<double2><<<nown, 256, 0, st>>>(F.A, D.ptr, D.dofs, D.val_ptr, D.inv64, 0, order);
   DPG_CHECK_LAUNCH();
   // FP64 inverses (FP64 path, or the mixed path under DPGMG_FLAG_PATCH_FP64,
-  // which rounds them to complex64 after theta is estimated)
+  // which rounds them to complex64 after theta is estimated).  Patches of a class
+  // share the stored block here too; the smoother streams it (no class product:
+  // the FP64 path's would run on the FP64 pipe, the option's blocks are all
+  // complex64, and neither form was built or measured).
   invert_patches<double2>(A, D, lp, order, D.inv64, F.mesh.offU, dinfo, st);
   A.release(order);
 }
@@ -1029,17 +1032,16 @@ static bool share_patches(const SystemImpl& S) { return !(S.op.flags & DPGMG_FLA
 // The class product is planned when the blocks are shared by at least
 // CLS_MIN_SHARE patches on average (by entries); below that it reads as many
 // bytes as the streaming product, which keeps more of them in flight.  Above,
-// setup times both: many patches gain (18,513 patches, 451 -> 92 us), a level
+// setup times both: many patches gain (18,513 patches, 451 -> 99 us), a level
 // with few items loses (405 macro patches of up to 488 DOFs: 24 us streamed).
 constexpr double CLS_MIN_SHARE = 2.0;
 
 // Work items of a class product: mem lists the members class by class, items
 // are (first member, members, first output, CLS_* shape), the longest first
 // (sum length times tile size), so that short ones end the launch.
-// most: members per item at most.
 template <class F>
 static void class_items(const std::vector<std::vector<int32_t>>& members, F&& size_of, std::vector<int32_t>& mem,
-                        std::vector<int4>& items, int most = 32) {
+                        std::vector<int4>& items) {
   for (const auto& m : members) {
     const int64_t n = size_of(m[0]), m0 = (int64_t)mem.size();
     const int cnt = (int)m.size();
@@ -1047,7 +1049,7 @@ static void class_items(const std::vector<std::vector<int32_t>>& members, F&& si
     for (int64_t a = 0; a < n; a += 64) {
       const bool half = n - a <= 32;
       for (int q = 0; q < cnt;) {
-        const int left = std::min(cnt - q, most);
+        const int left = std::min(cnt - q, 32);
         const int shape = half ? (left > 16 ? CLS_32x32 : CLS_32x16)
                                : (left > 16 ? CLS_64x32 : (left > 8 ? CLS_64x16 : CLS_64x8));
         const int w = shape == CLS_64x8 ? 8 : (shape == CLS_64x16 || shape == CLS_32x16 ? 16 : 32);
