@@ -1123,7 +1123,7 @@ static void plan_cell_classes(LevelPlan& lp, const std::vector<int32_t>& cells, 
   if (nI == 0) {   // CG operator by cells (the finest level's, which is a p level)
     const int T = (n + 15) / 16;
     // warps' shares (16 rows x 8 cells) per CTA: up to 28 (p = 3: every row of
-    // the cells, 158 us; 16 shares 165 us, which convert the cells' values
+    // the cells, 154 us; 16 shares 7 us more, which convert the cells' values
     // twice), 8 where that leaves SMs without work
     for (int share : {28, 8}) {
       lp.dgitems.clear();
