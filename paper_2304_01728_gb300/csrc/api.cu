@@ -27,13 +27,13 @@ long long thread_launch_count() { return t_launches; }
 
 static std::atomic<int> g_running{0};
 static std::atomic<long long> g_started{0};
-GpuWork::GpuWork() {
+GpuJob::GpuJob() {
   ++g_running;
   ++g_started;
 }
-GpuWork::~GpuWork() { --g_running; }
-int gpu_work_running() { return g_running.load(); }
-long long gpu_work_started() { return g_started.load(); }
+GpuJob::~GpuJob() { --g_running; }
+int gpu_jobs_running() { return g_running.load(); }
+long long gpu_jobs_started() { return g_started.load(); }
 
 void* Alloc::get(size_t bytes) {
   bytes = (bytes + 255) & ~(size_t)255;
@@ -235,7 +235,7 @@ static void fill_bytes_per_iter(SystemImpl& S) {
 }
 
 void setup_system(SystemImpl& S, const dpgmg_problem* pb, const dpgmg_opts* op, size_t budget, cudaStream_t st) {
-  GpuWork work;
+  GpuJob job;
   S.pb = *pb;
   S.op = *op;
   const int64_t ne = (int64_t)pb->n[0] * pb->n[1] * pb->n[2];

@@ -29,14 +29,14 @@ void set_last_error(const std::string& m);
 // Setups and solves of this process in flight, and how many have ever begun: a
 // timing on the GPU is undisturbed when its setup is the only one and none begins
 // meanwhile.
-struct GpuWork {
-  GpuWork();
-  ~GpuWork();
-  GpuWork(const GpuWork&) = delete;
-  GpuWork& operator=(const GpuWork&) = delete;
+struct GpuJob {
+  GpuJob();
+  ~GpuJob();
+  GpuJob(const GpuJob&) = delete;
+  GpuJob& operator=(const GpuJob&) = delete;
 };
-int gpu_work_running();
-long long gpu_work_started();
+int gpu_jobs_running();
+long long gpu_jobs_started();
 
 void count_launch();
 void count_launches(long long n);

@@ -2296,8 +2296,8 @@ static int pick_variant(const TuneKey& key, const Evict& ev, cudaStream_t st, st
     }
   } ev2(2 * TUNE_REPS * forms.size());
   auto at = [&](size_t v, int r, int end) { return ev2.e[2 * (v * TUNE_REPS + r) + end]; };
-  const long long work = gpu_work_started();
-  const bool crowded = gpu_work_running() > 1;
+  const long long begun = gpu_jobs_started();
+  const bool crowded = gpu_jobs_running() > 1;
   for (int G : forms) run(G);
   for (int r = 0; r < TUNE_REPS; ++r)
     for (size_t v = 0; v < forms.size(); ++v) {
@@ -2312,7 +2312,7 @@ static int pick_variant(const TuneKey& key, const Evict& ev, cudaStream_t st, st
     for (int r = 0; r < TUNE_REPS; ++r) DPG_CUDA(cudaEventElapsedTime(&ms[v][r], at(v, r, 0), at(v, r, 1)));
   std::lock_guard<std::mutex> lk(g_tune_mu);
   TuneRecord& rec = g_tune[key];
-  rec.add(ms, !crowded && gpu_work_started() == work);
+  rec.add(ms, !crowded && gpu_jobs_started() == begun);
   return forms[rec.best()];
 }
 
@@ -2487,7 +2487,7 @@ void prepare_solve(SystemImpl& S, cudaStream_t st) {
 }
 
 int pcg_solve(SystemImpl& S, cudaStream_t st, double2* xout, dpgmg_stats* stats, const double2* x0) {
-  GpuWork work;
+  GpuJob job;
   ensure_workspace(S, st);
   WS& W = *reinterpret_cast<WS*>(S.ws);
   const ECSRDev& A = cg_operator(S, W, st);
@@ -2632,7 +2632,7 @@ int pcg_solve(SystemImpl& S, cudaStream_t st, double2* xout, dpgmg_stats* stats,
 // graph captured for the current set of active columns (captured again when
 // a column converges).
 int pcg_solve_block(SystemImpl& S, cudaStream_t st, int K, const double2* B, double2* X, dpgmg_stats* stats) {
-  GpuWork work;
+  GpuJob job;
   ensure_workspace(S, st);
   WS& W = *reinterpret_cast<WS*>(S.ws);
   const ECSRDev& A = cg_operator(S, W, st);
